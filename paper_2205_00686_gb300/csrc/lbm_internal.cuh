@@ -90,12 +90,16 @@ template <class R>
 struct Phys {
     // EOS: p = rho Rg T/(1 - b rho) - a h^2 rho^2/(1 + 2 b rho - b^2 rho^2),
     // h = 1 + kpr (1 - sqrt(T/Tc))
-    R a, b, Rg, kpr, inv_Tc, akTc;   // akTc = a kpr / Tc
-    R two_over_G, negG;
+    R a, b, Rg, kpr, inv_Tc;
+    R one_p_kpr;
+    R two_over_G, negG, negG_12;
     // D2Q9 MRT rates and Li forcing
     R s_e, s_eps, s_q, s_p;
     R hs_e, hs_eps, hs_q, hs_p;      // 1 - s/2
     R sig_e, sig_eps;                // sigma / (1/s - 1/2)
+    // unit rates: the collision's combined factors (collide9_unit)
+    R u_m, u_d, u_g7, u_g8;          // (1 - s_p)/4, s_p/4, hs_p/2, hs_p/4
+    R u_ax, u_dg, u_0;               // the sigma terms' factors of |12 s|^2
     // D2Q5
     R cv, inv_cv, w_dot, w5_0, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
     R one_m_vs1, one_m_vs4;
@@ -121,9 +125,10 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.Rg = (R)d.Rg;
     p.kpr = (R)kpr;
     p.inv_Tc = (R)(1.0 / Tc);
-    p.akTc = (R)(d.a * kpr / Tc);
+    p.one_p_kpr = (R)(1.0 + kpr);
     p.two_over_G = (R)(2.0 / d.G);
     p.negG = (R)(-d.G);
+    p.negG_12 = (R)(-d.G / 12.0);
     p.s_e = (R)d.s_e;
     p.s_eps = (R)d.s_eps;
     p.s_q = (R)d.s_q;
@@ -134,6 +139,19 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.hs_p = (R)(1.0 - 0.5 * d.s_p);
     p.sig_e = (R)(d.sigma / (1.0 / d.s_e - 0.5));
     p.sig_eps = (R)(d.sigma / (1.0 / d.s_eps - 0.5));
+    p.u_m = (R)(0.25 * (1.0 - d.s_p));
+    p.u_d = (R)(0.25 * d.s_p);
+    p.u_g7 = (R)(0.5 * (1.0 - 0.5 * d.s_p));
+    p.u_g8 = (R)(0.25 * (1.0 - 0.5 * d.s_p));
+    {
+        // |F_m|^2 / psi^2 = G^2 |12 s|^2 / 144; e and epsilon get +-half of
+        // sigma / (1/s - 1/2) times it (s_e = s_eps = 1)
+        const double k = d.G * d.G / 144.0, se = 0.5 * d.sigma / (1.0 / d.s_e - 0.5),
+                     sp = 0.5 * d.sigma / (1.0 / d.s_eps - 0.5);
+        p.u_ax = (R)(k * (2.0 * sp - se) / 36.0);
+        p.u_dg = (R)(k * (2.0 * se - sp) / 36.0);
+        p.u_0 = (R)(-k * (se + sp) / 9.0);
+    }
     p.cv = (R)d.cv;
     p.inv_cv = (R)(1.0 / d.cv);
     p.w_dot = (R)d.w_dot;
@@ -174,28 +192,43 @@ __device__ __forceinline__ float f_rcp(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// FP64 reciprocal by the Newton-Raphson iteration for 1/x,
-// r <- r + r (1 - x r), which squares the relative error at each step: from
-// the hardware approximation rcp.approx.ftz.f64 two steps reach the FP64
-// rounding level (within about one ulp of 1/x, not always the correctly
-// rounded value).  The FP64 step divides six times per node and is bound by
-// the GB300's FP64 pipe.  Operands are O(1) here (rho, 1 - b rho, rho c_v,
-// sqrt(T/Tc)); a zero, infinite or NaN operand gives a non-finite result,
-// which the step reports.
+// FP64 reciprocal and square root.  The GB300 executes two FP64 lanes per SM
+// and clock, so an FP64 step is bound by the number of FP64 instructions.
+// Both start from the hardware approximation of the seed, with e = 1 - x r
+// (or 1 - x y^2) of about 2^-20, and take the first two terms of the series
+// 1/(1-e) = 1 + e + e^2 + ... (or (1-e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ...): what
+// is left out is of order e^3 ~ 2^-60, below the FP64 rounding, so the result
+// is within about one ulp (not always the correctly rounded value).  Three
+// and five FP64 instructions, against four for two Newton-Raphson steps and
+// about ten for the IEEE square root.  With eos_node, collide9_unit and the
+// rho c_v forms of the step's thermal stages, which count FP64 operations the
+// same way (about 168 per node instead of 220), the FP64 step on 1999 x 1501
+// went from 1.355 to 1.067 ms; in FP32 the same forms took the 4096^2 step
+// from 340.3 to 336.1 us.  A zero, infinite or NaN reciprocal
+// operand gives a non-finite result, which the step reports; a square-root
+// operand outside the normal range (zero, negative, NaN among them) takes
+// the IEEE square root.
 __device__ __forceinline__ double f_rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ float f_sqrt(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double f_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ double f_sqrt(double x) {
+    // high words of 2^-1000 .. 2^1000, compared as integers (an FP64 compare
+    // would take a slot of the FP64 pipe)
+    if ((unsigned)(__double2hiint(x) - 0x01700000) > 0x7d000000u) return sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y;
+    const double e = fma(-t, y, 1.0);
+    return fma(t * e, fma(0.375, e, 0.5), t);
+}
 
 // Two-lane arithmetic.  In float it maps to Blackwell's paired FP32
 // instructions (one FADD2 / FMUL2 / FFMA2 does the work of two), each lane
@@ -211,6 +244,13 @@ __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c) {
     return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
 }
+// c - a b
+__device__ __forceinline__ float2 pnfma(float2 a, float2 b, float2 c) {
+    return __ffma2_rn(a, make_float2(-b.x, -b.y), c);
+}
+__device__ __forceinline__ double2 pnfma(double2 a, double2 b, double2 c) {
+    return make_double2(fma(-a.x, b.x, c.x), fma(-a.y, b.y, c.y));
+}
 __device__ __forceinline__ float2 psub(float2 a, float2 b) {
     return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
 }
@@ -225,34 +265,72 @@ __device__ __forceinline__ R eos_p(const Phys<R>& P, R rho, R T) {
     return rho * P.Rg * T / (R(1) - br) - P.a * h * h * rho * rho / (R(1) + R(2) * br - br * br);
 }
 
-// (dp_EOS/dT)_rho = rho Rg/(1 - b rho) + a k h rho^2 / (sqrt(T/Tc) Tc (1 + 2 b rho - b^2 rho^2))
-template <class R>
-__device__ __forceinline__ R eos_dpdT(const Phys<R>& P, R rho, R T) {
-    R st = rsq(T * P.inv_Tc);
-    R h = R(1) + P.kpr * (R(1) - st);
-    R br = P.b * rho;
-    return rho * P.Rg / (R(1) - br) + P.akTc * h * rho * rho / (st * (R(1) + R(2) * br - br * br));
-}
-
 template <class R>
 __device__ __forceinline__ R psi2_of(const Phys<R>& P, R rho, R T) {
     return P.two_over_G * (eos_p(P, rho, T) - rho * R(1.0 / 3.0));
 }
 
-// psi^2 and T (dp/dT)_rho of one node from shared sub-expressions:
-// st = sqrt(T/Tc), h = 1 + k (1 - st), ib = 1/(1 - b rho),
-// r2id = rho^2 / (1 + 2 b rho - b^2 rho^2)
+// psi^2 and T (dp/dT)_rho of one node, with D1 = 1 - b rho and
+// D2 = 1 + 2 b rho - b^2 rho^2 = 2 - D1^2 over one common reciprocal:
+//   p = rho (Rg T D2 - a h^2 rho D1) / (D1 D2)
+//   T (dp/dT)_rho = rho (Rg T D2 + a k h sqrt(T/Tc) rho D1) / (D1 D2)
+// (T / sqrt(T/Tc) = Tc sqrt(T/Tc), so no second reciprocal).  One square
+// root and one reciprocal, 22 other operations.
 template <class R>
 __device__ __forceinline__ void eos_node(const Phys<R>& P, R rho, R T, R* psi2, R* TdpdT) {
     const R st = f_sqrt(T * P.inv_Tc);
-    const R h = R(1) + P.kpr * (R(1) - st);
-    const R br = P.b * rho;
-    const R ib = f_rcp(R(1) - br);
-    const R r2id = rho * rho * f_rcp(R(1) + br * (R(2) - br));
-    const R rRib = rho * P.Rg * ib;
-    const R p = rRib * T - P.a * h * h * r2id;
+    const R h = P.one_p_kpr - P.kpr * st;
+    const R ah = P.a * h;
+    const R d1 = R(1) - P.b * rho;
+    const R d2 = R(2) - d1 * d1;
+    const R s = rho * f_rcp(d1 * d2);
+    const R u = P.Rg * T * d2, w = rho * d1;
+    const R p = s * (u - ah * h * w);
     *psi2 = P.two_over_G * (p - rho * R(1.0 / 3.0));
-    *TdpdT = T * (rRib + P.akTc * h * r2id * f_rcp(st));
+    *TdpdT = s * (u + P.kpr * ah * st * w);
+}
+
+// D2Q9 collision at unit rates (s_e = s_eps = s_q = 1: those moments leave the
+// collision at m^eq + F/2), so f* = M^{-1} m* needs of f only rho, j and the
+// stress moments m_7, m_8 (Eqs. 5, 7, 8).  With K = rho u.u + u.F and
+// |12 s|^2 of the force stencil,
+//   f*_0          = 4/9 rho - 2/3 K + u_0 |12 s|^2
+//   axis part     = 1/9 rho + 1/12 K + u_ax |12 s|^2, +- m*_7/4, +- (j + F)/3
+//   diagonal part = 1/36 rho + 1/12 K + u_dg |12 s|^2, +- m*_8/4,
+//                   +- ((j + F)_x +- (j + F)_y)/12
+// rhod: deviation of rho from the storage reference (f is stored as
+// deviations); rho: the density itself.
+template <class R, class R2>
+__device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rho, R rhod, R2 j, R m7, R m8,
+                                              R2 u, R2 F, R2 s12, R* f, int stride) {
+    const R2 ru = pmul(pr(rho, rho), u);
+    const R2 uu = pmul(ru, u);      // rho (ux^2, uy^2)
+    const R2 uF = pmul(u, F);       // (ux Fx, uy Fy)
+    const R2 K2 = padd(uu, uF);
+    const R K = K2.x + K2.y;
+    const R S = s12.x * s12.x + s12.y * s12.y;
+    const R b7 = P.u_m * m7 + (P.u_d * (uu.x - uu.y) + P.u_g7 * (uF.x - uF.y));
+    const R b8 = P.u_m * m8 + (P.u_d * (ru.x * u.y) + P.u_g8 * (u.x * F.y + u.y * F.x));
+    const R2 cc = pfma(pr(rhod, rhod), pr(R(1.0 / 9.0), R(1.0 / 36.0)),
+                       pfma(pr(S, S), pr(P.u_ax, P.u_dg), pr(K * R(1.0 / 12.0), K * R(1.0 / 12.0))));
+    const R2 js = padd(j, F);
+    // axis directions: (1, 2) = (ax + b7, ax - b7) + js/3, (3, 4) the same
+    // minus js/3; diagonals: (5, 8) = (dg + b8, dg - b8) + (jx + jy, jx - jy)/12,
+    // (7, 6) the same minus that
+    const R2 cb = pr(cc.x + b7, cc.x - b7), db = pr(cc.y + b8, cc.y - b8);
+    const R2 sd = pr(js.x + js.y, js.x - js.y);
+    const R2 t3 = pr(R(1.0 / 3.0), R(1.0 / 3.0)), t12 = pr(R(1.0 / 12.0), R(1.0 / 12.0));
+    const R2 f12 = pfma(js, t3, cb), f58 = pfma(sd, t12, db);
+    const R2 f34 = pnfma(js, t3, cb), f76 = pnfma(sd, t12, db);
+    f[0] = rhod * R(4.0 / 9.0) + (P.u_0 * S - K * R(2.0 / 3.0));
+    f[1 * stride] = f12.x;
+    f[2 * stride] = f12.y;
+    f[3 * stride] = f34.x;
+    f[4 * stride] = f34.y;
+    f[5 * stride] = f58.x;
+    f[6 * stride] = f76.y;
+    f[7 * stride] = f76.x;
+    f[8 * stride] = f58.y;
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {

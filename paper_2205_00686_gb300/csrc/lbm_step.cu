@@ -66,9 +66,12 @@ struct StepSmem {
     typename Vec2<R>::T u[3][NT];
     R fs[3][9][NT];     // post-collision f (deviation form)
     R gs[3][3][NT];     // post-collision g_1, g_2, g_3 (deviation form)
-    // per column and row: g_dev[0..4], rho, then P^{n-1} and T (dp/dT)_rho,
+    // per column and row: g_dev[0..4], rho c_v, then P^{n-1} and E (stage A),
     // which stage C replaces by the row's post-collision g*_0 and g*_4
     typename Vec4<R>::T own[5][2][NT];
+    // FP64: 1 / (rho c_v) and the deviation of T, from stage A to stage C (in
+    // FP32 forming them again is cheaper than the shared-memory traffic)
+    typename Vec2<R>::T own2[5][sizeof(R) == 8 ? NT : 1];
     int unit;
 };
 
@@ -112,7 +115,7 @@ struct StageSmem {
     typename Vec2<R>::T u[3][NT];
     R fs[3][9][NT];
     R gs[3][3][NT];
-    typename Vec2<R>::T own[5][NT];   // rho and T (dp/dT)_rho, from stage A to stage C
+    typename Vec2<R>::T own[5][NT];   // rho c_v and E, from stage A to stage C
     unsigned long long mbar[D + 1];
     unsigned long long probe;   // never armed: the wait-timeout test hook waits on it
     int unit;
@@ -251,10 +254,10 @@ struct Sweep {
     bool stalled;   // a staged-row wait ran out in this unit
     // staged form: what stage D5 of a row uses from its own column stays in
     // registers from stage C of that row (one iteration earlier) instead of
-    // shared memory: the row's g, rho, g*_0, g*_2 and g*_4 (c: written by
+    // shared memory: the row's g, rho c_v, g*_0, g*_2 and g*_4 (c: written by
     // C(k-3); d: read by D5(k-4)), and g*_2 of the row below (e)
-    R cg[5], crho, cgs0, cgs2, cgs4;
-    R dg[5], drho, dgs0, dgs2, dgs4, egs2;
+    R cg[5], cC, cgs0, cgs2, cgs4;
+    R dg[5], dC, dgs0, dgs2, dgs4, egs2;
 
     __device__ __forceinline__ Sweep(const Inst& I_, const Unit& U, const Phys<R>& P_, SM& S_,
                                      WallRings<R, NT>& WR_, unsigned mph0)
@@ -346,7 +349,7 @@ struct Sweep {
         errbits = 0;
 #pragma unroll
         for (int q = 0; q < 5; ++q) cg[q] = dg[q] = R(0);
-        crho = drho = R(1);
+        cC = dC = R(1);
         cgs0 = cgs2 = cgs4 = dgs0 = dgs2 = dgs4 = egs2 = R(0);
         // rotating ring slots: a0 = slot of row k, a1 = row k-1, a2 = row k-2
         // (ring of 3, so row k-3 is a0 again); b0 = slot of row k in the ring of 5
@@ -512,7 +515,7 @@ struct Sweep {
         {
             const int r = k - 3;
             if (STEADY || (r >= y0 - 1 && r < y1 + 1 && rowvalid(r) && inC)) {
-                R g0, g1, g2, g3, g4, rho, Pp, TdpdT;
+                R g0, g1, g2, g3, g4, C, Pp, E;
                 if constexpr (STG) {
                     const TG* gr = &S.gR[gC][0][sidx + goff];
                     g0 = st_val(gr[0]);
@@ -522,25 +525,26 @@ struct Sweep {
                     g4 = st_val(gr[4 * NTG]);
                     Pp = S.pR[gC][sidx];
                     const R2 ow = S.own[bC][t];
-                    rho = ow.x;
-                    TdpdT = ow.y;
+                    C = ow.x;
+                    E = ow.y;
                 } else {
                     const R4 o0 = S.own[bC][0][t];
                     const R4 o1 = S.own[bC][1][t];
                     g0 = o0.x; g1 = o0.y; g2 = o0.z; g3 = o0.w; g4 = o1.x;
-                    rho = o1.y; Pp = o1.z; TdpdT = o1.w;
+                    C = o1.y; Pp = o1.z; E = o1.w;
                 }
-                // (m_1, m_2) = (g1 - g3, g2 - g4) and the pair sums (g1 + g3, g2 + g4)
+                // (m_1, m_2) = (g1 - g3, g2 - g4)
                 const R2 m12 = psub(pr(g1, g2), pr(g3, g4));
-                const R2 p13 = padd(pr(g1, g2), pr(g3, g4));
                 const R m1 = m12.x, m2 = m12.y;
-                const R Td = (g0 + p13.x) + p13.y;
-                const R m3d = p13.x + p13.y;
-                const R m4 = p13.x - p13.y;
-                // Eqs. 49-50: c_s^2 d_x T = -varsigma_1 m_1^(1), m_1^eq = 0
-                const R2 dT = pmul(pr(-P.vs1_cs2h, -P.vs1_cs2h), m12);
-                const R dTx = dT.x;
-                const R dTy = dT.y;
+                R Td, iC = R(0);
+                if constexpr (sizeof(R) == 8) {
+                    const R2 o2 = S.own2[bC][t];
+                    iC = o2.x;
+                    Td = o2.y;
+                } else {
+                    const R2 p13 = padd(pr(g1, g2), pr(g3, g4));
+                    Td = (g0 + p13.x) + p13.y;
+                }
                 // neighbour rows: solid -> u = 0, open -> the boundary row
                 const bool vd = STEADY || pery || r - 1 >= 0, vu = STEADY || pery || r + 1 < ny;
                 const R2 uc = S.u[a0][t];
@@ -558,17 +562,17 @@ struct Sweep {
                 } else {
                     uN0.x = uN0.y = uN1.x = uN1.y = uN2.x = uN2.y = R(0);
                 }
-                // isotropic central difference, (1/c_s^2) sum_i w_i c_i phi(x + c_i)
-                const R divu = (uE.x - uW.x + uN1.y - uS1.y) * R(1.0 / 3.0) +
-                               ((uN2.x + uS2.x - uN0.x - uS0.x) +
-                                (uN2.y + uN0.y - uS2.y - uS0.y)) * R(1.0 / 12.0);
-                const R C = rho * P.cv;
-                // Q = -[rho c_v u.grad T + T (dp/dT)_rho div u]  (Eq. 20)
-                const R Q = -(C * (uc.x * dTx + uc.y * dTy) + TdpdT * divu);
-                // P^n = Q / (rho c_v); S = w^ rho c_v (dt/2) d_t^2 T with
-                // d_t^2 T ~ P^n - P^{n-1} (Eq. 24), i.e. (Q - rho c_v P^{n-1}) / 2
-                const R Pn = Q * f_rcp(rho) * P.inv_cv;
-                const R Qs = first ? Q : Q + R(0.5) * (Q - C * Pp);
+                // isotropic central difference, 12 (1/c_s^2) sum_i w_i c_i phi(x + c_i)
+                const R div12 = (uE.x - uW.x + uN1.y - uS1.y) * R(4) +
+                                ((uN2.x + uS2.x - uN0.x - uS0.x) +
+                                 (uN2.y + uN0.y - uS2.y - uS0.y));
+                // P^n = Q / (rho c_v) = -[u.grad T + T (dp/dT)_rho div u / (rho c_v)]
+                // (Eq. 20) with c_s^2 grad T = -varsigma_1 (m_1, m_2) (Eqs. 49-50,
+                // m^eq = 0) and E = T (dp/dT)_rho / (12 rho c_v)
+                const R Pn = P.vs1_cs2h * (uc.x * m1 + uc.y * m2) - E * div12;
+                // S = w^ rho c_v (dt/2) d_t^2 T with d_t^2 T ~ P^n - P^{n-1}
+                // (Eq. 24): Q + S = rho c_v (P^n + (P^n - P^{n-1}) / 2)
+                const R dP = first ? Pn : Pn + R(0.5) * (Pn - Pp);
                 // moment-space collision (Eqs. 39, 40, 47), deviation form
                 const R hc = R(0.5) * P.one_m_vs1;
                 const R2 h12 = pmul(pr(hc, hc), m12);
@@ -576,7 +580,7 @@ struct Sweep {
                 R gs0, gs1, gs2, gs3, gs4;
                 if (UNIT) {
                     // varsigma_3 = varsigma_4 = 1: m3* = w_dot (T + Qs), m4* = 0
-                    const R TQ = Td + Qs;
+                    const R TQ = Td + C * dP;
                     const R a = R(0.25) * P.w_dot * TQ;
                     // unfused: stage D5 subtracts g_0 from g*_0, and the
                     // staged form hands g*_0 over in a register
@@ -587,6 +591,8 @@ struct Sweep {
                     gs3 = g34.x;
                     gs4 = g34.y;
                 } else {
+                    const R Qs = C * dP;
+                    const R m3d = (g1 + g3) + (g2 + g4), m4 = (g1 + g3) - (g2 + g4);
                     const R m0s = Td + Qs;
                     const R m3s = m3d - P.vs3 * (m3d - P.w_dot * Td) + P.w_dot * Qs;
                     const R m4s = P.one_m_vs4 * m4;
@@ -612,7 +618,7 @@ struct Sweep {
                     cg[2] = g2;
                     cg[3] = g3;
                     cg[4] = g4;
-                    crho = rho;
+                    cC = C;
                     cgs0 = gs0;
                     cgs2 = gs2;
                     cgs4 = gs4;
@@ -620,7 +626,7 @@ struct Sweep {
                     S.gs[a0][1][t] = gs2;
                     R4 oo;
                     oo.x = g4;
-                    oo.y = rho;
+                    oo.y = sizeof(R) == 8 ? iC : C;   // what D5 divides by or multiplies with
                     oo.z = gs0;
                     oo.w = gs4;
                     S.own[bC][1][t] = oo;
@@ -689,7 +695,7 @@ struct Sweep {
                     else A3 = S.gs[a1][2][xr1];
                     const R A2 = vd ? egs2 : (dirS ? twS2 - dgs4 : dgs4);
                     const R A4 = vu ? cgs4 : (dirN ? twN2 - dgs2 : dgs2);
-                    const R iC = f_rcp(drho * P.cv);
+                    const R iC = f_rcp(dC);
                     go[0] = dg[0] + (dgs0 - dg[0]) * iC;
                     // g_i + (A_i - g_i) / (rho c_v) for (1, 3) and (2, 4) in pairs
                     const R2 iC2 = pr(iC, iC);
@@ -711,7 +717,7 @@ struct Sweep {
             egs2 = dgs2;
 #pragma unroll
             for (int q = 0; q < 5; ++q) dg[q] = cg[q];
-            drho = crho;
+            dC = cC;
             dgs0 = cgs0;
             dgs2 = cgs2;
             dgs4 = cgs4;
@@ -759,6 +765,9 @@ struct Sweep {
             }
             R q2, TdpdT;
             eos_node(P, rho_a, T_a, &q2, &TdpdT);
+            const R C_a = rho_a * P.cv;
+            const R iC_a = ir_a * P.inv_cv;
+            const R E_a = TdpdT * (iC_a * R(1.0 / 12.0));
             if (colvalid && !(q2 >= R(0))) errbits |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
             psi_a = f_sqrt(q2);
             S.psi[a0][t] = psi_a;
@@ -769,15 +778,16 @@ struct Sweep {
             }
             if constexpr (STG) {
                 R2 ow;
-                ow.x = rho_a;
-                ow.y = TdpdT;
+                ow.x = C_a;
+                ow.y = E_a;
                 S.own[b0][t] = ow;
             } else {
                 R4 o0, o1;
                 o0.x = ga[0]; o0.y = ga[1]; o0.z = ga[2]; o0.w = ga[3];
-                o1.x = ga[4]; o1.y = rho_a; o1.z = pa; o1.w = TdpdT;
+                o1.x = ga[4]; o1.y = C_a; o1.z = pa; o1.w = E_a;
                 S.own[b0][0][t] = o0;
                 S.own[b0][1][t] = o1;
+                if constexpr (sizeof(R) == 8) S.own2[b0][t] = pr(iC_a, Td);
             }
             // this unit's output rows only (steady iterations also load the
             // three rows above the segment)
@@ -832,13 +842,12 @@ struct Sweep {
                                     WR.T[a1][xr1], &errbits);
                 }
                 // Eq. 9 with varpi(1) = 1/3, varpi(2) = 1/12, both components
-                // at once: s = (pE - pW, pN - pS) / 3 + (dA + dB, dA - dB) / 12
+                // at once: 12 s = 4 (pE - pW, pN - pS) + (dA + dB, dA - dB)
                 const R dA = pNE - pSW, dB = pSE - pNW;
-                const R2 sxy = pfma(psub(pr(pE, pN), pr(pW, pS)), pr(R(1.0 / 3.0), R(1.0 / 3.0)),
-                                    pmul(pr(dA + dB, dA - dB), pr(R(1.0 / 12.0), R(1.0 / 12.0))));
-                const R sx = sxy.x, sy = sxy.y;
-                const R gp = P.negG * psip;
-                const R2 Fm = pmul(pr(gp, gp), sxy);
+                const R2 s12 = pfma(psub(pr(pE, pN), pr(pW, pS)), pr(R(4), R(4)),
+                                    pr(dA + dB, dA - dB));
+                const R gp = P.negG_12 * psip;
+                const R2 Fm = pmul(pr(gp, gp), s12);
                 const R Fx = Fm.x;
                 const R Fy = Fm.y - P.gravity * (rhop - rho_ave);
                 R ux = R(0), uy = R(0);
@@ -861,56 +870,8 @@ struct Sweep {
                             for (int q = 0; q < 9; ++q) fsw[q * NT] = fp[q];
                         }
                     } else if (UNIT) {
-                        // s_e = s_eps = s_q = 1: those moments leave the
-                        // collision at m^eq + F/2, so f* = M^{-1} m* needs of f
-                        // only rho, j and the stresses m_7, m_8 (Eqs. 5, 7, 8)
-                        const R rr = rhop;
-                        const R2 u2 = pr(ux, uy), F2 = pr(Fx, Fy);
-                        const R2 ru = pmul(pr(rr, rr), u2);          // rho u
-                        const R2 uu = pmul(ru, u2);                  // rho (ux^2, uy^2)
-                        const R2 uFc = pmul(u2, F2);                 // (ux Fx, uy Fy)
-                        const R2 s2 = pmul(sxy, sxy);
-                        const R ruu = uu.x + uu.y;
-                        const R uF = uFc.x + uFc.y;
-                        const R Fm2 = P.negG * P.negG * (s2.x + s2.y);
-                        const R m7 = m7p;
-                        const R m8 = m8p;
-                        const R F7 = R(2) * (uFc.x - uFc.y);
-                        const R F8 = ux * Fy + uy * Fx;
-                        // deviation-form m*_e, m*_eps (storage shifts them by
-                        // -2 rho_ref and rho_ref)
-                        const R t3 = R(3) * (ruu + uF);
-                        const R m1s = R(-2) * rhodp + t3 + R(0.5) * P.sig_e * Fm2;
-                        const R m2s = rhodp - t3 - R(0.5) * P.sig_eps * Fm2;
-                        const R b0 = rhodp * R(1.0 / 9.0);
-                        const R2 b12 = pmul(pr(m1s, m2s), pr(R(1.0 / 36.0), R(1.0 / 36.0)));
-                        const R b1 = b12.x, b2 = b12.y;
-                        const R b7 = (m7 - P.s_p * (m7 - (uu.x - uu.y)) + P.hs_p * F7) * R(0.25);
-                        const R b8 = (m8 - P.s_p * (m8 - ru.x * uy) + P.hs_p * F8) * R(0.25);
-                        // j* = j + F; q* = -(j + F) / 1 -> combined axis / diagonal terms
-                        const R2 js = padd(pr(jxp, jyp), F2);
-                        const R2 XY3 = pmul(js, pr(R(1.0 / 3.0), R(1.0 / 3.0)));
-                        const R2 XY12 = pmul(js, pr(R(1.0 / 12.0), R(1.0 / 12.0)));
-                        const R cax = b0 - b1 - R(2) * b2;
-                        const R cdg = b0 + R(2) * b1 + b2;
-                        // axis directions: (1, 2) = (cax + b7, cax - b7) + (X3, Y3),
-                        // (3, 4) = the same minus (X3, Y3); diagonals: (5, 8) =
-                        // (cdg + b8, cdg - b8) + (X12 + Y12, X12 - Y12), (7, 6) the
-                        // same minus
-                        const R2 cb = pr(cax + b7, cax - b7);
-                        const R2 f12 = padd(cb, XY3), f34 = psub(cb, XY3);
-                        const R2 db = pr(cdg + b8, cdg - b8);
-                        const R2 sd = pr(XY12.x + XY12.y, XY12.x - XY12.y);
-                        const R2 f58 = padd(db, sd), f76 = psub(db, sd);
-                        fsw[0 * NT] = b0 + R(4) * (b2 - b1);
-                        fsw[1 * NT] = f12.x;
-                        fsw[2 * NT] = f12.y;
-                        fsw[3 * NT] = f34.x;
-                        fsw[4 * NT] = f34.y;
-                        fsw[5 * NT] = f58.x;
-                        fsw[6 * NT] = f76.y;
-                        fsw[7 * NT] = f76.x;
-                        fsw[8 * NT] = f58.y;
+                        collide9_unit(P, rhop, rhodp, pr(jxp, jyp), m7p, m8p, pr(ux, uy), pr(Fx, Fy),
+                                      s12, fsw, NT);
                     } else {
                         const R* f = fp;
                         const R rr = rhop;
@@ -930,7 +891,7 @@ struct Sweep {
                         const R ne8 = (f[5] + f[7]) - (f[6] + f[8]) - rux * uy;
                         // Li forcing (Eq. 8); |F_m|^2 / psi^2 = G^2 |sum varpi psi c|^2
                         const R uF = ux * Fx + uy * Fy;
-                        const R Fm2 = P.negG * P.negG * (sx * sx + sy * sy);
+                        const R Fm2 = P.negG_12 * P.negG_12 * (s12.x * s12.x + s12.y * s12.y);
                         const R F1 = R(6) * uF + P.sig_e * Fm2;
                         const R F2 = R(-6) * uF - P.sig_eps * Fm2;
                         const R F7 = R(2) * (ux * Fx - uy * Fy);
@@ -992,7 +953,7 @@ struct Sweep {
                     if (vu) A4 = S.own[bC][1][t].w;
                     else A4 = dirN ? twN2 - gsc[1 * NT] : gsc[1 * NT];
                     const R A0 = o1.z;
-                    const R iC = f_rcp(o1.y * P.cv);
+                    const R iC = sizeof(R) == 8 ? o1.y : f_rcp(o1.y);
                     go[0] = o0.x + (A0 - o0.x) * iC;
                     // as in the staged form: (1, 3) and (2, 4) in pairs
                     const R2 iC2 = pr(iC, iC);
