@@ -368,7 +368,13 @@ int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged)
  * persistent grid in one wave.  The autotuner times load paths x thread
  * counts x heights (powers of two and the whole-wave heights) on a scratch
  * domain of the same size and precision, applies the fastest and caches the
- * choice per (precision, size). */
+ * choice per (precision, size).
+ * Small domains (up to about 740 x 740 in FP32, 600 x 600 in FP64) take another
+ * form of the same arithmetic unless a tile or load path is asked for: lbm_step
+ * runs up to 1024 steps in one cooperative launch over tiles of nodes.  The
+ * state is bit for bit the sweep's (with buoyancy, up to the rounding of the
+ * density sum).  lbm_set_tile and lbm_set_staging select the sweep,
+ * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile. */
 int lbm_set_tile(lbm_ctx* ctx, int threads, int rows);
 int lbm_get_tile(const lbm_ctx* ctx, int* threads, int* rows);
 int lbm_autotune(lbm_ctx* ctx, int steps_per_trial);

@@ -35,7 +35,7 @@
 
 #include "lbm.h"
 #include "lbm3d.h"
-#include "lbm_internal.cuh"
+#include "lbm_node.cuh"
 
 namespace lbm {
 namespace {

@@ -20,6 +20,7 @@ using namespace lbm;
 namespace {
 
 const int kGraphLen = 32;      // launches per captured graph
+const int kTileSteps = 1024;   // most steps per launch of the small-domain form
 const size_t kAlign = 256;
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -113,9 +114,9 @@ uint32_t crc32_update(uint32_t crc, const void* data, size_t n) {
     return ~crc;
 }
 
-// tile autotuner cache: (prec, nx, ny) -> (threads, rows, staged)
+// tile autotuner cache: (prec, nx, ny) -> (threads, rows, staged, small form)
 struct Tile {
-    int threads, rows, staged;
+    int threads, rows, staged, tiled;
 };
 std::map<std::tuple<int, int, int>, Tile>& tune_cache() {
     static std::map<std::tuple<int, int, int>, Tile> m;
@@ -213,6 +214,8 @@ struct lbm_ctx {
     unsigned* sched = nullptr;
     Unit* units = nullptr;
     int n_units = 0, grid = 1, threads = 128, rows = 64, staged = 0, wait_probe = 0;
+    TilePlan tile;             // small-domain form (tile.tx == 0: not for this domain)
+    bool tiled = false;        // lbm_step takes it (unless a sweep tile was asked for)
     cudaGraphExec_t graph = nullptr;
     long long step = 0;
     long long target = 0;      // the step the domain stops at (0: none), as on the device
@@ -349,6 +352,25 @@ static int enqueue_steps(cudaStream_t st, cudaGraphExec_t* graph, const StepLaun
     }
     for (int i = 0; i < n; ++i)
         if (step_launch(prec, threads, L, st)) return cuda_err(errctx, cudaGetLastError(), "step launch");
+    return LBM_OK;
+}
+
+// queues n steps of the small-domain form
+static int enqueue_tiled(lbm_ctx* c, int n) {
+    TileLaunch L;
+    L.inst = c->inst;
+    L.bar = c->sched;
+    L.tx = c->tile.tx;
+    L.ty = c->tile.ty;
+    L.ring0 = c->tile.ring0;
+    L.ntx = c->tile.ntx;
+    L.n_tiles = c->tile.n_tiles;
+    L.targets = c->target > 0 ? 1 : 0;
+    for (; n > 0; n -= L.steps) {
+        L.steps = std::min(n, kTileSteps);
+        if (tile_launch(c->prec, c->tile, L, c->phys, c->stream))
+            return cuda_err(c, cudaGetLastError(), "step launch");
+    }
     return LBM_OK;
 }
 
@@ -502,10 +524,13 @@ int lbm_create(int nx, int ny, const lbm_params* params, const lbm_bc* bc, int p
                             staged, nx, ny);
     }
     int rc = ctx_apply_tile(c, threads, rows, staged);
+    if (rc == LBM_OK && tile_plan(prec, I, c->phys, num_sms(), &c->tile))
+        rc = set_err(c, LBM_ECUDA, "occupancy query failed");
     if (rc) {
         lbm_destroy(c);
         return rc;
     }
+    c->tiled = c->tile.tx > 0 && (it == tune_cache().end() || it->second.tiled);
     *out = c;
     return LBM_OK;
 }
@@ -548,6 +573,8 @@ int lbm_init_fields(lbm_ctx* c, const double* rho, const double* ux, const doubl
     memset(&h, 0, sizeof(h));
     h.mass[2] = sr;
     e = cudaMemcpyAsync(c->ctl, &h, sizeof(h), cudaMemcpyHostToDevice, c->stream);
+    // the launches leave their work counters at 0 unless a wait ran out
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->sched, 0, 2 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_err(c, e, "lbm_init_fields");
     c->step = 0;
@@ -590,7 +617,8 @@ int lbm_step(lbm_ctx* c, int n) {
     if (c->batch) return set_err(c, LBM_ESTATE, "context is attached to a batch");
     if (c->sticky) return c->sticky;
     if (n == 0) return LBM_OK;
-    int rc = enqueue_steps(c->stream, &c->graph, ctx_launch(c), c->prec, c->threads, n, c);
+    int rc = c->tiled ? enqueue_tiled(c, n)
+                      : enqueue_steps(c->stream, &c->graph, ctx_launch(c), c->prec, c->threads, n, c);
     if (rc == LBM_OK) c->step = step_after(c, n);
     return rc;
 }
@@ -708,6 +736,7 @@ int lbm_set_populations(lbm_ctx* c, const double* f, const double* g, const doub
     h.step = step;
     h.mass[(step + 2) % 3] = rho_ave_prev * (double)N;
     if (!rc) rc = cuda_err(c, cudaMemcpyAsync(c->ctl, &h, sizeof(h), cudaMemcpyHostToDevice, c->stream), "ctl");
+    if (!rc) rc = cuda_err(c, cudaMemsetAsync(c->sched, 0, 2 * sizeof(unsigned), c->stream), "work counters");
     if (!rc) rc = cuda_err(c, cudaStreamSynchronize(c->stream), "lbm_set_populations");
     cudaFree(buf);
     if (rc) return rc;
@@ -875,6 +904,7 @@ int lbm_load(lbm_ctx* c, const char* path) {
     for (int k = 0; k < 3; ++k) h.mass[k] = hd.mass[k];
     if (e == cudaSuccess) e = cudaMemcpy(c->ctl, &h, sizeof(h), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->inst_dev, &c->inst, sizeof(Inst), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(c->sched, 0, 2 * sizeof(unsigned));
     if (e != cudaSuccess) return cuda_err(c, e, "lbm_load");
     c->step = hd.step;
     c->target = 0;
@@ -1072,7 +1102,9 @@ int lbm_set_tile(lbm_ctx* c, int threads, int rows) {
     if (!c || (threads != 128 && threads != 192 && threads != 224 && threads != 256) || rows < 1)
         return LBM_EINVAL;
     if (c->batch) return set_err(c, LBM_ESTATE, "context is attached to a batch");
-    return ctx_apply_tile(c, threads, std::min(rows, c->ny), c->staged);
+    int rc = ctx_apply_tile(c, threads, std::min(rows, c->ny), c->staged);
+    if (rc == LBM_OK) c->tiled = false;
+    return rc;
 }
 
 int lbm_set_staging(lbm_ctx* c, int on) {
@@ -1082,7 +1114,9 @@ int lbm_set_staging(lbm_ctx* c, int on) {
         return set_err(c, LBM_EINVAL,
                        "bulk-copy staging needs FP32 storage of f and open x, or periodic x "
                        "with nx >= 32 a multiple of 4 (FP32 g) or 8 (FP16 g)");
-    return ctx_apply_tile(c, c->threads, c->rows, on ? 1 : 0);
+    int rc = ctx_apply_tile(c, c->threads, c->rows, on ? 1 : 0);
+    if (rc == LBM_OK) c->tiled = false;
+    return rc;
 }
 
 int lbm_get_staging(const lbm_ctx* c) { return c ? c->staged : LBM_EINVAL; }
@@ -1146,6 +1180,7 @@ int lbm_autotune(lbm_ctx* c, int steps) {
             rows_c.erase(std::unique(rows_c.begin(), rows_c.end()), rows_c.end());
             for (int rows : rows_c) {
                 if (ctx_apply_tile(s, thr_c[ti], rows, staged)) continue;
+                s->tiled = false;
                 lbm_step(s, 2);
                 cudaEventRecord(e0, s->stream);
                 lbm_step(s, steps);
@@ -1161,11 +1196,24 @@ int lbm_autotune(lbm_ctx* c, int steps) {
                 }
             }
         }
+    bool tiled = false;
+    if (s->tile.tx > 0) {
+        s->tiled = true;
+        lbm_step(s, 2);
+        cudaEventRecord(e0, s->stream);
+        lbm_step(s, steps);
+        cudaEventRecord(e1, s->stream);
+        float ms = 0.f;
+        if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
+            tiled = ms < best;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     lbm_destroy(s);
-    tune_cache()[std::make_tuple(c->prec, c->nx, c->ny)] = Tile{bt, br, bs};
-    return ctx_apply_tile(c, bt, br, bs);
+    tune_cache()[std::make_tuple(c->prec, c->nx, c->ny)] = Tile{bt, br, bs, tiled ? 1 : 0};
+    rc = ctx_apply_tile(c, bt, br, bs);
+    if (rc == LBM_OK) c->tiled = tiled;
+    return rc;
 }
 
 // ---- batch ---------------------------------------------------------------

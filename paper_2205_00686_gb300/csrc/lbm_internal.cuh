@@ -102,7 +102,7 @@ struct Phys {
     R u_ax, u_dg, u_0;               // the sigma terms' factors of |12 s|^2
     // D2Q5
     R cv, inv_cv, w_dot, w5_0, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
-    R one_m_vs1, one_m_vs4;
+    R h_m, one_m_vs4;               // h_m = (1 - vs1) / 2
     R gravity;
     int frozen_flow, frozen_thermal;
 };
@@ -160,7 +160,7 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.vs1_cs2h = (R)(d.vs1 / (0.5 * d.w_dot));
     p.vs3 = (R)d.vs3;
     p.vs4 = (R)d.vs4;
-    p.one_m_vs1 = (R)(1.0 - d.vs1);
+    p.h_m = (R)(0.5 * (1.0 - d.vs1));
     p.one_m_vs4 = (R)(1.0 - d.vs4);
     p.gravity = (R)d.gravity;
     p.frozen_flow = d.frozen_flow;
@@ -200,8 +200,7 @@ __device__ __forceinline__ float f_rcp(float x) {
 // is left out is of order e^3 ~ 2^-60, below the FP64 rounding, so the result
 // is within about one ulp (not always the correctly rounded value).  Three
 // and five FP64 instructions, against four for two Newton-Raphson steps and
-// about ten for the IEEE square root.  With eos_node, collide9_unit and the
-// rho c_v forms of the step's thermal stages, which count FP64 operations the
+// about ten for the IEEE square root.  With the node arithmetic of lbm_node.cuh, which count FP64 operations the
 // same way (about 168 per node instead of 220), the FP64 step on 1999 x 1501
 // went from 1.355 to 1.067 ms; in FP32 the same forms took the 4096^2 step
 // from 340.3 to 336.1 us.  A zero, infinite or NaN reciprocal
@@ -230,32 +229,6 @@ __device__ __forceinline__ double f_sqrt(double x) {
     return fma(t * e, fma(0.375, e, 0.5), t);
 }
 
-// Two-lane arithmetic.  In float it maps to Blackwell's paired FP32
-// instructions (one FADD2 / FMUL2 / FFMA2 does the work of two), each lane
-// rounded as the scalar operation; in double it is componentwise.  Subtraction
-// is a fused multiply-add with -1, which is exact in the product.
-__device__ __forceinline__ float2 pr(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 pr(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ double2 pmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c) {
-    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
-}
-// c - a b
-__device__ __forceinline__ float2 pnfma(float2 a, float2 b, float2 c) {
-    return __ffma2_rn(a, make_float2(-b.x, -b.y), c);
-}
-__device__ __forceinline__ double2 pnfma(double2 a, double2 b, double2 c) {
-    return make_double2(fma(-a.x, b.x, c.x), fma(-a.y, b.y, c.y));
-}
-__device__ __forceinline__ float2 psub(float2 a, float2 b) {
-    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
-}
-__device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-
 // Peng-Robinson pressure (Eq. 10) and psi^2 = 2 (p_EOS - rho/3) / G.
 template <class R>
 __device__ __forceinline__ R eos_p(const Phys<R>& P, R rho, R T) {
@@ -268,69 +241,6 @@ __device__ __forceinline__ R eos_p(const Phys<R>& P, R rho, R T) {
 template <class R>
 __device__ __forceinline__ R psi2_of(const Phys<R>& P, R rho, R T) {
     return P.two_over_G * (eos_p(P, rho, T) - rho * R(1.0 / 3.0));
-}
-
-// psi^2 and T (dp/dT)_rho of one node, with D1 = 1 - b rho and
-// D2 = 1 + 2 b rho - b^2 rho^2 = 2 - D1^2 over one common reciprocal:
-//   p = rho (Rg T D2 - a h^2 rho D1) / (D1 D2)
-//   T (dp/dT)_rho = rho (Rg T D2 + a k h sqrt(T/Tc) rho D1) / (D1 D2)
-// (T / sqrt(T/Tc) = Tc sqrt(T/Tc), so no second reciprocal).  One square
-// root and one reciprocal, 22 other operations.
-template <class R>
-__device__ __forceinline__ void eos_node(const Phys<R>& P, R rho, R T, R* psi2, R* TdpdT) {
-    const R st = f_sqrt(T * P.inv_Tc);
-    const R h = P.one_p_kpr - P.kpr * st;
-    const R ah = P.a * h;
-    const R d1 = R(1) - P.b * rho;
-    const R d2 = R(2) - d1 * d1;
-    const R s = rho * f_rcp(d1 * d2);
-    const R u = P.Rg * T * d2, w = rho * d1;
-    const R p = s * (u - ah * h * w);
-    *psi2 = P.two_over_G * (p - rho * R(1.0 / 3.0));
-    *TdpdT = s * (u + P.kpr * ah * st * w);
-}
-
-// D2Q9 collision at unit rates (s_e = s_eps = s_q = 1: those moments leave the
-// collision at m^eq + F/2), so f* = M^{-1} m* needs of f only rho, j and the
-// stress moments m_7, m_8 (Eqs. 5, 7, 8).  With K = rho u.u + u.F and
-// |12 s|^2 of the force stencil,
-//   f*_0          = 4/9 rho - 2/3 K + u_0 |12 s|^2
-//   axis part     = 1/9 rho + 1/12 K + u_ax |12 s|^2, +- m*_7/4, +- (j + F)/3
-//   diagonal part = 1/36 rho + 1/12 K + u_dg |12 s|^2, +- m*_8/4,
-//                   +- ((j + F)_x +- (j + F)_y)/12
-// rhod: deviation of rho from the storage reference (f is stored as
-// deviations); rho: the density itself.
-template <class R, class R2>
-__device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rho, R rhod, R2 j, R m7, R m8,
-                                              R2 u, R2 F, R2 s12, R* f, int stride) {
-    const R2 ru = pmul(pr(rho, rho), u);
-    const R2 uu = pmul(ru, u);      // rho (ux^2, uy^2)
-    const R2 uF = pmul(u, F);       // (ux Fx, uy Fy)
-    const R2 K2 = padd(uu, uF);
-    const R K = K2.x + K2.y;
-    const R S = s12.x * s12.x + s12.y * s12.y;
-    const R b7 = P.u_m * m7 + (P.u_d * (uu.x - uu.y) + P.u_g7 * (uF.x - uF.y));
-    const R b8 = P.u_m * m8 + (P.u_d * (ru.x * u.y) + P.u_g8 * (u.x * F.y + u.y * F.x));
-    const R2 cc = pfma(pr(rhod, rhod), pr(R(1.0 / 9.0), R(1.0 / 36.0)),
-                       pfma(pr(S, S), pr(P.u_ax, P.u_dg), pr(K * R(1.0 / 12.0), K * R(1.0 / 12.0))));
-    const R2 js = padd(j, F);
-    // axis directions: (1, 2) = (ax + b7, ax - b7) + js/3, (3, 4) the same
-    // minus js/3; diagonals: (5, 8) = (dg + b8, dg - b8) + (jx + jy, jx - jy)/12,
-    // (7, 6) the same minus that
-    const R2 cb = pr(cc.x + b7, cc.x - b7), db = pr(cc.y + b8, cc.y - b8);
-    const R2 sd = pr(js.x + js.y, js.x - js.y);
-    const R2 t3 = pr(R(1.0 / 3.0), R(1.0 / 3.0)), t12 = pr(R(1.0 / 12.0), R(1.0 / 12.0));
-    const R2 f12 = pfma(js, t3, cb), f58 = pfma(sd, t12, db);
-    const R2 f34 = pnfma(js, t3, cb), f76 = pnfma(sd, t12, db);
-    f[0] = rhod * R(4.0 / 9.0) + (P.u_0 * S - K * R(2.0 / 3.0));
-    f[1 * stride] = f12.x;
-    f[2 * stride] = f12.y;
-    f[3 * stride] = f34.x;
-    f[4 * stride] = f34.y;
-    f[5 * stride] = f58.x;
-    f[6 * stride] = f76.y;
-    f[7 * stride] = f76.x;
-    f[8 * stride] = f58.y;
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {
@@ -379,6 +289,27 @@ inline bool stage_eligible(const Inst& I, int prec) {
     if (prec != 1 && prec != 2) return false;
     if (I.flow[EW] != PERIODIC) return true;
     return I.nx % (prec == 2 ? 8 : 4) == 0 && I.nx >= 32;
+}
+
+// Small-domain form (lbm_tile.cu): tiles of tx x ty nodes, one thread per
+// node, several steps per launch.  tx = 0: the domain takes the sweep.
+struct TilePlan {
+    int tx = 0, ty = 0, threads = 0, ring0 = 0, ntx = 0, n_tiles = 0, grid = 0;
+    size_t smem = 0;
+};
+struct TileLaunch {
+    Inst inst;
+    unsigned* bar;     // grid counter, 0 between launches
+    int tx, ty, ring0, ntx, n_tiles, steps;
+    int targets;       // the domain has a target step (lbm_set_target)
+};
+int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out);
+int tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys, cudaStream_t st);
+
+// The unit-rate form applies when every non-hydrodynamic rate is exactly 1
+// (s_e = s_eps = s_q = 1 and varsigma_3 = varsigma_4 = 1, the paper's choice).
+inline bool unit_rates(const PhysD& d) {
+    return d.s_e == 1.0 && d.s_eps == 1.0 && d.s_q == 1.0 && d.vs3 == 1.0 && d.vs4 == 1.0;
 }
 
 int step_launch(int prec, int threads, const StepLaunch& L, cudaStream_t st);

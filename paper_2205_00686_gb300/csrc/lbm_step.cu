@@ -43,16 +43,10 @@
 // ever waits on another.
 #include <type_traits>
 
-#include "lbm_internal.cuh"
+#include "lbm_node.cuh"
 
 namespace lbm {
 
-template <class R>
-struct Vec2;
-template <>
-struct Vec2<float> { typedef float2 T; };
-template <>
-struct Vec2<double> { typedef double2 T; };
 template <class R>
 struct Vec4;
 template <>
@@ -157,11 +151,6 @@ __device__ __forceinline__ bool mbar_test(unsigned long long* m, unsigned parity
         : "memory");
     return ok != 0;
 }
-// a product rounded on its own, never fused into a later add (a value that
-// one stage hands to another in a register then rounds as one passed through
-// shared memory)
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 // bounded wait for an mbarrier phase: gives up after ~2^31 clocks (about a
 // second at the GB300's clock), records ERR_TIMEOUT and sets *stalled; a
 // thread that has stalled does not wait again on the same pipeline (its
@@ -178,17 +167,6 @@ __device__ __forceinline__ void wait_row(unsigned long long* m, unsigned parity,
             return;
         }
     }
-}
-
-// ghost-layer psi of a wall (Section 3.3): rho_ghost = rho(layer 2) +
-// tan(pi/2 - theta) |rho(x+1, layer 1) - rho(x-1, layer 1)|
-template <class R>
-__device__ __forceinline__ R ghost_psi(const Phys<R>& P, R rho_far, R rho_p, R rho_m, R cot, R Tg,
-                                       int* err) {
-    const R rg = rho_far + cot * rabs(rho_p - rho_m);
-    const R q2 = psi2_of(P, rg, Tg);
-    if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
-    return f_sqrt(q2);
 }
 
 // State of one CTA's sweep over one unit.  iter<STEADY>(k) runs both phases
@@ -533,17 +511,14 @@ struct Sweep {
                     g0 = o0.x; g1 = o0.y; g2 = o0.z; g3 = o0.w; g4 = o1.x;
                     C = o1.y; Pp = o1.z; E = o1.w;
                 }
-                // (m_1, m_2) = (g1 - g3, g2 - g4)
-                const R2 m12 = psub(pr(g1, g2), pr(g3, g4));
-                const R m1 = m12.x, m2 = m12.y;
                 R Td, iC = R(0);
+                const R gl[5] = {g0, g1, g2, g3, g4};
                 if constexpr (sizeof(R) == 8) {
                     const R2 o2 = S.own2[bC][t];
                     iC = o2.x;
                     Td = o2.y;
                 } else {
-                    const R2 p13 = padd(pr(g1, g2), pr(g3, g4));
-                    Td = (g0 + p13.x) + p13.y;
+                    Td = sum5(gl);
                 }
                 // neighbour rows: solid -> u = 0, open -> the boundary row
                 const bool vd = STEADY || pery || r - 1 >= 0, vu = STEADY || pery || r + 1 < ny;
@@ -562,54 +537,16 @@ struct Sweep {
                 } else {
                     uN0.x = uN0.y = uN1.x = uN1.y = uN2.x = uN2.y = R(0);
                 }
-                // isotropic central difference, 12 (1/c_s^2) sum_i w_i c_i phi(x + c_i)
-                const R div12 = (uE.x - uW.x + uN1.y - uS1.y) * R(4) +
-                                ((uN2.x + uS2.x - uN0.x - uS0.x) +
-                                 (uN2.y + uN0.y - uS2.y - uS0.y));
-                // P^n = Q / (rho c_v) = -[u.grad T + T (dp/dT)_rho div u / (rho c_v)]
-                // (Eq. 20) with c_s^2 grad T = -varsigma_1 (m_1, m_2) (Eqs. 49-50,
-                // m^eq = 0) and E = T (dp/dT)_rho / (12 rho c_v)
-                const R Pn = P.vs1_cs2h * (uc.x * m1 + uc.y * m2) - E * div12;
-                // S = w^ rho c_v (dt/2) d_t^2 T with d_t^2 T ~ P^n - P^{n-1}
-                // (Eq. 24): Q + S = rho c_v (P^n + (P^n - P^{n-1}) / 2)
-                const R dP = first ? Pn : Pn + R(0.5) * (Pn - Pp);
-                // moment-space collision (Eqs. 39, 40, 47), deviation form
-                const R hc = R(0.5) * P.one_m_vs1;
-                const R2 h12 = pmul(pr(hc, hc), m12);
-                const R h1 = h12.x, h2 = h12.y;
-                R gs0, gs1, gs2, gs3, gs4;
-                if (UNIT) {
-                    // varsigma_3 = varsigma_4 = 1: m3* = w_dot (T + Qs), m4* = 0
-                    const R TQ = Td + C * dP;
-                    const R a = R(0.25) * P.w_dot * TQ;
-                    // unfused: stage D5 subtracts g_0 from g*_0, and the
-                    // staged form hands g*_0 over in a register
-                    gs0 = mul_rn(P.w5_0, TQ);
-                    const R2 g12 = padd(pr(a, a), h12), g34 = psub(pr(a, a), h12);
-                    gs1 = g12.x;
-                    gs2 = g12.y;
-                    gs3 = g34.x;
-                    gs4 = g34.y;
-                } else {
-                    const R Qs = C * dP;
-                    const R m3d = (g1 + g3) + (g2 + g4), m4 = (g1 + g3) - (g2 + g4);
-                    const R m0s = Td + Qs;
-                    const R m3s = m3d - P.vs3 * (m3d - P.w_dot * Td) + P.w_dot * Qs;
-                    const R m4s = P.one_m_vs4 * m4;
-                    const R a = R(0.25) * (m3s + m4s), b = R(0.25) * (m3s - m4s);
-                    gs0 = m0s - m3s;
-                    gs1 = a + h1;
-                    gs2 = b + h2;
-                    gs3 = a - h1;
-                    gs4 = b - h2;
-                }
+                const R div12 = div12_of<R>(uW, uE, uS0, uS1, uS2, uN0, uN1, uN2);
+                R gs[5];
+                const R Pn = thermal5<UNIT>(P, gl, Td, C, E, uc, div12, Pp, first, gs);
                 // g*_1 and g*_3 are read by the neighbour columns; g*_0, g*_2
                 // and g*_4 only by this column's stage D5 (rows r, r + 1 and
                 // r - 1).  The register-prefetch form keeps g*_2 in the gs
                 // ring and g*_0, g*_4 in the row's own slot in place of
                 // P^{n-1} and T (dp/dT)_rho
-                S.gs[a0][0][t] = gs1;
-                S.gs[a0][2][t] = gs3;
+                S.gs[a0][0][t] = gs[1];
+                S.gs[a0][2][t] = gs[3];
                 if constexpr (STG) {
                     // the rest is read only by this column's D5 (rows r and
                     // r + 1): registers
@@ -619,16 +556,16 @@ struct Sweep {
                     cg[3] = g3;
                     cg[4] = g4;
                     cC = C;
-                    cgs0 = gs0;
-                    cgs2 = gs2;
-                    cgs4 = gs4;
+                    cgs0 = gs[0];
+                    cgs2 = gs[2];
+                    cgs4 = gs[4];
                 } else {
-                    S.gs[a0][1][t] = gs2;
+                    S.gs[a0][1][t] = gs[2];
                     R4 oo;
                     oo.x = g4;
                     oo.y = sizeof(R) == 8 ? iC : C;   // what D5 divides by or multiplies with
-                    oo.z = gs0;
-                    oo.w = gs4;
+                    oo.z = gs[0];
+                    oo.w = gs[4];
                     S.own[bC][1][t] = oo;
                 }
                 if (inD && (STEADY || (r >= y0 && r < y1))) Pdst[(size_t)r * pitch + gx] = Pn;
@@ -695,8 +632,8 @@ struct Sweep {
                     else A3 = S.gs[a1][2][xr1];
                     const R A2 = vd ? egs2 : (dirS ? twS2 - dgs4 : dgs4);
                     const R A4 = vu ? cgs4 : (dirN ? twN2 - dgs2 : dgs2);
-                    const R iC = f_rcp(dC);
-                    go[0] = dg[0] + (dgs0 - dg[0]) * iC;
+                    const R iC = blend_iC(dC, R(0));
+                    go[0] = blend(dg[0], dgs0, iC);
                     // g_i + (A_i - g_i) / (rho c_v) for (1, 3) and (2, 4) in pairs
                     const R2 iC2 = pr(iC, iC);
                     const R2 g13 = pr(dg[1], dg[3]), g24 = pr(dg[2], dg[4]);
@@ -747,47 +684,37 @@ struct Sweep {
             }
         }
         if (doA && (STEADY || colvalid)) {
-            // pair sums and differences of (f1, f2) & (f3, f4) and (f5, f6) & (f7, f8)
-            const R2 sA = padd(pr(fa[1], fa[2]), pr(fa[3], fa[4]));   // (f1 + f3, f2 + f4)
-            const R2 dA = psub(pr(fa[1], fa[2]), pr(fa[3], fa[4]));   // (f1 - f3, f2 - f4)
-            const R2 sB = padd(pr(fa[5], fa[6]), pr(fa[7], fa[8]));   // (f5 + f7, f6 + f8)
-            const R2 dB = psub(pr(fa[5], fa[6]), pr(fa[7], fa[8]));   // (f5 - f7, f6 - f8)
-            rhod_a = (fa[0] + (sA.x + sA.y)) + (sB.x + sB.y);
-            rho_a = rhod_a + rho_ref;
-            ir_a = f_rcp(rho_a);
-            const R Td = ((ga[0] + ga[1]) + (ga[2] + ga[3])) + ga[4];
-            const R T_a = Td + T_ref;
-            jx_a = dA.x + (dB.x - dB.y);    // (f1 - f3) + (f5 - f7) - (f6 - f8)
-            jy_a = dA.y + (dB.x + dB.y);    // (f2 - f4) + (f5 - f7) + (f6 - f8)
+            Node<R> nd;
+            node_fields(P, rho_ref, T_ref, fa, ga, nd);
+            rhod_a = nd.rhod;
+            rho_a = nd.rho;
+            ir_a = nd.ir;
+            jx_a = nd.jx;
+            jy_a = nd.jy;
             if constexpr (UNIT) {
-                m7_a = sA.x - sA.y;
-                m8_a = sB.x - sB.y;
+                m7_a = nd.m7;
+                m8_a = nd.m8;
             }
-            R q2, TdpdT;
-            eos_node(P, rho_a, T_a, &q2, &TdpdT);
-            const R C_a = rho_a * P.cv;
-            const R iC_a = ir_a * P.inv_cv;
-            const R E_a = TdpdT * (iC_a * R(1.0 / 12.0));
-            if (colvalid && !(q2 >= R(0))) errbits |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
-            psi_a = f_sqrt(q2);
+            if (colvalid && !(nd.q2 >= R(0))) errbits |= (nd.q2 != nd.q2) ? ERR_NONFINITE : ERR_PSI;
+            psi_a = nd.psi;
             S.psi[a0][t] = psi_a;
             if (wallS || wallN) {
                 // only the wetting ghost layer reads rho and T of neighbours
                 WR.rho[a0][t] = rho_a;
-                WR.T[a0][t] = T_a;
+                WR.T[a0][t] = nd.T;
             }
             if constexpr (STG) {
                 R2 ow;
-                ow.x = C_a;
-                ow.y = E_a;
+                ow.x = nd.C;
+                ow.y = nd.E;
                 S.own[b0][t] = ow;
             } else {
                 R4 o0, o1;
                 o0.x = ga[0]; o0.y = ga[1]; o0.z = ga[2]; o0.w = ga[3];
-                o1.x = ga[4]; o1.y = C_a; o1.z = pa; o1.w = E_a;
+                o1.x = ga[4]; o1.y = nd.C; o1.z = pa; o1.w = nd.E;
                 S.own[b0][0][t] = o0;
                 S.own[b0][1][t] = o1;
-                if constexpr (sizeof(R) == 8) S.own2[b0][t] = pr(iC_a, Td);
+                if constexpr (sizeof(R) == 8) S.own2[b0][t] = pr(nd.iC, nd.Td);
             }
             // this unit's output rows only (steady iterations also load the
             // three rows above the segment)
@@ -841,24 +768,10 @@ struct Sweep {
                     pNE = ghost_psi(P, WR.rho[a2][xr1], WR.rho[a1][cRR], WR.rho[a1][cRL], cot,
                                     WR.T[a1][xr1], &errbits);
                 }
-                // Eq. 9 with varpi(1) = 1/3, varpi(2) = 1/12, both components
-                // at once: 12 s = 4 (pE - pW, pN - pS) + (dA + dB, dA - dB)
-                const R dA = pNE - pSW, dB = pSE - pNW;
-                const R2 s12 = pfma(psub(pr(pE, pN), pr(pW, pS)), pr(R(4), R(4)),
-                                    pr(dA + dB, dA - dB));
-                const R gp = P.negG_12 * psip;
-                const R2 Fm = pmul(pr(gp, gp), s12);
-                const R Fx = Fm.x;
-                const R Fy = Fm.y - P.gravity * (rhop - rho_ave);
-                R ux = R(0), uy = R(0);
-                if (!P.frozen_flow) {
-                    const R2 uu2 = pmul(pfma(pr(Fx, Fy), pr(R(0.5), R(0.5)), pr(jxp, jyp)), pr(irp, irp));
-                    ux = uu2.x;
-                    uy = uu2.y;
-                }
-                R2 uv;
-                uv.x = ux;
-                uv.y = uy;
+                const R2 s12 = force_stencil<R>(pW, pE, pSW, pS, pSE, pNW, pN, pNE);
+                const R2 F = force_of<R>(P, s12, psip, rhop, rho_ave);
+                R2 uv = pr(R(0), R(0));
+                if (!P.frozen_flow) uv = velocity<R>(F, pr(jxp, jyp), irp);
                 S.u[a1][t] = uv;
                 if (STEADY || (r >= y0 - 1 && r < y1 + 1 && inC)) {
                     R* fsw = &S.fs[a1][0][t];
@@ -870,56 +783,9 @@ struct Sweep {
                             for (int q = 0; q < 9; ++q) fsw[q * NT] = fp[q];
                         }
                     } else if (UNIT) {
-                        collide9_unit(P, rhop, rhodp, pr(jxp, jyp), m7p, m8p, pr(ux, uy), pr(Fx, Fy),
-                                      s12, fsw, NT);
+                        collide9_unit(P, rhop, rhodp, pr(jxp, jyp), m7p, m8p, uv, F, s12, fsw, NT);
                     } else {
-                        const R* f = fp;
-                        const R rr = rhop;
-                        const R rux = rr * ux, ruy = rr * uy;
-                        const R ruu = rux * ux + ruy * uy;
-                        const R s14 = (f[1] + f[3]) + (f[2] + f[4]);
-                        const R s58 = (f[5] + f[7]) + (f[6] + f[8]);
-                        // non-equilibrium parts m - m^eq of the moments of Eq. 7
-                        // (deviation storage shifts m_e by -2 rho_ref, m_eps by rho_ref)
-                        const R ne1 = R(2) * (s58 + rhodp - f[0]) - (R(2) * f[0] + s14) - R(3) * ruu;
-                        const R ne2 = (R(4) * f[0] - R(2) * s14 + s58) - rhodp + R(3) * ruu;
-                        const R d13 = f[1] - f[3], d24 = f[2] - f[4];
-                        const R d58 = f[5] - f[7], d68 = f[6] - f[8];
-                        const R ne4 = (d58 - d68 - R(2) * d13) + rux;
-                        const R ne6 = (d58 + d68 - R(2) * d24) + ruy;
-                        const R ne7 = (f[1] + f[3]) - (f[2] + f[4]) - (rux * ux - ruy * uy);
-                        const R ne8 = (f[5] + f[7]) - (f[6] + f[8]) - rux * uy;
-                        // Li forcing (Eq. 8); |F_m|^2 / psi^2 = G^2 |sum varpi psi c|^2
-                        const R uF = ux * Fx + uy * Fy;
-                        const R Fm2 = P.negG_12 * P.negG_12 * (s12.x * s12.x + s12.y * s12.y);
-                        const R F1 = R(6) * uF + P.sig_e * Fm2;
-                        const R F2 = R(-6) * uF - P.sig_eps * Fm2;
-                        const R F7 = R(2) * (ux * Fx - uy * Fy);
-                        const R F8 = ux * Fy + uy * Fx;
-                        // m* - m = -S (m - m^eq) + (I - S/2) F; for j the
-                        // change is exactly F because rho u = j + F/2
-                        const R a1m = (P.hs_e * F1 - P.s_e * ne1) * R(1.0 / 36.0);
-                        const R a2m = (P.hs_eps * F2 - P.s_eps * ne2) * R(1.0 / 36.0);
-                        const R a3 = Fx * R(1.0 / 6.0), a5 = Fy * R(1.0 / 6.0);
-                        const R a4 = -(P.s_q * ne4 + P.hs_q * Fx) * R(1.0 / 12.0);
-                        const R a6 = -(P.s_q * ne6 + P.hs_q * Fy) * R(1.0 / 12.0);
-                        const R a7 = (P.hs_p * F7 - P.s_p * ne7) * R(0.25);
-                        const R a8 = (P.hs_p * F8 - P.s_p * ne8) * R(0.25);
-                        // f* = f + M^{-1} (m* - m), M^{-1} = M^T diag(1/9, 1/36,
-                        // 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
-                        const R cax = -a1m - R(2) * a2m;   // common to the axis directions
-                        const R cdg = R(2) * a1m + a2m;    // common to the diagonals
-                        const R ex = a3 - R(2) * a4, ey = a5 - R(2) * a6;
-                        const R dx = a3 + a4, dy = a5 + a6;
-                        fsw[0 * NT] = f[0] + R(4) * (a2m - a1m);
-                        fsw[1 * NT] = f[1] + cax + ex + a7;
-                        fsw[2 * NT] = f[2] + cax + ey - a7;
-                        fsw[3 * NT] = f[3] + cax - ex + a7;
-                        fsw[4 * NT] = f[4] + cax - ey - a7;
-                        fsw[5 * NT] = f[5] + cdg + dx + dy + a8;
-                        fsw[6 * NT] = f[6] + cdg - dx + dy - a8;
-                        fsw[7 * NT] = f[7] + cdg - dx - dy + a8;
-                        fsw[8 * NT] = f[8] + cdg + dx - dy - a8;
+                        collide9(P, rhop, rhodp, fp, uv, F, s12, fsw, NT);
                     }
                 }
             }
@@ -953,8 +819,8 @@ struct Sweep {
                     if (vu) A4 = S.own[bC][1][t].w;
                     else A4 = dirN ? twN2 - gsc[1 * NT] : gsc[1 * NT];
                     const R A0 = o1.z;
-                    const R iC = sizeof(R) == 8 ? o1.y : f_rcp(o1.y);
-                    go[0] = o0.x + (A0 - o0.x) * iC;
+                    const R iC = blend_iC(o1.y, o1.y);
+                    go[0] = blend(o0.x, A0, iC);
                     // as in the staged form: (1, 3) and (2, 4) in pairs
                     const R2 iC2 = pr(iC, iC);
                     const R2 g13 = pr(o0.y, o0.w), g24 = pr(o0.z, o1.x);
@@ -1130,12 +996,6 @@ __global__ void __launch_bounds__(NT, (PREC == 0) ? 1 : (512 / NT))
             __threadfence();
         }
     }
-}
-
-// The unit-rate form applies when every non-hydrodynamic rate is exactly 1
-// (s_e = s_eps = s_q = 1 and varsigma_3 = varsigma_4 = 1, the paper's choice).
-static bool unit_rates(const PhysD& d) {
-    return d.s_e == 1.0 && d.s_eps == 1.0 && d.s_q == 1.0 && d.vs3 == 1.0 && d.vs4 == 1.0;
 }
 
 template <int PREC, int NT, bool STG>
