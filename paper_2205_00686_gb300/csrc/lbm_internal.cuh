@@ -34,7 +34,7 @@ struct Ctl {
     // step counter and density ring stay as they are
     long long target;
     int err;
-    int pad;
+    int done;          // CTAs that have finished (three-dimensional marching step)
 };
 
 __device__ __forceinline__ bool ctl_stopped(const Ctl* c) {
@@ -99,9 +99,9 @@ struct Phys {
     R sig_e, sig_eps;                // sigma / (1/s - 1/2)
     // unit rates: the collision's combined factors (collide9_unit)
     R u_m, u_d, u_g7, u_g8;          // (1 - s_p)/4, s_p/4, hs_p/2, hs_p/4
-    R u_ax, u_dg, u_0;               // the sigma terms' factors of |12 s|^2
+    R u_ax, u_dg;                    // the sigma terms' factors of |12 s|^2
     // D2Q5
-    R cv, inv_cv, w_dot, w5_0, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
+    R cv, inv_cv, w_dot, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
     R h_m, one_m_vs4;               // h_m = (1 - vs1) / 2
     R gravity;
     int frozen_flow, frozen_thermal;
@@ -150,12 +150,10 @@ inline Phys<R> make_phys(const PhysD& d) {
                      sp = 0.5 * d.sigma / (1.0 / d.s_eps - 0.5);
         p.u_ax = (R)(k * (2.0 * sp - se) / 36.0);
         p.u_dg = (R)(k * (2.0 * se - sp) / 36.0);
-        p.u_0 = (R)(-k * (se + sp) / 9.0);
     }
     p.cv = (R)d.cv;
     p.inv_cv = (R)(1.0 / d.cv);
     p.w_dot = (R)d.w_dot;
-    p.w5_0 = (R)(1.0 - d.w_dot);
     p.w5_1 = (R)(0.25 * d.w_dot);
     p.vs1_cs2h = (R)(d.vs1 / (0.5 * d.w_dot));
     p.vs3 = (R)d.vs3;

@@ -172,10 +172,13 @@ __device__ __forceinline__ R2 velocity(R2 F, R2 j, R ir) {
 // collision at m^eq + F/2), so f* = M^{-1} m* needs of f only rho, j and the
 // stress moments m_7, m_8 (Eqs. 5, 7, 8).  With K = rho u.u + u.F and
 // |12 s|^2 of the force stencil,
-//   f*_0          = 4/9 rho - 2/3 K + u_0 |12 s|^2
+//   f*_0          = what the others leave of rho (4/9 rho - 2/3 K + ...)
 //   axis part     = 1/9 rho + 1/12 K + u_ax |12 s|^2, +- m*_7/4, +- (j + F)/3
 //   diagonal part = 1/36 rho + 1/12 K + u_dg |12 s|^2, +- m*_8/4,
 //                   +- ((j + F)_x +- (j + F)_y)/12
+// With f*_0 as the remainder and the float 1/12 rounded down, so that 2/3 + 4/12
+// is 1, mass and momentum are kept to the rounding of the populations (each
+// weight rounded by itself adds 3e-8 of them every step in FP32).
 // rhod: deviation of rho from the storage reference (f is stored as
 // deviations); rho: the density itself.
 template <class R, class R2>
@@ -199,10 +202,11 @@ __device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rho, R rhod, R
     // (7, 6) the same minus that
     const R2 cb = pr(radd(cc.x, b7), rsub(cc.x, b7)), db = pr(radd(cc.y, b8), rsub(cc.y, b8));
     const R2 sd = pr(radd(js.x, js.y), rsub(js.x, js.y));
-    const R2 t3 = pr(R(1.0 / 3.0), R(1.0 / 3.0)), t12 = pr(R(1.0 / 12.0), R(1.0 / 12.0));
+    const R w12 = sizeof(R) == 4 ? R(0x1.555554p-4) : R(1.0 / 12.0);
+    const R2 t3 = pr(R(1.0 / 3.0), R(1.0 / 3.0)), t12 = pr(w12, w12);
     const R2 f12 = pfma(js, t3, cb), f58 = pfma(sd, t12, db);
     const R2 f34 = pnfma(js, t3, cb), f76 = pnfma(sd, t12, db);
-    f[0] = rfma(rhod, R(4.0 / 9.0), rfma(P.u_0, S, rmul(K, R(-2.0 / 3.0))));
+    f[0] = rfma(R(-4), radd(cc.x, cc.y), rhod);
     f[1 * stride] = f12.x;
     f[2 * stride] = f12.y;
     f[3 * stride] = f34.x;
@@ -292,7 +296,7 @@ __device__ __forceinline__ R thermal5(const Phys<R>& P, const R* g, R Td, R C, R
         // varsigma_3 = varsigma_4 = 1: m3* = w_dot (T + Q + S), m4* = 0
         const R TQ = rfma(C, dP, Td);
         const R a = rmul(P.w5_1, TQ);
-        gs[0] = rmul(P.w5_0, TQ);
+        gs[0] = rfma(R(-4), a, TQ);     // what the others leave of T
         const R2 g12 = padd(pr(a, a), h12), g34 = psub(pr(a, a), h12);
         gs[1] = g12.x;
         gs[2] = g12.y;
