@@ -46,9 +46,9 @@ typedef struct {
 typedef struct lbm3d_ctx lbm3d_ctx;
 
 /* Device bytes of the state of an nx x ny x nz domain at prec (LBM_FP64 or
- * LBM_FP32): two copies of f (19), g (7) and P, 15 per-node scalars (rho, T,
- * psi, T dp/dT, j, 1/(rho c_v), u, F, |F_m|^2/psi^2), plus the psi of the two
- * wall ghost layers.  0 for invalid arguments. */
+ * LBM_FP32): two copies of f (19), g (7) and P, 15 per-node scalars (the
+ * current state's rho, j, psi, T dp/dT/(rho c_v), stresses, T, u), plus two
+ * layers in reserve.  0 for invalid arguments. */
 size_t lbm3d_state_bytes(int nx, int ny, int nz, int prec);
 
 /* Creates a context; stream as in lbm_create (NULL: a library stream).
@@ -84,15 +84,14 @@ int lbm3d_get_populations(lbm3d_ctx* ctx, double* f, double* g, double* P);
 int lbm3d_diagnostics(lbm3d_ctx* ctx, double rho_l, double rho_g, int sessile, lbm_diag* out);
 
 /* Selects how a step runs; the state and its result are the same either way
- * (same arithmetic per node; sums over nodes in another order).  fused != 0
- * (the default in FP32): one kernel per step marching through the z planes
- * of 16 x 16 node tiles, zseg planes per CTA (0: chosen from the domain and
- * the device), recomputing the fields the stencils need around each tile, so
- * that f, g and P are read and written once per step.  fused == 0 (the
- * default in FP64, where the recomputation costs more than the traffic it
- * saves): kernels over the nodes (force and velocity; collisions with the
- * push of f and g; the next state's fields), which keep per-node fields in
- * device memory between them.
+ * (same arithmetic per node; sums over nodes in another order).  Both forms
+ * first compute the state's fields node by node.  fused != 0 (the default in
+ * FP32): one kernel then does the rest of the step, marching through the z
+ * planes of 32 x 8 node tiles, zseg planes per CTA (0: chosen from the domain
+ * and the device).  fused == 0 (the default in FP64): kernels over the nodes
+ * (force and velocity; collisions with the push of f and g), which keep u and F
+ * in device memory between them.  Domains with more than 113 million nodes in
+ * a plane run the latter in either case.
  * The steps of Section 3.2 (Eqs. 5, 9, 11, 20, 24, 39, 49-50) in three
  * dimensions; the paper has no counterpart of the choice.  Takes effect at
  * the next lbm3d_step.  LBM_EINVAL for a NULL context or zseg < 0. */

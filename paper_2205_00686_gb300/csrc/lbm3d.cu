@@ -3,11 +3,12 @@
 // energy moment) + D3Q7 temperature lattice with the rho c_v-weighted
 // streaming of Eq. 39, x and y periodic, z periodic or walls.
 //
-// Two forms of the step give the same result.  k3_fused (below; the default
-// in FP32) does the whole step in one kernel over z-marching tiles.  The other
-// form (the default in FP64) is three kernels over the nodes plus a
-// one-thread counter update, because every stage needs neighbours of the
-// previous one:
+// Two forms of the step give the same result.  Both start with
+//   k3_macro    rho, j, the stress moments, psi, T dp/dT of the state from
+//               f(t), g(t), and the density sum for buoyancy
+// Then k3_march (below; the default in FP32) does the rest of the step in one
+// kernel over z-marching tiles.  The other form (the default in FP64) is two
+// more kernels over the nodes plus a one-thread counter update:
 //   k3_force    psi of the 18 neighbours (ghost layer at walls) -> F_m, F,
 //               u = (j + F/2)/rho, |F_m|^2/psi^2                (Eqs. 9, 11)
 //   k3_collide  div u (neighbour u), grad T (local moments), Q, P^n, S;
@@ -15,16 +16,19 @@
 //               (bounce-back at walls); g*_i blended into the destination's
 //               g(t+1) = g + (g* - g)/(rho c_v) (anti-bounce-back at walls),
 //               P^n stored                          (Eqs. 5, 20, 24, 39)
-//   k3_macro    rho, j, T, psi, T dp/dT, 1/(rho c_v) of the new state from
-//               f(t+1), g(t+1), and the density sum for buoyancy
-// Per node and step (FP32) this moves about 1.9 times the 216 B of one read
-// and one write of the state: f is read again after the push to build the
-// next state's fields, and u, F and the per-node fields pass through memory.
 //
-// Reciprocals use f_rcp as in two dimensions (the hardware approximation in
-// FP32; Newton-Raphson from it, within about one ulp, in FP64).
-// Populations are stored as deviations f_i - w_i rho_ref and g_i - w^_i T_ref.
-// Planes are [q][nz][ny][pitch], 64-bit offsets.
+// Populations are stored as deviations f_i - w_i rho_ref and g_i - w^_i T_ref,
+// in blocks of 32 nodes along x: a block holds its 19 (or 7) populations one
+// after the other, 32 nodes each (128 bytes in FP32), so all populations of a
+// node lie at constant offsets from one address (as planes they need 64-bit
+// address arithmetic for each) and a tile row of 32 nodes is one block.
+// The other per-node fields are planes [nz][ny][pitch], 64-bit offsets.
+//
+// At unit rates (s_e = s_eps = s_q = 1 and varsigma_3 = varsigma_4 = 1, the
+// paper's setting) the collision needs of f only rho, j and the five stress
+// moments (collide19_unit): about 310 operations per node and step instead
+// of 770, which is what bounds the FP64 step, and no moment matrices (96^3
+// FP64 in the step over nodes: 1080 -> 601 us).
 #include <math.h>
 #include <string.h>
 
@@ -175,16 +179,23 @@ __host__ __device__ constexpr int hx(int i) { return i == 1 ? 1 : (i == 2 ? -1 :
 __host__ __device__ constexpr int hy(int i) { return i == 3 ? 1 : (i == 4 ? -1 : 0); }
 __host__ __device__ constexpr int hz(int i) { return i == 5 ? 1 : (i == 6 ? -1 : 0); }
 
-enum { A_RHO = 0, A_T, A_PSI, A_TDPDT, A_JX, A_JY, A_JZ, A_IC, A_N };   // aux: 1/(rho c_v) last
-enum { B_UX = 0, B_UY, B_UZ, B_FX, B_FY, B_FZ, B_FM2, B_N };            // aux2 planes
+// per-node planes: the fields of the current state (rho as its deviation from
+// rho_ref, which keeps the precision of the populations) and, for the step over
+// nodes and the read-out, T, u and F (which share planes with the stresses)
+enum { Q_RHO = 0, Q_PSI, Q_E, Q_JX, Q_JY, Q_JZ, Q_S, Q_T = Q_S + 5, Q_UX, Q_UY, Q_UZ, Q_N,
+       Q_FX = Q_S, Q_FY, Q_FZ, Q_F2, Q_IC };   // E = T dp/dT / (12 rho c_v), IC = 1/(rho c_v)
+
+// Blocks of XB nodes along x: population i of node n at fofs(n) + i XB, gofs(n)
+// + i XB (the pitch is a multiple of 32)
+constexpr int XB = 32;
+__host__ __device__ __forceinline__ size_t fofs(size_t n) { return (n / XB) * (19 * XB) + n % XB; }
+__host__ __device__ __forceinline__ size_t gofs(size_t n) { return (n / XB) * (7 * XB) + n % XB; }
 
 struct Dom3 {
     void* f[2];
     void* g[2];
     void* P[2];
     void* aux;
-    void* aux2;
-    void* ghost;      // wall ghost-layer psi [2][ny][pitch] (fused step)
     Ctl* ctl;
     int nx, ny, nz, pitch;
     size_t plane;
@@ -196,18 +207,35 @@ template <class R>
 struct Lat3 {
     R s_e, s_eps, s_q, s_p;
     R sig_e3;            // (19/2) sigma / (1/s_e - 1/2), the sigma term of e
-    R vs0, vs1, vs3, vs4, w7_0, w7_1, cs2h, cv, gravity;
+    R vs0, vs1, vs3, vs4, w7_0, w7_1, cs2h, cv, inv_cv, gravity;
+    // unit rates: 1 - s_p, 2 - s_p; the sigma term's factors of |12 s|^2 in the
+    // axis and diagonal populations; (1 - vs1)/2; vs1 / cs2h
+    R c_m, c_f, h_ax, h_dg, h_m, vs1_cs2h;
+    R rho_ref, T_ref;
+    R tw2[2];            // 2 w^_i (T_wall - T_ref) of the bottom and the top
     int frozen_flow, frozen_thermal;
 };
 
 template <class R>
-Lat3<R> make_lat3(const lbm_params& p) {
+Lat3<R> make_lat3(const lbm_params& p, const Dom3& D) {
     Lat3<R> L;
     L.s_e = (R)p.s_e;
     L.s_eps = (R)p.s_eps;
     L.s_q = (R)p.s_q;
-    L.s_p = (R)(1.0 / (3.0 * p.nu + 0.5));
+    const double s_p = 1.0 / (3.0 * p.nu + 0.5);
+    L.s_p = (R)s_p;
     L.sig_e3 = (R)(9.5 * p.sigma / (1.0 / p.s_e - 0.5));
+    L.c_m = (R)(1.0 - s_p);
+    L.c_f = (R)(2.0 - s_p);
+    {
+        // half the sigma source of e, as a factor of |12 s|^2 = 144 |F_m|^2 / (G psi)^2,
+        // times the row entries over the row's norm
+        const double h = 0.5 * 9.5 * p.sigma / (1.0 / p.s_e - 0.5) * p.G * p.G / 144.0;
+        L.h_ax = (R)(h * mrow(1, 1) / (double)mnorm(1));
+        L.h_dg = (R)(h * mrow(1, 7) / (double)mnorm(1));
+    }
+    L.rho_ref = (R)D.rho_ref;
+    L.T_ref = (R)D.T_ref;
     const double cs2h = p.w_dot / 3.0;
     L.cs2h = (R)cs2h;
     L.vs0 = (R)p.vs0;
@@ -216,7 +244,11 @@ Lat3<R> make_lat3(const lbm_params& p) {
     L.vs4 = (R)p.vs4;
     L.w7_0 = (R)(1.0 - p.w_dot);
     L.w7_1 = (R)(p.w_dot / 6.0);
+    L.h_m = (R)(0.5 * (1.0 - 1.0 / (p.lambda / cs2h + 0.5)));
+    L.vs1_cs2h = (R)(1.0 / (p.lambda / cs2h + 0.5) / cs2h);
+    for (int e = 0; e < 2; ++e) L.tw2[e] = (R)(2.0 * (p.w_dot / 6.0) * (D.T_edge[e] - D.T_ref));
     L.cv = (R)p.cv;
+    L.inv_cv = (R)(1.0 / p.cv);
     L.gravity = (R)p.gravity;
     L.frozen_flow = p.frozen_flow;
     L.frozen_thermal = p.frozen_thermal;
@@ -246,6 +278,198 @@ PhysD phys_of(const lbm_params& p) {
     d.frozen_flow = p.frozen_flow;
     d.frozen_thermal = p.frozen_thermal;
     return d;
+}
+
+// ---- node arithmetic -------------------------------------------------------
+// rho - rho_ref, j and the five stress moments (3p_xx, p_ww, p_xy, p_yz, p_xz) of
+// a node's populations, from the sums and differences of opposite directions
+template <class R>
+struct Mom3 {
+    R rhod, j[3], st[5];
+};
+
+template <bool STRESS, class R>
+__device__ __forceinline__ void moments3(const R* f, Mom3<R>& m) {
+    typedef typename Vec2<R>::T R2;
+    const R2 s12 = padd(pr(f[1], f[3]), pr(f[2], f[4])), d12 = psub(pr(f[1], f[3]), pr(f[2], f[4]));
+    const R s3 = f[5] + f[6], d3 = f[5] - f[6];
+    const R2 s45 = padd(pr(f[7], f[9]), pr(f[8], f[10])), d45 = psub(pr(f[7], f[9]), pr(f[8], f[10]));
+    const R2 s67 = padd(pr(f[11], f[13]), pr(f[12], f[14])), d67 = psub(pr(f[11], f[13]), pr(f[12], f[14]));
+    const R2 s89 = padd(pr(f[15], f[17]), pr(f[16], f[18])), d89 = psub(pr(f[15], f[17]), pr(f[16], f[18]));
+    const R xy = s45.x + s45.y, xz = s67.x + s67.y, yz = s89.x + s89.y;
+    const R yz_ax = s12.y + s3;
+    m.rhod = (f[0] + (s12.x + yz_ax)) + ((xy + xz) + yz);
+    m.j[0] = d12.x + ((d45.x + d45.y) + (d67.x + d67.y));
+    m.j[1] = d12.y + ((d45.x - d45.y) + (d89.x + d89.y));
+    m.j[2] = d3 + ((d67.x - d67.y) + (d89.x - d89.y));
+    if (STRESS) {
+        m.st[0] = R(2) * (s12.x - yz) + ((xy + xz) - yz_ax);
+        m.st[1] = (s12.y - s3) + (xy - xz);
+        m.st[2] = s45.x - s45.y;
+        m.st[3] = s89.x - s89.y;
+        m.st[4] = s67.x - s67.y;
+    }
+}
+
+// D3Q19 collision at unit rates: the moments but rho, j and the stresses leave
+// it at m^eq + F/2, so f* = M^{-1} m* closes over rho, j + F, K = rho u.u + u.F
+// and the relaxed stresses N = (1 - s_p) m + s_p m^eq + (1 - s_p/2) F:
+//   rest      rho less the others (rho/3 - K/2 + h_0 |12 s|^2)
+//   axis a    rho/18 + h_ax |12 s|^2 + stress_a +- (j + F)_a / 6
+//   diagonal  rho/36 + K/24 + h_dg |12 s|^2 + stress_ab +- N_ab/4
+//             +- ((j + F)_a +- (j + F)_b) / 12
+// (the pi moments enter the stress parts at -1/2 of their p counterparts'
+// equilibrium + F/2).  The rest population is what the others leave of rho and
+// 1/6 is rounded down, 1/12 up, so that 2/6 + 8/12 is 1: with each weight
+// rounded by itself mass and momentum grow by 3e-8 a step in FP32 (256^3 after
+// 100 steps: fields 1.4e-6 off the FP64 ones).
+template <class R>
+__device__ __forceinline__ void collide19_unit(const Lat3<R>& L, R rho, const Mom3<R>& m, const R* u,
+                                               const R* F, R S, R* f) {
+    const R rx = rho * u[0], ry = rho * u[1], rz = rho * u[2];
+    const R exx = rx * u[0], eyy = ry * u[1], ezz = rz * u[2];
+    const R fxx = u[0] * F[0], fyy = u[1] * F[1], fzz = u[2] * F[2];
+    const R eyz = eyy + ezz, fyz = fyy + fzz;
+    const R K = (exx + eyz) + (fxx + fyz);
+    // equilibrium and force of 3p_xx (half: the force row is 2 axx) and p_ww
+    const R pxx = R(2) * exx - eyz, axx = R(2) * fxx - fyz;
+    const R pww = eyy - ezz, aww = fyy - fzz;
+    const R n9 = L.c_m * m.st[0] + (L.s_p * pxx + L.c_f * axx);
+    const R n11 = L.c_m * m.st[1] + (L.s_p * pww + L.c_f * aww);
+    const R hf = R(0.5) * L.c_f;
+    const R n13 = L.c_m * m.st[2] + (L.s_p * (rx * u[1]) + hf * (u[0] * F[1] + u[1] * F[0]));
+    const R n14 = L.c_m * m.st[3] + (L.s_p * (ry * u[2]) + hf * (u[1] * F[2] + u[2] * F[1]));
+    const R n15 = L.c_m * m.st[4] + (L.s_p * (rx * u[2]) + hf * (u[0] * F[2] + u[2] * F[0]));
+    // stress parts: a = N/36 (or N/12), b = (m^eq + F/2)/72 (or /24)
+    const R b9 = (pxx + axx) * R(1.0 / 72.0), b11 = (pww + aww) * R(1.0 / 24.0);
+    const R pa = n9 * R(1.0 / 36.0) + b9, pd = n9 * R(1.0 / 36.0) - R(0.5) * b9;
+    const R qa = n11 * R(1.0 / 12.0) + b11, qd = n11 * R(1.0 / 12.0) - R(0.5) * b11;
+    const R ax = m.rhod * R(1.0 / 18.0) + L.h_ax * S;
+    const R dg = m.rhod * R(1.0 / 36.0) + (K * R(1.0 / 24.0) + L.h_dg * S);
+    const R jx = m.j[0] + F[0], jy = m.j[1] + F[1], jz = m.j[2] + F[2];
+    const R a0 = ax + R(2) * pa, a1 = (ax - pa) + qa, a2 = (ax - pa) - qa;
+    const R dxy = (dg + pd) + qd, dxz = (dg + pd) - qd, dyz = dg - R(2) * pd;
+    const R c6 = sizeof(R) == 4 ? R(0x1.555554p-3) : R(1.0 / 6.0), c12 = R(1.0 / 12.0), q = R(0.25);
+    f[0] = (m.rhod - R(6) * ax) - R(12) * dg;
+    f[1] = a0 + c6 * jx;
+    f[2] = a0 - c6 * jx;
+    f[3] = a1 + c6 * jy;
+    f[4] = a1 - c6 * jy;
+    f[5] = a2 + c6 * jz;
+    f[6] = a2 - c6 * jz;
+    const R e7 = dxy + q * n13, e9 = dxy - q * n13, e11 = dxz + q * n15, e13 = dxz - q * n15;
+    const R e15 = dyz + q * n14, e17 = dyz - q * n14;
+    const R o7 = jx + jy, o9 = jx - jy, o11 = jx + jz, o13 = jx - jz, o15 = jy + jz, o17 = jy - jz;
+    f[7] = e7 + c12 * o7;
+    f[8] = e7 - c12 * o7;
+    f[9] = e9 + c12 * o9;
+    f[10] = e9 - c12 * o9;
+    f[11] = e11 + c12 * o11;
+    f[12] = e11 - c12 * o11;
+    f[13] = e13 + c12 * o13;
+    f[14] = e13 - c12 * o13;
+    f[15] = e15 + c12 * o15;
+    f[16] = e15 - c12 * o15;
+    f[17] = e17 + c12 * o17;
+    f[18] = e17 - c12 * o17;
+}
+
+// D3Q19 collision at general rates, in moment space: f* = f + M^T dm with
+// dm = (-S (m - m^eq) + (I - S/2) Fbar) / |row|^2 (d'Humieres equilibria:
+// w_eps = 3, w_epsj = -11/2, w_xx = -1/2); Fm2 = |F_m|^2 / psi^2
+template <class R>
+__device__ __forceinline__ void collide19(const Lat3<R>& L, R rho, const R* u, const R* F, R Fm2, R (&f)[19]) {
+    R m[19];
+    moments19(f, m);
+    // deviation storage: m(abs) = m(dev) + rho_ref M w, M w = (1, -11, 3, 0 ...)
+    m[0] += L.rho_ref;
+    m[1] += R(-11) * L.rho_ref;
+    m[2] += R(3) * L.rho_ref;
+    const R ux = u[0], uy = u[1], uz = u[2], Fx = F[0], Fy = F[1], Fz = F[2];
+    const R uu = ux * ux + uy * uy + uz * uz;
+    const R uF = ux * Fx + uy * Fy + uz * Fz;
+    R meq[19], Fb[19], sk[19];
+    meq[0] = rho;                            Fb[0] = 0;                  sk[0] = 0;
+    meq[1] = rho * (R(-11) + R(19) * uu);    Fb[1] = R(38) * uF + L.sig_e3 * Fm2;  sk[1] = L.s_e;
+    meq[2] = rho * (R(3) - R(5.5) * uu);     Fb[2] = R(-11) * uF;        sk[2] = L.s_eps;
+    meq[3] = rho * ux;                       Fb[3] = Fx;                 sk[3] = 1;
+    meq[4] = R(-2.0 / 3.0) * rho * ux;       Fb[4] = R(-2.0 / 3.0) * Fx; sk[4] = L.s_q;
+    meq[5] = rho * uy;                       Fb[5] = Fy;                 sk[5] = 1;
+    meq[6] = R(-2.0 / 3.0) * rho * uy;       Fb[6] = R(-2.0 / 3.0) * Fy; sk[6] = L.s_q;
+    meq[7] = rho * uz;                       Fb[7] = Fz;                 sk[7] = 1;
+    meq[8] = R(-2.0 / 3.0) * rho * uz;       Fb[8] = R(-2.0 / 3.0) * Fz; sk[8] = L.s_q;
+    const R pxx = R(3) * ux * ux - uu, axx = R(2) * ux * Fx - uy * Fy - uz * Fz;
+    const R pww = uy * uy - uz * uz, aww = uy * Fy - uz * Fz;
+    meq[9] = rho * pxx;                      Fb[9] = R(2) * axx;         sk[9] = L.s_p;
+    meq[10] = R(-0.5) * rho * pxx;           Fb[10] = -axx;              sk[10] = L.s_q;
+    meq[11] = rho * pww;                     Fb[11] = R(2) * aww;        sk[11] = L.s_p;
+    meq[12] = R(-0.5) * rho * pww;           Fb[12] = -aww;              sk[12] = L.s_q;
+    meq[13] = rho * ux * uy;                 Fb[13] = ux * Fy + uy * Fx; sk[13] = L.s_p;
+    meq[14] = rho * uy * uz;                 Fb[14] = uy * Fz + uz * Fy; sk[14] = L.s_p;
+    meq[15] = rho * ux * uz;                 Fb[15] = ux * Fz + uz * Fx; sk[15] = L.s_p;
+    meq[16] = 0;                             Fb[16] = 0;                 sk[16] = L.s_q;
+    meq[17] = 0;                             Fb[17] = 0;                 sk[17] = L.s_q;
+    meq[18] = 0;                             Fb[18] = 0;                 sk[18] = L.s_q;
+    R dm[19];
+#pragma unroll
+    for (int kk = 0; kk < 19; ++kk)
+        dm[kk] = (-sk[kk] * (m[kk] - meq[kk]) + (R(1) - R(0.5) * sk[kk]) * Fb[kk]) * R(1.0 / mnorm(kk));
+    add_inverse19(dm, f);
+}
+
+// 12 sum_i varpi(|c_i|^2) psi(x + c_i) c_i (Eq. 9; varpi 1/6 on the axes, 1/12 on
+// the diagonals) from pn(dx, dy, dz)
+template <class R, class Get>
+__device__ __forceinline__ void stencil3(Get pn, R* s) {
+    const R axy = pn(1, 1, 0) - pn(-1, -1, 0), bxy = pn(1, -1, 0) - pn(-1, 1, 0);
+    const R axz = pn(1, 0, 1) - pn(-1, 0, -1), bxz = pn(1, 0, -1) - pn(-1, 0, 1);
+    const R ayz = pn(0, 1, 1) - pn(0, -1, -1), byz = pn(0, 1, -1) - pn(0, -1, 1);
+    s[0] = R(2) * (pn(1, 0, 0) - pn(-1, 0, 0)) + ((axy + bxy) + (axz + bxz));
+    s[1] = R(2) * (pn(0, 1, 0) - pn(0, -1, 0)) + ((axy - bxy) + (ayz + byz));
+    s[2] = R(2) * (pn(0, 0, 1) - pn(0, 0, -1)) + ((axz - bxz) + (ayz - byz));
+}
+
+// Thermal stage: P^n (Eq. 20, with E = T dp/dT / (12 rho c_v) and c_s^2 grad T =
+// -varsigma_1 times the first moments) and the D3Q7 MRT collision of the
+// (deviation) populations g with source Q + S = rho c_v (P^n + (P^n - P^{n-1})/2)
+template <bool UNIT, class R>
+__device__ __forceinline__ R thermal7(const Lat3<R>& L, const R* g, R C, R E, R ux, R uy, R uz,
+                                      R div12, R Pp, bool first, R* gs) {
+    const R m1 = g[1] - g[2], m2 = g[3] - g[4], m3 = g[5] - g[6];
+    const R s1 = g[1] + g[2], s2 = g[3] + g[4], s3 = g[5] + g[6];
+    const R Td = g[0] + ((s1 + s2) + s3);
+    const R Pn = L.vs1_cs2h * (ux * m1 + uy * m2 + uz * m3) - E * div12;
+    const R dP = first ? Pn : Pn + R(0.5) * (Pn - Pp);
+    if (UNIT) {
+        // varsigma_3 = varsigma_4 = 1: only T and the first moments remain
+        const R TQ = Td + C * dP;
+        const R a = L.w7_1 * TQ;
+        gs[0] = TQ - R(6) * a;      // what the others leave of T
+        gs[1] = a + L.h_m * m1;
+        gs[2] = a - L.h_m * m1;
+        gs[3] = a + L.h_m * m2;
+        gs[4] = a - L.h_m * m2;
+        gs[5] = a + L.h_m * m3;
+        gs[6] = a - L.h_m * m3;
+    } else {
+        // closed-form inverse of the moment matrix (rows 1, c_x, c_y, c_z,
+        // |c|^2, c_x^2 - c_y^2, c_y^2 - c_z^2)
+        const R Qs = C * dP;
+        const R m4 = (s1 + s2) + s3, m5 = s1 - s2, m6 = s2 - s3;
+        const R wd = L.w7_1 * R(6);
+        const R t4 = m4 - L.vs3 * (m4 - wd * Td) + wd * Qs;
+        const R t5 = m5 - L.vs4 * m5, t6 = m6 - L.vs4 * m6;
+        const R b = (t4 - t5 + t6) * R(1.0 / 3.0);
+        const R a = b + t5, c = b - t6;
+        gs[0] = (Td + Qs) - t4;
+        gs[1] = R(0.5) * a + L.h_m * m1;
+        gs[2] = R(0.5) * a - L.h_m * m1;
+        gs[3] = R(0.5) * b + L.h_m * m2;
+        gs[4] = R(0.5) * b - L.h_m * m2;
+        gs[5] = R(0.5) * c + L.h_m * m3;
+        gs[6] = R(0.5) * c - L.h_m * m3;
+    }
+    return Pn;
 }
 
 __device__ __forceinline__ int wrapn(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
@@ -304,81 +528,75 @@ __device__ R psi_nb(const Dom3& D, const Phys<R>& P, int x, int y, int z, int* e
     const R* A = (const R*)D.aux;
     x = wrapn(x, D.nx);
     y = wrapn(y, D.ny);
-    if (z >= 0 && z < D.nz) return A[A_PSI * D.plane + nid<R>(D, x, y, z)];
-    if (!D.walls) return A[A_PSI * D.plane + nid<R>(D, x, y, wrapn(z, D.nz))];
+    if (z >= 0 && z < D.nz) return A[Q_PSI * D.plane + nid<R>(D, x, y, z)];
+    if (!D.walls) return A[Q_PSI * D.plane + nid<R>(D, x, y, wrapn(z, D.nz))];
     const int e = z < 0 ? 0 : 1;
     const int z1 = e == 0 ? 0 : D.nz - 1, z2 = e == 0 ? 1 : D.nz - 2;
-    const R* rho = A + A_RHO * D.plane;
+    const R* rho = A + Q_RHO * D.plane;
     const R dx = rho[nid<R>(D, wrapn(x + 1, D.nx), y, z1)] - rho[nid<R>(D, wrapn(x - 1, D.nx), y, z1)];
     const R dy = rho[nid<R>(D, x, wrapn(y + 1, D.ny), z1)] - rho[nid<R>(D, x, wrapn(y - 1, D.ny), z1)];
-    const R rg = rho[nid<R>(D, x, y, z2)] + (R)D.cot * rsq(dx * dx + dy * dy);
-    const R tg = A[A_T * D.plane + nid<R>(D, x, y, z1)];   // the fluid node's temperature
+    const R rg = (rho[nid<R>(D, x, y, z2)] + (R)D.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy);
+    const R tg = A[Q_T * D.plane + nid<R>(D, x, y, z1)];   // the fluid node's temperature
     const R q2 = psi2_of(P, rg, tg);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
     return f_sqrt(q2);
 }
 
 // F_m from the psi of the 18 neighbours and F = F_m + F_b at node n
-// (Eqs. 9, 11); |F_m|^2 / psi^2 for the sigma term
+// (Eqs. 9, 11); S = 144 |F_m|^2 / (G psi)^2 for the sigma term
 template <class R>
 __device__ __forceinline__ void force_at(const Dom3& D, const Phys<R>& P, const Lat3<R>& L,
                                          int x, int y, int z, size_t n, const Nbr& nb,
-                                         long long step, int* err, R* F, R* Fm2) {
+                                         long long step, int* err, R* F, R* S) {
     const R* A = (const R*)D.aux;
-    const R* psi_p = A + A_PSI * D.plane;
-    R sx = 0, sy = 0, sz = 0;
-#pragma unroll 19
-    for (int i = 1; i < 19; ++i) {
-        const R wv = qc2(i) == 1 ? R(1.0 / 6.0) : R(1.0 / 12.0);
-        // beyond a wall the neighbour is the ghost layer (Section 3.3)
-        const R pn = nbr_solid(nb, qz(i))
-                         ? psi_nb<R>(D, P, x + qx(i), y + qy(i), z + qz(i), err)
-                         : psi_p[(size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)))];
-        if (qx(i)) sx += wv * pn * R(qx(i));
-        if (qy(i)) sy += wv * pn * R(qy(i));
-        if (qz(i)) sz += wv * pn * R(qz(i));
+    const R* psi_p = A + Q_PSI * D.plane;
+    R s[3];
+    // beyond a wall the neighbour is the ghost layer (Section 3.3)
+    stencil3<R>([&](int cx, int cy, int cz) {
+        return nbr_solid(nb, cz) ? psi_nb<R>(D, P, x + cx, y + cy, z + cz, err)
+                                 : psi_p[(size_t)((long long)n + nbr_off(nb, cx, cy, cz))];
+    }, s);
+    const R gp = P.negG_12 * psi_p[n];
+    F[0] = gp * s[0];
+    F[1] = gp * s[1];
+    F[2] = gp * s[2];
+    if (L.gravity != R(0)) {
+        const R rho_ave = (R)(__ldcg(&D.ctl->mass[(step + 2) % 3]) * D.inv_n);
+        F[2] -= L.gravity * ((A[Q_RHO * D.plane + n] + L.rho_ref) - rho_ave);
     }
-    const R psi = psi_p[n];
-    const R rho = A[A_RHO * D.plane + n];
-    const R rho_ave = L.gravity != R(0) ? (R)(__ldcg(&D.ctl->mass[(step + 2) % 3]) * D.inv_n) : R(0);
-    F[0] = P.negG * psi * sx;
-    F[1] = P.negG * psi * sy;
-    F[2] = P.negG * psi * sz - L.gravity * (rho - rho_ave);
-    *Fm2 = P.negG * P.negG * (sx * sx + sy * sy + sz * sz);
+    *S = s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
 }
 
 template <class R>
-__global__ void __launch_bounds__(128) k3_force(Dom3 D, Phys<R> P, Lat3<R> L) {
+__global__ void __launch_bounds__(128) k3_force(Dom3 D, Phys<R> P, Lat3<R> L, int want_F) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
     if (x >= D.nx || y >= D.ny) return;
-    const R* A = (const R*)D.aux;
-    R* B = (R*)D.aux2;
+    R* A = (R*)D.aux;
     const size_t n = nid<R>(D, x, y, z);
     const Nbr nb = nbr_offsets(D, x, y, z);
     int err = 0;
-    R F[3], Fm2;
-    force_at<R>(D, P, L, x, y, z, n, nb, __ldcg(&D.ctl->step), &err, F, &Fm2);
-    R ux = 0, uy = 0, uz = 0;
+    R F[3], S;
+    force_at<R>(D, P, L, x, y, z, n, nb, __ldcg(&D.ctl->step), &err, F, &S);
+    R u[3] = {0, 0, 0};
     if (!L.frozen_flow) {
-        const R ir = f_rcp(A[A_RHO * D.plane + n]);
-        ux = (A[A_JX * D.plane + n] + R(0.5) * F[0]) * ir;
-        uy = (A[A_JY * D.plane + n] + R(0.5) * F[1]) * ir;
-        uz = (A[A_JZ * D.plane + n] + R(0.5) * F[2]) * ir;
+        const R ir = f_rcp(A[Q_RHO * D.plane + n] + L.rho_ref);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[a] = (A[(Q_JX + a) * D.plane + n] + R(0.5) * F[a]) * ir;
     }
-    B[B_UX * D.plane + n] = ux;
-    B[B_UY * D.plane + n] = uy;
-    B[B_UZ * D.plane + n] = uz;
-    B[B_FX * D.plane + n] = F[0];
-    B[B_FY * D.plane + n] = F[1];
-    B[B_FZ * D.plane + n] = F[2];
-    B[B_FM2 * D.plane + n] = Fm2;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) A[(Q_UX + a) * D.plane + n] = u[a];
+    if (want_F) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) A[(Q_FX + a) * D.plane + n] = F[a];
+        A[Q_F2 * D.plane + n] = S;
+    }
     if (err) atomicOr(&D.ctl->err, err);
 }
 
 // ---------------------------------------------------------------------------
-template <class R>
+template <class R, bool UNIT>
 __global__ void __launch_bounds__(128) k3_collide(Dom3 D, Phys<R> P, Lat3<R> L) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -386,184 +604,109 @@ __global__ void __launch_bounds__(128) k3_collide(Dom3 D, Phys<R> P, Lat3<R> L) 
     if (x >= D.nx || y >= D.ny) return;
     const long long step = __ldcg(&D.ctl->step);
     const int par = (int)(step & 1);
-    const R* fc = (const R*)D.f[par];
+    const size_t n = nid<R>(D, x, y, z);
+    const R* fc = (const R*)D.f[par] + fofs(n);
     R* fn = (R*)D.f[par ^ 1];
     const R* gc = (const R*)D.g[par];
-    const R* Pc = (const R*)D.P[par];
-    R* Pn_out = (R*)D.P[par ^ 1];
     R* gn = (R*)D.g[par ^ 1];
     const R* A = (const R*)D.aux;
-    const R* B = (const R*)D.aux2;
-    const size_t n = nid<R>(D, x, y, z);
-    const R rho = A[A_RHO * D.plane + n];
-    const R TdpdT = A[A_TDPDT * D.plane + n];
-    const R ux = B[B_UX * D.plane + n], uy = B[B_UY * D.plane + n], uz = B[B_UZ * D.plane + n];
+    const R rho = A[Q_RHO * D.plane + n] + L.rho_ref;
+    const R u[3] = {A[Q_UX * D.plane + n], A[Q_UY * D.plane + n], A[Q_UZ * D.plane + n]};
+    const R F[3] = {A[Q_FX * D.plane + n], A[Q_FY * D.plane + n], A[Q_FZ * D.plane + n]};
+    const R S = A[Q_F2 * D.plane + n];
+    const size_t gno = gofs(n);
     R g[7];
-#pragma unroll 19
-    for (int i = 0; i < 7; ++i) g[i] = gc[i * D.plane + n];
-
-    const R Fx = B[B_FX * D.plane + n], Fy = B[B_FY * D.plane + n], Fz = B[B_FZ * D.plane + n];
-    const R Fm2 = B[B_FM2 * D.plane + n];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) g[i] = gc[gno + i * XB];
     const Nbr nb = nbr_offsets(D, x, y, z);
-    // div u: (1/c_s^2) sum_i w_i c_i . u(x + c_i); walls carry u = 0
-    R divu = 0;
-#pragma unroll 19
+    // 12 div u = 12 (1/c_s^2) sum_i w_i c_i . u(x + c_i); walls carry u = 0
+    R dva = 0, dvd = 0;
+#pragma unroll
     for (int i = 1; i < 19; ++i) {
         if (nbr_solid(nb, qz(i))) continue;
         const size_t m = (size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)));
-        R cu = 0;
-        if (qx(i)) cu += R(qx(i)) * B[B_UX * D.plane + m];
-        if (qy(i)) cu += R(qy(i)) * B[B_UY * D.plane + m];
-        if (qz(i)) cu += R(qz(i)) * B[B_UZ * D.plane + m];
-        divu += R(3.0 * qw(i)) * cu;
+        R& acc = qc2(i) == 1 ? dva : dvd;
+        if (qx(i)) acc += R(qx(i)) * A[Q_UX * D.plane + m];
+        if (qy(i)) acc += R(qy(i)) * A[Q_UY * D.plane + m];
+        if (qz(i)) acc += R(qz(i)) * A[Q_UZ * D.plane + m];
     }
-    // grad T from the local first moments: c^_s^2 d_a T = -vs1 m^_a
-    const R m1 = g[1] - g[2], m2 = g[3] - g[4], m3 = g[5] - g[6];
-    const R k = -L.vs1 / L.cs2h;
-    const R dTx = k * m1, dTy = k * m2, dTz = k * m3;
-    const R C = rho * L.cv;
-    const R Q = -(C * (ux * dTx + uy * dTy + uz * dTz) + TdpdT * divu);
-    const R Pn = Q * f_rcp(C);
-    const R Qs = step == 0 ? Q : Q + R(0.5) * (Q - C * Pc[n]);
+    const R C = rho * P.cv;
+    R gs[7];
+    const R Pn = thermal7<UNIT>(L, g, C, A[Q_E * D.plane + n], u[0], u[1], u[2], R(2) * dva + dvd,
+                                ((const R*)D.P[par])[n], step == 0, gs);
+    ((R*)D.P[par ^ 1])[n] = Pn;
 
-    // ---- D3Q19 MRT collision in moment space
+    // ---- D3Q19 MRT collision, pushed to x + c_i (bounce-back through walls)
     R f[19];
-#pragma unroll 19
-    for (int i = 0; i < 19; ++i) f[i] = fc[i * D.plane + n];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) f[i] = fc[i * XB];
     if (L.frozen_flow) {
-#pragma unroll 19
-        for (int i = 0; i < 19; ++i) fn[i * D.plane + n] = f[i];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) fn[fofs(n) + i * XB] = f[i];
     } else {
-        R m[19];
-        moments19(f, m);
-        // deviation storage: m(abs) = m(dev) + rho_ref M w, M w = (1, -11, 3, 0 ...)
-        const R rr = (R)D.rho_ref;
-        m[0] += rr;
-        m[1] += R(-11) * rr;
-        m[2] += R(3) * rr;
-        const R uu = ux * ux + uy * uy + uz * uz;
-        const R uF = ux * Fx + uy * Fy + uz * Fz;
-        // equilibria (d'Humieres: w_eps = 3, w_epsj = -11/2, w_xx = -1/2)
-        R meq[19], Fb[19], sk[19];
-        meq[0] = rho;                            Fb[0] = 0;                  sk[0] = 0;
-        meq[1] = rho * (R(-11) + R(19) * uu);    Fb[1] = R(38) * uF + L.sig_e3 * Fm2;  sk[1] = L.s_e;
-        meq[2] = rho * (R(3) - R(5.5) * uu);     Fb[2] = R(-11) * uF;        sk[2] = L.s_eps;
-        meq[3] = rho * ux;                       Fb[3] = Fx;                 sk[3] = 1;
-        meq[4] = R(-2.0 / 3.0) * rho * ux;       Fb[4] = R(-2.0 / 3.0) * Fx; sk[4] = L.s_q;
-        meq[5] = rho * uy;                       Fb[5] = Fy;                 sk[5] = 1;
-        meq[6] = R(-2.0 / 3.0) * rho * uy;       Fb[6] = R(-2.0 / 3.0) * Fy; sk[6] = L.s_q;
-        meq[7] = rho * uz;                       Fb[7] = Fz;                 sk[7] = 1;
-        meq[8] = R(-2.0 / 3.0) * rho * uz;       Fb[8] = R(-2.0 / 3.0) * Fz; sk[8] = L.s_q;
-        const R pxx = R(3) * ux * ux - uu, axx = R(2) * ux * Fx - uy * Fy - uz * Fz;
-        const R pww = uy * uy - uz * uz, aww = uy * Fy - uz * Fz;
-        meq[9] = rho * pxx;                      Fb[9] = R(2) * axx;         sk[9] = L.s_p;
-        meq[10] = R(-0.5) * rho * pxx;           Fb[10] = -axx;              sk[10] = L.s_q;
-        meq[11] = rho * pww;                     Fb[11] = R(2) * aww;        sk[11] = L.s_p;
-        meq[12] = R(-0.5) * rho * pww;           Fb[12] = -aww;              sk[12] = L.s_q;
-        meq[13] = rho * ux * uy;                 Fb[13] = ux * Fy + uy * Fx; sk[13] = L.s_p;
-        meq[14] = rho * uy * uz;                 Fb[14] = uy * Fz + uz * Fy; sk[14] = L.s_p;
-        meq[15] = rho * ux * uz;                 Fb[15] = ux * Fz + uz * Fx; sk[15] = L.s_p;
-        meq[16] = 0;                             Fb[16] = 0;                 sk[16] = L.s_q;
-        meq[17] = 0;                             Fb[17] = 0;                 sk[17] = L.s_q;
-        meq[18] = 0;                             Fb[18] = 0;                 sk[18] = L.s_q;
-        // dm = -S (m - m^eq) + (I - S/2) Fbar, scaled by 1/|row|^2
-        R dm[19];
-#pragma unroll 19
-        for (int kk = 0; kk < 19; ++kk)
-            dm[kk] = (-sk[kk] * (m[kk] - meq[kk]) + (R(1) - R(0.5) * sk[kk]) * Fb[kk]) *
-                     R(1.0 / mnorm(kk));
-        // f* = f + M^T dm, pushed to x + c_i (bounce-back through walls)
-        add_inverse19(dm, f);
-#pragma unroll 19
-        for (int i = 0; i < 19; ++i) {
-            const R v = f[i];
-            if (nbr_solid(nb, qz(i)))
-                fn[qopp(i) * D.plane + n] = v;
-            else
-                fn[i * D.plane + (size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)))] = v;
+        if constexpr (UNIT) {
+            Mom3<R> m;
+            moments3<true>(f, m);
+            collide19_unit(L, rho, m, u, F, S, f);
+        } else {
+            collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
         }
+        static_for<19>([&](auto icn) {
+            constexpr int i = decltype(icn)::value;
+            if (nbr_solid(nb, qz(i)))
+                fn[fofs(n) + qopp(i) * XB] = f[i];
+            else
+                fn[fofs((size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)))) + i * XB] = f[i];
+        });
     }
 
-    // ---- D3Q7 MRT collision (deviation form), closed-form inverse of the
-    // moment matrix (rows 1, c_x, c_y, c_z, |c|^2, c_x^2 - c_y^2, c_y^2 - c_z^2)
-    {
-        const R Td = g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6];
-        const R m4 = g[1] + g[2] + g[3] + g[4] + g[5] + g[6];
-        const R m5 = (g[1] + g[2]) - (g[3] + g[4]);
-        const R m6 = (g[3] + g[4]) - (g[5] + g[6]);
-        const R wd = L.w7_1 * R(6);
-        const R s0 = Td - L.vs0 * (Td - Td) + Qs;
-        const R s1 = m1 - L.vs1 * m1, s2 = m2 - L.vs1 * m2, s3 = m3 - L.vs1 * m3;
-        const R s4 = m4 - L.vs3 * (m4 - wd * Td) + wd * Qs;
-        const R s5 = m5 - L.vs4 * m5, s6 = m6 - L.vs4 * m6;
-        const R b = (s4 - s5 + s6) * R(1.0 / 3.0);
-        const R a = b + s5, c = b - s6;
-        R gs[7];
-        gs[0] = s0 - s4;
-        gs[1] = R(0.5) * (a + s1);
-        gs[2] = R(0.5) * (a - s1);
-        gs[3] = R(0.5) * (b + s2);
-        gs[4] = R(0.5) * (b - s2);
-        gs[5] = R(0.5) * (c + s3);
-        gs[6] = R(0.5) * (c - s3);
-        // weighted streaming (Eq. 39) from this node's side: g*_i lands on
-        // x = y + c_i as g_i(x) + (g*_i - g_i(x)) / (rho(x) c_v), with g_i(x)
-        // and rho(x) those of the current state; through a wall g*_i
-        // returns to this node as the opposite direction, A = 2 w^ T_w - g*_i
-        // (Dirichlet) or g*_i (adiabatic)
-        if (L.frozen_thermal) {
-#pragma unroll 7
-            for (int i = 0; i < 7; ++i) gn[i * D.plane + n] = g[i];
-        } else {
-#pragma unroll 7
-            for (int i = 0; i < 7; ++i) {
-                if ((i == 5 && nb.zhi) || (i == 6 && nb.zlo)) {
-                    const int e = i == 5 ? 1 : 0, o = i == 5 ? 6 : 5;
-                    const R Ai = D.therm[e] == T_DIRICHLET
-                                     ? R(2) * L.w7_1 * (R)(D.T_edge[e] - D.T_ref) - gs[i]
-                                     : gs[i];
-                    gn[o * D.plane + n] = g[o] + (Ai - g[o]) * A[A_IC * D.plane + n];
-                } else {
-                    const size_t m = (size_t)((long long)n + nbr_off(nb, hx(i), hy(i), hz(i)));
-                    const R go = gc[i * D.plane + m];
-                    gn[i * D.plane + m] = go + (gs[i] - go) * A[A_IC * D.plane + m];
-                }
+    // weighted streaming (Eq. 39) from this node's side: g*_i lands on
+    // x = y + c_i as g_i(x) + (g*_i - g_i(x)) / (rho(x) c_v), with g_i(x)
+    // and rho(x) those of the current state; through a wall g*_i
+    // returns to this node as the opposite direction, A = 2 w^ T_w - g*_i
+    // (Dirichlet) or g*_i (adiabatic)
+    if (L.frozen_thermal) {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) gn[gno + i * XB] = g[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+            if ((i == 5 && nb.zhi) || (i == 6 && nb.zlo)) {
+                const int e = i == 5 ? 1 : 0, o = i == 5 ? 6 : 5;
+                const R Ai = D.therm[e] == T_DIRICHLET ? L.tw2[e] - gs[i] : gs[i];
+                gn[gno + o * XB] = g[o] + (Ai - g[o]) * A[Q_IC * D.plane + n];
+            } else {
+                const size_t m = (size_t)((long long)n + nbr_off(nb, hx(i), hy(i), hz(i)));
+                const size_t gm = gofs(m) + i * XB;
+                const R go = gc[gm];
+                gn[gm] = go + (gs[i] - go) * A[Q_IC * D.plane + m];
             }
         }
     }
-    Pn_out[n] = Pn;
 }
 
 // ---------------------------------------------------------------------------
 // macroscopic fields of a node from its (deviation) populations
 template <class R>
-__device__ __forceinline__ void macro_node(const Dom3& D, const Phys<R>& P, R cv, const R* f19,
-                                           const R* g7, size_t n, int* err, R* rho_out) {
-    R* A = (R*)D.aux;
-    R rd = 0, jx = 0, jy = 0, jz = 0, Td = 0;
-#pragma unroll 19
-    for (int i = 0; i < 19; ++i) {
-        rd += f19[i];
-        if (qx(i)) jx += R(qx(i)) * f19[i];
-        if (qy(i)) jy += R(qy(i)) * f19[i];
-        if (qz(i)) jz += R(qz(i)) * f19[i];
-    }
-#pragma unroll 19
-    for (int i = 0; i < 7; ++i) Td += g7[i];
-    const R rho = rd + (R)D.rho_ref, T = Td + (R)D.T_ref;
-    R q2, TdpdT;
-    eos_node(P, rho, T, &q2, &TdpdT);
+struct Fld3 {
+    R rho, T, psi, C, ic, E;
+};
+template <class R>
+__device__ __forceinline__ void fields3(const Phys<R>& P, const Lat3<R>& L, R rhod, R Td, Fld3<R>& o,
+                                        int* err) {
+    o.rho = rhod + L.rho_ref;
+    o.T = Td + L.T_ref;
+    R q2, tdp;
+    eos_node(P, o.rho, o.T, &q2, &tdp);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
-    if (!(T == T) || !(rho == rho)) *err |= ERR_NONFINITE;
-    A[A_RHO * D.plane + n] = rho;
-    A[A_T * D.plane + n] = T;
-    A[A_PSI * D.plane + n] = f_sqrt(q2);
-    A[A_TDPDT * D.plane + n] = TdpdT;
-    A[A_IC * D.plane + n] = f_rcp(rho * cv);
-    A[A_JX * D.plane + n] = jx;
-    A[A_JY * D.plane + n] = jy;
-    A[A_JZ * D.plane + n] = jz;
-    *rho_out = rho;
+    o.psi = f_sqrt(q2);
+    o.C = o.rho * L.cv;
+    o.ic = f_rcp(o.C);
+    o.E = tdp * (o.ic * R(1.0 / 12.0));
+}
+template <class R>
+__device__ __forceinline__ R sum7(const R* g) {
+    return g[0] + (((g[1] + g[2]) + (g[3] + g[4])) + (g[5] + g[6]));
 }
 
 // block sum of rho into the density ring (FP64), for the buoyancy of the
@@ -577,11 +720,14 @@ __device__ __forceinline__ void add_mass(const Dom3& D, double v, int slot) {
     if (t == 0) massq_add(&D.ctl->massq[slot], red[0] + red[1] + red[2] + red[3], massq_scale(D.inv_n));
 }
 
-// macroscopic fields of the current state (next = 0) or of the state the
-// step in progress has just written (next = 1), with its density sum into
-// slot (step + next) % 3 for buoyancy
+// Fields of the current state from its populations, into the planes, with
+// its density sum into slot step % 3 for buoyancy.  want: W_STRESS the stress
+// moments (for k3_march at unit rates), W_IC 1/(rho c_v) (k3_collide), W_T the
+// temperature everywhere (else only next to the walls, for the ghost layer).
+// Bound by its traffic, 26 populations read and 6 to 11 fields written.
+enum { W_STRESS = 1, W_IC = 2, W_T = 4 };
 template <class R>
-__global__ void __launch_bounds__(128) k3_macro(Dom3 D, Phys<R> P, R cv, int use_mass, int next) {
+__global__ void __launch_bounds__(128) k3_macro(Dom3 D, Phys<R> P, Lat3<R> L, int use_mass, int want) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -589,95 +735,99 @@ __global__ void __launch_bounds__(128) k3_macro(Dom3 D, Phys<R> P, R cv, int use
     double msum = 0.0;
     const long long step = __ldcg(&D.ctl->step);
     if (in) {
-        const int par = (int)(step & 1) ^ next;
-        const R* fc = (const R*)D.f[par];
-        const R* gc = (const R*)D.g[par];
+        const int par = (int)(step & 1);
         const size_t n = nid<R>(D, x, y, z);
+        const R* fc = (const R*)D.f[par] + fofs(n);
+        const R* gc = (const R*)D.g[par] + gofs(n);
         R f[19], g[7];
-#pragma unroll 19
-        for (int i = 0; i < 19; ++i) f[i] = fc[i * D.plane + n];
-#pragma unroll 19
-        for (int i = 0; i < 7; ++i) g[i] = gc[i * D.plane + n];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) f[i] = __ldg(fc + i * XB);
+#pragma unroll
+        for (int i = 0; i < 7; ++i) g[i] = __ldg(gc + i * XB);
         int err = 0;
-        R rho;
-        macro_node<R>(D, P, cv, f, g, n, &err, &rho);
+        Mom3<R> m;
+        Fld3<R> o;
+        moments3<true>(f, m);
+        fields3(P, L, m.rhod, sum7(g), o, &err);
+        R* A = (R*)D.aux + n;
+        A[Q_RHO * D.plane] = m.rhod;
+        A[Q_PSI * D.plane] = o.psi;
+        A[Q_E * D.plane] = o.E;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) A[(Q_JX + a) * D.plane] = m.j[a];
+        if (want & W_STRESS) {
+#pragma unroll
+            for (int a = 0; a < 5; ++a) A[(Q_S + a) * D.plane] = m.st[a];
+        }
+        if (want & W_IC) A[Q_IC * D.plane] = o.ic;
+        if ((want & W_T) || (D.walls && (z == 0 || z == D.nz - 1))) A[Q_T * D.plane] = o.T;
         if (err) atomicOr(&D.ctl->err, err);
-        msum = (double)rho;
+        if (use_mass) msum = (double)o.rho;
     }
-    if (use_mass) add_mass(D, in ? msum : 0.0, (int)((step + next) % 3));
+    if (use_mass) add_mass(D, in ? msum : 0.0, (int)(step % 3));
 }
 
-// end of a step: publish the density sum the step's blend accumulated (the
-// new state's, slot (s + 1) % 3), clear the slot the next step's blend
+// end of a step: publish its density sum, clear the slot the next step
 // accumulates into and advance the counter
-__global__ void k3_advance(Ctl* ctl, double qscale) {
-    const long long s = ctl->step;
-    ctl->mass[(s + 1) % 3] = massq_value(ctl->massq[(s + 1) % 3], qscale);
-    ctl->massq[(s + 2) % 3] = 0;
+__device__ __forceinline__ void end_step(Ctl* ctl, long long s, double qscale) {
+    ctl->mass[s % 3] = massq_value(__ldcg(&ctl->massq[s % 3]), qscale);
+    ctl->massq[(s + 1) % 3] = 0;
     ctl->step = s + 1;
 }
+__global__ void k3_advance(Ctl* ctl, double qscale) { end_step(ctl, ctl->step, qscale); }
 
 // ---------------------------------------------------------------------------
-// Fused step: one kernel for the whole step.  A CTA takes an xy tile of
-// TX x TY nodes and a segment [z0, z1) of planes and marches k through the
-// planes, the stages skewed so that each reads only planes its predecessors
-// have finished (two barriers per plane):
-//   A(k)     rho, j, T, psi, T dp/dT, 1/(rho c_v) on the tile + 2 halo nodes
-//            from f(t), g(t) (beyond a wall: the ghost-layer psi, Section 3.3)
-//   C(k-3)   on the tile: div u, grad T, Q, P^n, S and the D3Q7 collision
-//            (Eqs. 20, 24, 49-50); g*_i blended into the destination's
-//            g(t+1) = g + (g* - g)/(rho c_v) (Eq. 39; anti-bounce-back at
-//            walls)
-//   B(k-1)   F_m, F, u on the tile + 1 (Eqs. 9, 11); on the tile the D3Q19
-//            collision (Eq. 5) with f*_i pushed to x + c_i (bounce-back at
-//            walls) and the new state's density sum
-// Shared-memory rings carry psi, rho, 1/(rho c_v), j, T dp/dT and u between
-// the stages.  Each node is collided by the CTA that owns it, which writes
-// its post-collision populations straight to their destinations in f(t+1)
-// and g(t+1); only the fields the stencils need (two halo nodes of psi, one
-// of u) are recomputed around the tile.  The step reads f, g, P once and
-// writes them once (the halo and destination reads come from L2): no u, F
-// or g* planes and no second read of f for the next state's fields.
-
-// ring slot of plane k (k >= -8)
-__device__ __forceinline__ int ring(int k, int s) { return (k + 24) % s; }
-
-#ifndef K3_TILE_X
-#define K3_TILE_X 16
-#define K3_TILE_Y 16
-#define K3_THREADS 256
-#endif
+// Marching step: after k3_macro has written the state's fields, one kernel does
+// the rest of the step.  A CTA takes an xy tile of 32 x 8 nodes and a segment
+// [z0, z1) of planes and marches k through the planes, the stages skewed so
+// that each reads only planes its predecessors have finished (two barriers per
+// plane):
+//   psi(k) into shared memory on the tile + 2 (beyond a wall: the ghost-layer
+//          psi, Section 3.3)
+//   C(k-3) on the tile: div u, grad T, Q, P^n, S and the D3Q7 collision
+//          (Eqs. 20, 24, 49-50); g*_i blended into the destination's
+//          g(t+1) = g + (g* - g)/(rho c_v) (Eq. 39; anti-bounce-back at walls)
+//   B(k-1) F_m, F, u and 1/(rho c_v) on the tile + 1 (Eqs. 9, 11); on the tile
+//          the D3Q19 collision (Eq. 5) with f*_i pushed to x + c_i
+//          (bounce-back at walls)
+// Each node is collided by the CTA that owns it, which writes its
+// post-collision populations straight to their destinations in f(t+1) and
+// g(t+1).  At unit rates f itself is not read again: rho, j and the stresses
+// are enough.  What the next iteration reads from memory is loaded into registers at the
+// start of phase 2, so that it arrives while stage B computes.
+//
+// Bound by memory latency more than by bandwidth: it moves about 190 B per
+// node (FP32), k3_macro 148.  256^3 FP32 per step: one kernel that recomputed
+// the fields around each 16 x 16 tile from f 1390 us (its halo columns cost one
+// sector per lane, L1 77 % busy), with the unit-rate collision and blocked
+// populations 1316; this form with its loads at the end of phase 2 1206, psi
+// and stage C's at the start 1123, stage B's too (two register sets) 988
+// (17.0 GLUPS; k3_macro 346 us of it, at 7 TB/s).  Three CTAs per SM spill
+// (80 registers) and take 1165.  32 x 8 tiles rather than 16 x 16: full 128-byte
+// rows, and stencil reads without bank conflicts.
 template <class R>
 struct Tile3 {
-    static constexpr int TX = K3_TILE_X, TY = K3_TILE_Y, NT = K3_THREADS;
-    static constexpr int W2 = TX + 4, N2 = W2 * (TY + 4);   // tile + 2: fields, psi
-    static constexpr int W1 = TX + 2, N1 = W1 * (TY + 2);   // tile + 1: F, u
-    static constexpr int NI = TX * TY;                       // the tile: collisions
-    static constexpr int NB = N1 - NI;                       // tile + 1 outside the tile
-    // psi 3, rho 4, 1/(rho c_v) 5, j 2 x 3, T dp/dT 4 planes of tile + 2; u 3 x 3 of tile + 1
-    static constexpr int ELEMS = 22 * N2 + 9 * N1;
+    static constexpr int TX = 32, TY = 8, NT = 256;
+    static constexpr int W2 = TX + 4, N2 = W2 * (TY + 4);   // tile + 2: psi
+    static constexpr int W1 = TX + 2, N1 = W1 * (TY + 2);   // tile + 1: u, 1/(rho c_v)
+    static constexpr int NB = N1 - TX * TY;                  // the ring around the tile
+    static constexpr int ELEMS = 3 * N2 + 12 * N1;           // psi 3 planes, u 3 x 3, 1/(rho c_v) 3
     static constexpr size_t BYTES = (size_t)ELEMS * sizeof(R);
-    // FP32: three CTAs per SM (80 registers, no spills; 11.7 against 10.1
-    // GLUPS with two at 120 registers, against 10.2 with four, which spill);
-    // FP64 needs ~240 registers
-    static constexpr int MIN_BLOCKS = (sizeof(R) == 4 && NT <= 256) ? 3 : 1;
-    static_assert(NI <= NT, "the collisions take one tile node per thread");
-    static_assert(N2 <= 2 * NT && N1 <= 2 * NT, "two passes per stage");
+    static constexpr int MIN_BLOCKS = sizeof(R) == 4 ? 2 : 1;   // CTAs per SM
+    static_assert(TX * TY == NT && N2 <= 2 * NT && NB <= NT, "one tile node per thread, psi in two passes");
 };
 
-template <class R>
+template <class R, bool UNIT>
 __global__ void __launch_bounds__(Tile3<R>::NT, Tile3<R>::MIN_BLOCKS)
-k3_fused(Dom3 D, Phys<R> P, Lat3<R> L, int zseg, int use_mass) {
+k3_march(const __grid_constant__ Dom3 D, const __grid_constant__ Phys<R> P, const __grid_constant__ Lat3<R> L,
+         int zseg) {
     using G = Tile3<R>;
-    constexpr int TX = G::TX, TY = G::TY, NT = G::NT, W2 = G::W2, N2 = G::N2, W1 = G::W1,
-                  N1 = G::N1, NI = G::NI, NB = G::NB;
+    constexpr int TX = G::TX, TY = G::TY, NT = G::NT, W2 = G::W2, N2 = G::N2, W1 = G::W1, N1 = G::N1,
+                  NB = G::NB;
     extern __shared__ __align__(16) unsigned char k3_smem[];
     R* const s_psi = reinterpret_cast<R*>(k3_smem);   // [3][N2]
-    R* const s_rho = s_psi + 3 * N2;                   // [4][N2]
-    R* const s_ic = s_rho + 4 * N2;                    // [5][N2] 1 / (rho c_v)
-    R* const s_j = s_ic + 5 * N2;                      // [2][3][N2]
-    R* const s_tdp = s_j + 6 * N2;                     // [4][N2]
-    R* const s_u = s_tdp + 4 * N2;                     // [3][3][N1]
+    R* const s_u = s_psi + 3 * N2;                     // [3][3][N1]
+    R* const s_ic = s_u + 9 * N1;                      // [3][N1] 1 / (rho c_v)
 
     const int tid = threadIdx.x;
     const int ntx = (D.nx + TX - 1) / TX;
@@ -685,185 +835,188 @@ k3_fused(Dom3 D, Phys<R> P, Lat3<R> L, int zseg, int use_mass) {
     const int z0 = (int)blockIdx.y * zseg, z1 = min(D.nz, z0 + zseg);
     const long long step = __ldcg(&D.ctl->step);
     const int par = (int)(step & 1);
-    const R* __restrict__ fc = (const R*)D.f[par];
-    R* __restrict__ fnx = (R*)D.f[par ^ 1];
-    const R* __restrict__ gc = (const R*)D.g[par];
-    R* __restrict__ gnx = (R*)D.g[par ^ 1];
-    const R* __restrict__ Pc = (const R*)D.P[par];
-    R* __restrict__ Pnx = (R*)D.P[par ^ 1];
-    const size_t PL = D.plane, ZS = (size_t)D.ny * D.pitch;
-    const R rho_ref = (R)D.rho_ref, T_ref = (R)D.T_ref;
+    const bool first = step == 0;
+    const R* __restrict__ const fc = (const R*)D.f[par];
+    R* __restrict__ const fnx = (R*)D.f[par ^ 1];
+    const R* __restrict__ const gc = (const R*)D.g[par];
+    R* __restrict__ const gnx = (R*)D.g[par ^ 1];
+    const R* __restrict__ const Pc = (const R*)D.P[par];
+    R* __restrict__ const Pnx = (R*)D.P[par ^ 1];
+    const R* __restrict__ const A = (const R*)D.aux;
+    const size_t ZS = (size_t)D.ny * D.pitch, PL = D.plane;
     const R rho_ave = L.gravity != R(0) ? (R)(__ldcg(&D.ctl->mass[(step + 2) % 3]) * D.inv_n) : R(0);
 
-    // in-plane offsets of the nodes this thread takes in stage A (the tile's
-    // local coordinates wrap periodically onto the domain)
-    int oA[2];
+    // in-plane element offsets (32 bits: the host keeps larger planes on the
+    // step over nodes), each the sum of a column and a row part
+    auto fX = [&](int x) { return (unsigned)(x / XB) * (19u * XB) + (unsigned)(x % XB); };
+    auto gX = [&](int x) { return (unsigned)(x / XB) * (7u * XB) + (unsigned)(x % XB); };
+    const unsigned fP = 19u * (unsigned)D.pitch, gP = 7u * (unsigned)D.pitch;
+    // the tile node this thread takes, its wrapped neighbour columns and rows
+    // (a tile that reaches beyond the domain wraps onto it, as its halo does)
+    const int cx = tid % TX, cy = tid / TX;
+    const int gx = wrapm(x0 + cx, D.nx), gy = wrapm(y0 + cy, D.ny);
+    const bool own = x0 + cx < D.nx && y0 + cy < D.ny;
+    const int xm = gx == 0 ? D.nx - 1 : gx - 1, xp = gx == D.nx - 1 ? 0 : gx + 1;
+    const int ym = gy == 0 ? D.ny - 1 : gy - 1, yp = gy == D.ny - 1 ? 0 : gy + 1;
+    const unsigned fx0 = fX(gx), fxm = fX(xm), fxp = fX(xp);
+    const unsigned fy0 = gy * fP, fym = ym * fP, fyp = yp * fP;
+    const unsigned gx0 = gX(gx), gxm = gX(xm), gxp = gX(xp);
+    const unsigned gy0 = gy * gP, gym = ym * gP, gyp = yp * gP;
+    const unsigned oN = (unsigned)gy * D.pitch + gx;
+    const int c2 = (cy + 2) * W2 + cx + 2, c1 = (cy + 1) * W1 + cx + 1;
+    // its node of the ring around the tile (tid < NB) and its nodes of tile + 2
+    int rx = 0, ry = 0;
+    if (tid < W1) { rx = tid - 1; ry = -1; }
+    else if (tid < 2 * W1) { rx = tid - W1 - 1; ry = TY; }
+    else if (tid < 2 * W1 + TY) { rx = -1; ry = tid - 2 * W1; }
+    else if (tid < NB) { rx = TX; ry = tid - 2 * W1 - TY; }
+    const int r2 = (ry + 2) * W2 + rx + 2, r1 = (ry + 1) * W1 + rx + 1;
+    const unsigned rN = (unsigned)wrapm(y0 + ry, D.ny) * D.pitch + wrapm(x0 + rx, D.nx);
+    unsigned pN[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const int a = tid + r * NT;
-        const int ax = a < N2 ? a % W2 - 2 : 0, ay = a < N2 ? a / W2 - 2 : 0;
-        oA[r] = wrapm(y0 + ay, D.ny) * D.pitch + wrapm(x0 + ax, D.nx);
+        pN[r] = a < N2 ? (unsigned)wrapm(y0 + a / W2 - 2, D.ny) * D.pitch + wrapm(x0 + a % W2 - 2, D.nx) : 0u;
     }
-    // this thread's node on the ring of tile + 1 around the tile (tid < NB),
-    // where stage B computes F and u only
-    int rx = 0, ry = 0;
-    if (tid < NB) {
-        if (tid < W1) { rx = tid - 1; ry = -1; }
-        else if (tid < 2 * W1) { rx = tid - W1 - 1; ry = TY; }
-        else if (tid < 2 * W1 + TY) { rx = -1; ry = tid - 2 * W1; }
-        else { rx = TX; ry = tid - 2 * W1 - TY; }
-    }
-    // the tile node this thread takes in stages B (F, u and the collision)
-    // and C; its wrapped neighbour offsets for the pushes
-    const int cx = tid % TX, cy = tid / TX;
-    const int gxo = x0 + cx, gyo = y0 + cy;
-    const bool own_xy = tid < NI && gxo < D.nx && gyo < D.ny;
-    const int oC = own_xy ? gyo * D.pitch + gxo : 0;
-    const long long oxp = own_xy && gxo == D.nx - 1 ? -(long long)(D.nx - 1) : 1;
-    const long long oxm = own_xy && gxo == 0 ? (long long)(D.nx - 1) : -1;
-    const long long oyp = own_xy && gyo == D.ny - 1 ? -(long long)(D.ny - 1) * D.pitch : D.pitch;
-    const long long oym = own_xy && gyo == 0 ? (long long)(D.ny - 1) * D.pitch : -(long long)D.pitch;
-    auto inplane = [&](int qxv, int qyv) {
-        return (qxv > 0 ? oxp : (qxv < 0 ? oxm : 0)) + (qyv > 0 ? oyp : (qyv < 0 ? oym : 0));
-    };
-    int err = 0;
-    double msum = 0.0;
-    int kzA = wrapm(z0 - 2, D.nz);   // the plane of A(k), wrapped; advanced with k
 
-    for (int k = z0 - 2; k <= z1 + 2; ++k, kzA = kzA + 1 == D.nz ? 0 : kzA + 1) {
-        // ================= phase 1: A(k), C(k - 3)
+    int err = 0;
+    // psi of the ghost layer beyond a wall at in-plane node n (Section 3.3): rho_ghost =
+    // rho(layer 2) + tan(pi/2 - theta) |tangential difference of rho at layer 1|,
+    // at the temperature of layer 1
+    auto ghost = [&](unsigned n, bool lo) -> R {
+        const int x = (int)(n % (unsigned)D.pitch), y = (int)(n / (unsigned)D.pitch);
+        const size_t za = lo ? 0 : (size_t)(D.nz - 1) * ZS, zb = lo ? ZS : (size_t)(D.nz - 2) * ZS;
+        const R* const rho = A + Q_RHO * PL;
+        const size_t row = za + n - x;
+        const R dx = rho[row + (x == D.nx - 1 ? 0 : x + 1)] - rho[row + (x == 0 ? D.nx - 1 : x - 1)];
+        const R dy = rho[za + (size_t)(y == D.ny - 1 ? 0 : y + 1) * D.pitch + x] -
+                     rho[za + (size_t)(y == 0 ? D.ny - 1 : y - 1) * D.pitch + x];
+        R q2, tdp;
+        eos_node(P, (rho[zb + n] + L.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy), A[Q_T * PL + za + n], &q2, &tdp);
+        if (!(q2 >= R(0))) err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
+        return f_sqrt(q2);
+    };
+
+    // ---- loads ahead: psi of plane k, what B needs of plane p, C of plane q
+    R a_psi[2], b_o[9], b_r[4], c_g[7], c_t[6], c_P, c_rho, c_E;
+    auto beyond = [&](int z) { return D.walls && (z < 0 || z >= D.nz); };
+    auto load_psi = [&](int k, size_t zk) {
+        if (k > z1 + 1) return;
+        if (!beyond(k)) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (r == 0 || tid + NT < N2) a_psi[r] = __ldg(A + Q_PSI * PL + zk + pN[r]);
+        } else if (k == -1 || k == D.nz) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (r == 0 || tid + NT < N2) a_psi[r] = ghost(pN[r], k < 0);
+        }
+    };
+    auto b_active = [&](int p) { return p >= z0 - 1 && p <= z1 && !beyond(p); };
+    auto load_b = [&](int p, size_t zp, R* b_o, R* b_r) {
+        if (!b_active(p)) return;
+        const R* const a = A + zp + oN;
+        b_o[0] = __ldg(a + Q_RHO * PL);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) b_o[1 + i] = __ldg(a + (Q_JX + i) * PL);
+        if (UNIT && p >= z0 && p < z1) {
+#pragma unroll
+            for (int i = 0; i < 5; ++i) b_o[4 + i] = __ldg(a + (Q_S + i) * PL);
+        }
+        if (tid < NB) {
+            const R* const b = A + zp + rN;
+            b_r[0] = __ldg(b + Q_RHO * PL);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) b_r[1 + i] = __ldg(b + (Q_JX + i) * PL);
+        }
+    };
+    auto load_c = [&](int q) {
+        if (!(q >= z0 && q < z1 && own)) return;
+        const size_t zq = (size_t)q * ZS;
+        const size_t zp = q == D.nz - 1 ? 0 : zq + ZS, zm = q == 0 ? (size_t)(D.nz - 1) * ZS : zq - ZS;
+        const R* const g = gc + zq * 7;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) c_g[i] = __ldg(g + (gy0 + gx0) + i * XB);
+        // g_i of the nodes the blend goes to
+        c_t[0] = __ldg(g + (gy0 + gxp) + 1 * XB);
+        c_t[1] = __ldg(g + (gy0 + gxm) + 2 * XB);
+        c_t[2] = __ldg(g + (gyp + gx0) + 3 * XB);
+        c_t[3] = __ldg(g + (gym + gx0) + 4 * XB);
+        c_t[4] = __ldg(gc + zp * 7 + (gy0 + gx0) + 5 * XB);
+        c_t[5] = __ldg(gc + zm * 7 + (gy0 + gx0) + 6 * XB);
+        c_P = __ldg(Pc + zq + oN);
+        c_rho = __ldg(A + Q_RHO * PL + zq + oN);
+        c_E = __ldg(A + Q_E * PL + zq + oN);
+    };
+
+    int zk = wrapm(z0 - 2, D.nz);    // plane k, wrapped
+    int k3 = 0;                      // ring slot of plane k
+    load_psi(z0 - 2, (size_t)zk * ZS);
+    for (int k = z0 - 2; k <= z1 + 2; ++k) {
+        const int km = k3 == 0 ? 2 : k3 - 1, kp = k3 == 2 ? 0 : k3 + 1;   // slots of k - 1, k - 2 (= k + 1)
+        // ================= phase 1: psi(k), C(k - 3)
         if (k <= z1 + 1) {
-            R* const psA = s_psi + ring(k, 3) * N2;
-            if (D.walls && (k < 0 || k >= D.nz)) {
-                if (k == -1 || k == D.nz) {
-                    const R* gp = (const R*)D.ghost + (k < 0 ? (size_t)0 : ZS);
-#pragma unroll
-                    for (int r = 0; r < 2; ++r)
-                        if (tid + r * NT < N2) psA[tid + r * NT] = gp[oA[r]];
-                }
-            } else {
-                const size_t zo = (size_t)kzA * ZS;
-                R* const rA = s_rho + ring(k, 4) * N2;
-                R* const iA = s_ic + ring(k, 5) * N2;
-                R* const jA = s_j + ring(k, 2) * 3 * N2;
-                R* const tA = s_tdp + ring(k, 4) * N2;
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const int a = tid + r * NT;
-                    if (a < N2) {
-                        const size_t n = zo + oA[r];
-                        R f[19], g[7];
-#pragma unroll
-                        for (int i = 0; i < 19; ++i) f[i] = __ldg(fc + i * PL + n);
-#pragma unroll
-                        for (int i = 0; i < 7; ++i) g[i] = __ldg(gc + i * PL + n);
-                        R rd = 0, jx = 0, jy = 0, jz = 0, Td = 0;
-#pragma unroll
-                        for (int i = 0; i < 19; ++i) {
-                            rd += f[i];
-                            if (qx(i)) jx += R(qx(i)) * f[i];
-                            if (qy(i)) jy += R(qy(i)) * f[i];
-                            if (qz(i)) jz += R(qz(i)) * f[i];
-                        }
-#pragma unroll
-                        for (int i = 0; i < 7; ++i) Td += g[i];
-                        const R rho = rd + rho_ref, T = Td + T_ref;
-                        R q2, tdp;
-                        eos_node(P, rho, T, &q2, &tdp);
-                        if (!(q2 >= R(0))) err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
-                        if (!(T == T) || !(rho == rho)) err |= ERR_NONFINITE;
-                        psA[a] = f_sqrt(q2);
-                        rA[a] = rho;
-                        iA[a] = f_rcp(rho * L.cv);
-                        jA[a] = jx;
-                        jA[N2 + a] = jy;
-                        jA[2 * N2 + a] = jz;
-                        tA[a] = tdp;
-                    }
-                }
-            }
+            R* const ps = s_psi + k3 * N2 + tid;
+            ps[0] = a_psi[0];
+            if (tid + NT < N2) ps[NT] = a_psi[1];
         }
         {
             const int q = k - 3;
-            if (q >= z0 && q < z1 && own_xy) {
-                const size_t n = (size_t)q * ZS + oC;
+            if (q >= z0 && q < z1 && own) {
+                const size_t zq = (size_t)q * ZS;
                 const bool lo_wall = D.walls && q == 0, hi_wall = D.walls && q == D.nz - 1;
-                const R* const um = s_u + ring(q - 1, 3) * 3 * N1;
-                const R* const u0 = s_u + ring(q, 3) * 3 * N1;
-                const R* const up = s_u + ring(q + 1, 3) * 3 * N1;
-                const int c1 = (cy + 1) * W1 + cx + 1, c2 = (cy + 2) * W2 + cx + 2;
-                // div u: (1/c_s^2) sum_i w_i c_i . u(x + c_i); walls carry u = 0
-                // (3 w_i = 1/6 on the axes, 1/12 on the diagonals, summed apart)
+                const size_t zp = q == D.nz - 1 ? 0 : zq + ZS, zm = q == 0 ? (size_t)(D.nz - 1) * ZS : zq - ZS;
+                // planes q - 1, q, q + 1 = k - 4, k - 3, k - 2
+                const R* const um = s_u + km * 3 * N1 + c1;
+                const R* const u0 = s_u + k3 * 3 * N1 + c1;
+                const R* const up = s_u + kp * 3 * N1 + c1;
+                // 12 div u = 12 (1/c_s^2) sum_i w_i c_i . u(x + c_i); walls carry u = 0
                 R dva = 0, dvd = 0;
+                auto div_plane = [&](const R* u, int dz) {
 #pragma unroll
-                for (int i = 1; i < 19; ++i) {
-                    if ((qz(i) < 0 && lo_wall) || (qz(i) > 0 && hi_wall)) continue;
-                    const R* us = (qz(i) < 0 ? um : (qz(i) > 0 ? up : u0)) + c1 + qy(i) * W1 + qx(i);
-                    R& acc = qc2(i) == 1 ? dva : dvd;
-                    if (qx(i)) acc += R(qx(i)) * us[0];
-                    if (qy(i)) acc += R(qy(i)) * us[N1];
-                    if (qz(i)) acc += R(qz(i)) * us[2 * N1];
-                }
-                const R divu = dva * R(1.0 / 6.0) + dvd * R(1.0 / 12.0);
-                R g[7];
-#pragma unroll
-                for (int i = 0; i < 7; ++i) g[i] = gc[i * PL + n];
-                const R ux = u0[c1], uy = u0[N1 + c1], uz = u0[2 * N1 + c1];
-                const R rho = s_rho[ring(q, 4) * N2 + c2], TdpdT = s_tdp[ring(q, 4) * N2 + c2];
-                // grad T from the local first moments: c^_s^2 d_a T = -vs1 m^_a
-                const R m1 = g[1] - g[2], m2 = g[3] - g[4], m3 = g[5] - g[6];
-                const R kT = -L.vs1 / L.cs2h;
-                const R dTx = kT * m1, dTy = kT * m2, dTz = kT * m3;
-                const R C = rho * L.cv;
-                const R Q = -(C * (ux * dTx + uy * dTy + uz * dTz) + TdpdT * divu);
-                const R Pn = Q * f_rcp(C);
-                const R Qs = step == 0 ? Q : Q + R(0.5) * (Q - C * Pc[n]);
-                Pnx[n] = Pn;
-                // ---- D3Q7 MRT collision (deviation form), closed-form inverse
-                const R Td = g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6];
-                const R m4 = g[1] + g[2] + g[3] + g[4] + g[5] + g[6];
-                const R m5 = (g[1] + g[2]) - (g[3] + g[4]);
-                const R m6 = (g[3] + g[4]) - (g[5] + g[6]);
-                const R wd = L.w7_1 * R(6);
-                const R s0 = Td - L.vs0 * (Td - Td) + Qs;
-                const R s1 = m1 - L.vs1 * m1, s2 = m2 - L.vs1 * m2, s3 = m3 - L.vs1 * m3;
-                const R s4 = m4 - L.vs3 * (m4 - wd * Td) + wd * Qs;
-                const R s5 = m5 - L.vs4 * m5, s6 = m6 - L.vs4 * m6;
-                const R bq = (s4 - s5 + s6) * R(1.0 / 3.0);
-                const R aq = bq + s5, cq = bq - s6;
+                    for (int i = 1; i < 19; ++i) {
+                        if (qz(i) != dz) continue;
+                        const R* us = u + qy(i) * W1 + qx(i);
+                        R& acc = qc2(i) == 1 ? dva : dvd;
+                        if (qx(i)) acc += R(qx(i)) * us[0];
+                        if (qy(i)) acc += R(qy(i)) * us[N1];
+                        if (qz(i)) acc += R(qz(i)) * us[2 * N1];
+                    }
+                };
+                div_plane(u0, 0);
+                if (!lo_wall) div_plane(um, -1);
+                if (!hi_wall) div_plane(up, 1);
                 R gs[7];
-                gs[0] = s0 - s4;
-                gs[1] = R(0.5) * (aq + s1);
-                gs[2] = R(0.5) * (aq - s1);
-                gs[3] = R(0.5) * (bq + s2);
-                gs[4] = R(0.5) * (bq - s2);
-                gs[5] = R(0.5) * (cq + s3);
-                gs[6] = R(0.5) * (cq - s3);
+                Pnx[zq + oN] = thermal7<UNIT>(L, c_g, (c_rho + L.rho_ref) * P.cv, c_E, u0[0], u0[N1], u0[2 * N1],
+                                              R(2) * dva + dvd, c_P, first, gs);
                 // weighted streaming (Eq. 39) from this node's side: g*_i lands on
                 // x = y + c_i as g_i(x) + (g*_i - g_i(x)) / (rho(x) c_v) of the
                 // current state; through a wall it returns here as the opposite
                 // direction, A = 2 w^ T_w - g*_i (Dirichlet) or g*_i (adiabatic)
+                R* const go = gnx + zq * 7;
+                const unsigned o = gy0 + gx0;
                 if (L.frozen_thermal) {
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) gnx[i * PL + n] = g[i];
+                    for (int i = 0; i < 7; ++i) go[o + i * XB] = c_g[i];
                 } else {
-                    const long long zp = q == D.nz - 1 ? -(long long)(D.nz - 1) * (long long)ZS : (long long)ZS;
-                    const long long zm = q == 0 ? (long long)(D.nz - 1) * (long long)ZS : -(long long)ZS;
-#pragma unroll
-                    for (int i = 0; i < 7; ++i) {
-                        if ((i == 5 && hi_wall) || (i == 6 && lo_wall)) {
-                            const int e = i == 5 ? 1 : 0, o = i == 5 ? 6 : 5;
-                            const R Ai = D.therm[e] == T_DIRICHLET
-                                             ? R(2) * L.w7_1 * (R)(D.T_edge[e] - D.T_ref) - gs[i]
-                                             : gs[i];
-                            gnx[o * PL + n] = g[o] + (Ai - g[o]) * s_ic[ring(q, 5) * N2 + c2];
-                        } else {
-                            const long long off = inplane(hx(i), hy(i)) + (hz(i) > 0 ? zp : (hz(i) < 0 ? zm : 0));
-                            const size_t m = (size_t)((long long)n + off);
-                            const R go = gc[i * PL + m];
-                            const R iCm = s_ic[ring(q + hz(i), 5) * N2 + c2 + hy(i) * W2 + hx(i)];
-                            gnx[i * PL + m] = go + (gs[i] - go) * iCm;
-                        }
+                    const R* const i0 = s_ic + k3 * N1 + c1;
+                    const R ic = i0[0];
+                    go[o] = c_g[0] + (gs[0] - c_g[0]) * ic;
+                    go[(gy0 + gxp) + 1 * XB] = c_t[0] + (gs[1] - c_t[0]) * i0[1];
+                    go[(gy0 + gxm) + 2 * XB] = c_t[1] + (gs[2] - c_t[1]) * i0[-1];
+                    go[(gyp + gx0) + 3 * XB] = c_t[2] + (gs[3] - c_t[2]) * i0[W1];
+                    go[(gym + gx0) + 4 * XB] = c_t[3] + (gs[4] - c_t[3]) * i0[-W1];
+                    if (hi_wall) {
+                        const R a = D.therm[1] == T_DIRICHLET ? L.tw2[1] - gs[5] : gs[5];
+                        go[o + 6 * XB] = c_g[6] + (a - c_g[6]) * ic;
+                    } else {
+                        gnx[zp * 7 + o + 5 * XB] = c_t[4] + (gs[5] - c_t[4]) * s_ic[kp * N1 + c1];
+                    }
+                    if (lo_wall) {
+                        const R a = D.therm[0] == T_DIRICHLET ? L.tw2[0] - gs[6] : gs[6];
+                        go[o + 5 * XB] = c_g[5] + (a - c_g[5]) * ic;
+                    } else {
+                        gnx[zm * 7 + o + 6 * XB] = c_t[5] + (gs[6] - c_t[5]) * s_ic[km * N1 + c1];
                     }
                 }
             }
@@ -871,177 +1024,104 @@ k3_fused(Dom3 D, Phys<R> P, Lat3<R> L, int zseg, int use_mass) {
         __syncthreads();
 
         // ================= phase 2: B(k - 1)
+        const size_t zb = (size_t)zk * ZS;
+        zk = zk + 1 == D.nz ? 0 : zk + 1;
+        load_psi(k + 1, (size_t)zk * ZS);
+        load_c(k - 2);
+        R n_o[9], n_r[4];
+        load_b(k, zb, n_o, n_r);
         {
             const int p = k - 1;
-            if (p >= z0 - 1 && p <= z1 && !(D.walls && (p < 0 || p >= D.nz))) {
-                const bool own_z = p >= z0 && p < z1;
-                const R* const psm = s_psi + ring(p - 1, 3) * N2;
-                const R* const ps0 = s_psi + ring(p, 3) * N2;
-                const R* const psp = s_psi + ring(p + 1, 3) * N2;
-                const R* const rB = s_rho + ring(p, 4) * N2;
-                const R* const jB = s_j + ring(p, 2) * 3 * N2;
-                R* const uB = s_u + ring(p, 3) * 3 * N1;
-                // pass 0: this thread's ring node of tile + 1; pass 1: its tile node
-#pragma unroll 1
-                for (int r = 0; r < 2; ++r) {
-                    if (r == 0 ? tid >= NB : tid >= NI) continue;
-                    const int lx = r ? cx : rx, ly = r ? cy : ry;
-                    const int c2 = (ly + 2) * W2 + lx + 2;
-                    // sum_i varpi(|c_i|^2) psi(x + c_i) c_i with the axis (1/6) and
-                    // diagonal (1/12) neighbours summed apart and weighted once
-                    R ax = 0, ay = 0, az = 0, dx = 0, dy = 0, dz = 0;
+            if (b_active(p)) {
+                const R* const psm = s_psi + kp * N2;    // plane k - 2
+                const R* const ps0 = s_psi + km * N2;
+                const R* const psp = s_psi + k3 * N2;
+                R* const uB = s_u + km * 3 * N1;
+                R* const iB = s_ic + km * N1;
+                // F and u of a node of tile + 1; returns |12 s|^2 of the stencil
+                auto force = [&](int i2, int i1, R rho, const R* j, R* F, R* u) -> R {
+                    R s[3];
+                    stencil3<R>([&](int dx, int dy, int dz) {
+                        return (dz < 0 ? psm : (dz > 0 ? psp : ps0))[i2 + dy * W2 + dx];
+                    }, s);
+                    const R gpsi = P.negG_12 * ps0[i2];
 #pragma unroll
-                    for (int i = 1; i < 19; ++i) {
-                        const R* pp = qz(i) < 0 ? psm : (qz(i) > 0 ? psp : ps0);
-                        const R pn = pp[c2 + qy(i) * W2 + qx(i)];
-                        if (qc2(i) == 1) {
-                            if (qx(i)) ax += R(qx(i)) * pn;
-                            if (qy(i)) ay += R(qy(i)) * pn;
-                            if (qz(i)) az += R(qz(i)) * pn;
-                        } else {
-                            if (qx(i)) dx += R(qx(i)) * pn;
-                            if (qy(i)) dy += R(qy(i)) * pn;
-                            if (qz(i)) dz += R(qz(i)) * pn;
-                        }
+                    for (int a = 0; a < 3; ++a) F[a] = gpsi * s[a];
+                    F[2] -= L.gravity * (rho - rho_ave);
+                    const R ir = f_rcp(rho);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        u[a] = L.frozen_flow ? R(0) : (j[a] + R(0.5) * F[a]) * ir;
+                        uB[a * N1 + i1] = u[a];
                     }
-                    const R sx = ax * R(1.0 / 6.0) + dx * R(1.0 / 12.0);
-                    const R sy = ay * R(1.0 / 6.0) + dy * R(1.0 / 12.0);
-                    const R sz = az * R(1.0 / 6.0) + dz * R(1.0 / 12.0);
-                    const R psi = ps0[c2], rho = rB[c2];
-                    const R Fx = P.negG * psi * sx, Fy = P.negG * psi * sy;
-                    const R Fz = P.negG * psi * sz - L.gravity * (rho - rho_ave);
-                    R ux = 0, uy = 0, uz = 0;
-                    if (!L.frozen_flow) {
-                        const R ir = f_rcp(rho);
-                        ux = (jB[c2] + R(0.5) * Fx) * ir;
-                        uy = (jB[N2 + c2] + R(0.5) * Fy) * ir;
-                        uz = (jB[2 * N2 + c2] + R(0.5) * Fz) * ir;
-                    }
-                    const int c1 = (ly + 1) * W1 + lx + 1;
-                    uB[c1] = ux;
-                    uB[N1 + c1] = uy;
-                    uB[2 * N1 + c1] = uz;
-                    // the tile node: collide it if this CTA owns it
-                    if (r == 0 || !own_z || !own_xy) continue;
-                    const size_t n = (size_t)p * ZS + oC;
+                    iB[i1] = ir * P.inv_cv;
+                    return s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
+                };
+                R F[3], u[3];
+                if (tid < NB) force(r2, r1, b_r[0] + L.rho_ref, b_r + 1, F, u);
+                const R rho = b_o[0] + L.rho_ref;
+                const R S = force(c2, c1, rho, b_o + 1, F, u);
+                // the tile node: collide it if this CTA owns it
+                if (p >= z0 && p < z1 && own) {
+                    const size_t zc = (size_t)p * ZS;
+                    R* const b0 = fnx + zc * 19;
                     R f[19];
+                    if (!UNIT || L.frozen_flow) {
+                        const R* const fl = fc + zc * 19 + (fy0 + fx0);
 #pragma unroll
-                    for (int i = 0; i < 19; ++i) f[i] = fc[i * PL + n];
-                    if (L.frozen_flow) {
-                        R rd = 0;
-#pragma unroll
-                        for (int i = 0; i < 19; ++i) {
-                            fnx[i * PL + n] = f[i];
-                            rd += f[i];
-                        }
-                        if (use_mass) msum += (double)(rd + rho_ref);
-                        continue;
+                        for (int i = 0; i < 19; ++i) f[i] = fl[i * XB];
                     }
-                    // ---- D3Q19 MRT collision in moment space
-                    const R Fm2 = P.negG * P.negG * (sx * sx + sy * sy + sz * sz);
-                    R m[19];
-                    moments19(f, m);
-                    m[0] += rho_ref;
-                    m[1] += R(-11) * rho_ref;
-                    m[2] += R(3) * rho_ref;
-                    const R uu = ux * ux + uy * uy + uz * uz;
-                    const R uF = ux * Fx + uy * Fy + uz * Fz;
-                    R meq[19], Fb[19], sk[19];
-                    meq[0] = rho;                            Fb[0] = 0;                  sk[0] = 0;
-                    meq[1] = rho * (R(-11) + R(19) * uu);    Fb[1] = R(38) * uF + L.sig_e3 * Fm2;  sk[1] = L.s_e;
-                    meq[2] = rho * (R(3) - R(5.5) * uu);     Fb[2] = R(-11) * uF;        sk[2] = L.s_eps;
-                    meq[3] = rho * ux;                       Fb[3] = Fx;                 sk[3] = 1;
-                    meq[4] = R(-2.0 / 3.0) * rho * ux;       Fb[4] = R(-2.0 / 3.0) * Fx; sk[4] = L.s_q;
-                    meq[5] = rho * uy;                       Fb[5] = Fy;                 sk[5] = 1;
-                    meq[6] = R(-2.0 / 3.0) * rho * uy;       Fb[6] = R(-2.0 / 3.0) * Fy; sk[6] = L.s_q;
-                    meq[7] = rho * uz;                       Fb[7] = Fz;                 sk[7] = 1;
-                    meq[8] = R(-2.0 / 3.0) * rho * uz;       Fb[8] = R(-2.0 / 3.0) * Fz; sk[8] = L.s_q;
-                    const R pxx = R(3) * ux * ux - uu, axx = R(2) * ux * Fx - uy * Fy - uz * Fz;
-                    const R pww = uy * uy - uz * uz, aww = uy * Fy - uz * Fz;
-                    meq[9] = rho * pxx;                      Fb[9] = R(2) * axx;         sk[9] = L.s_p;
-                    meq[10] = R(-0.5) * rho * pxx;           Fb[10] = -axx;              sk[10] = L.s_q;
-                    meq[11] = rho * pww;                     Fb[11] = R(2) * aww;        sk[11] = L.s_p;
-                    meq[12] = R(-0.5) * rho * pww;           Fb[12] = -aww;              sk[12] = L.s_q;
-                    meq[13] = rho * ux * uy;                 Fb[13] = ux * Fy + uy * Fx; sk[13] = L.s_p;
-                    meq[14] = rho * uy * uz;                 Fb[14] = uy * Fz + uz * Fy; sk[14] = L.s_p;
-                    meq[15] = rho * ux * uz;                 Fb[15] = ux * Fz + uz * Fx; sk[15] = L.s_p;
-                    meq[16] = 0;                             Fb[16] = 0;                 sk[16] = L.s_q;
-                    meq[17] = 0;                             Fb[17] = 0;                 sk[17] = L.s_q;
-                    meq[18] = 0;                             Fb[18] = 0;                 sk[18] = L.s_q;
-                    R dm[19];
+                    if (L.frozen_flow) {
 #pragma unroll
-                    for (int kk = 0; kk < 19; ++kk)
-                        dm[kk] = (-sk[kk] * (m[kk] - meq[kk]) + (R(1) - R(0.5) * sk[kk]) * Fb[kk]) *
-                                 R(1.0 / mnorm(kk));
-                    add_inverse19(dm, f);   // f* = f + M^T dm
-                    // push to x + c_i; through a wall f*_i returns as f_opp(i)
-                    const long long zp = p == D.nz - 1 ? -(long long)(D.nz - 1) * (long long)ZS : (long long)ZS;
-                    const long long zm = p == 0 ? (long long)(D.nz - 1) * (long long)ZS : -(long long)ZS;
-                    const bool lo_wall = D.walls && p == 0, hi_wall = D.walls && p == D.nz - 1;
-                    R rd = 0;
-                    static_for<19>([&](auto icn) {
-                        constexpr int i = decltype(icn)::value;
-                        rd += f[i];
-                        if ((qz(i) < 0 && lo_wall) || (qz(i) > 0 && hi_wall)) {
-                            fnx[qopp(i) * PL + n] = f[i];
+                        for (int i = 0; i < 19; ++i) b0[(fy0 + fx0) + i * XB] = f[i];
+                    } else {
+                        if constexpr (UNIT) {
+                            Mom3<R> m;
+                            m.rhod = b_o[0];
+#pragma unroll
+                            for (int a = 0; a < 3; ++a) m.j[a] = b_o[1 + a];
+#pragma unroll
+                            for (int a = 0; a < 5; ++a) m.st[a] = b_o[4 + a];
+                            collide19_unit(L, rho, m, u, F, S, f);
                         } else {
-                            const long long off = inplane(qx(i), qy(i)) + (qz(i) > 0 ? zp : (qz(i) < 0 ? zm : 0));
-                            fnx[i * PL + (size_t)((long long)n + off)] = f[i];
+                            collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
                         }
-                    });
-                    // the new state's mass: streaming moves the f* without loss
-                    if (use_mass) msum += (double)(rd + rho_ref);
+                        // push to x + c_i; through a wall f*_i returns as f_opp(i)
+                        const bool lo_wall = D.walls && p == 0, hi_wall = D.walls && p == D.nz - 1;
+                        R* const bp = fnx + (p == D.nz - 1 ? 0 : zc + ZS) * 19;
+                        R* const bm = fnx + (p == 0 ? (size_t)(D.nz - 1) * ZS : zc - ZS) * 19;
+                        static_for<19>([&](auto icn) {
+                            constexpr int i = decltype(icn)::value;
+                            const unsigned o = (qx(i) > 0 ? fxp : (qx(i) < 0 ? fxm : fx0)) +
+                                               (qy(i) > 0 ? fyp : (qy(i) < 0 ? fym : fy0));
+                            if ((qz(i) < 0 && lo_wall) || (qz(i) > 0 && hi_wall))
+                                b0[(fy0 + fx0) + qopp(i) * XB] = f[i];
+                            else
+                                (qz(i) > 0 ? bp : (qz(i) < 0 ? bm : b0))[o + i * XB] = f[i];
+                        });
+                    }
                 }
             }
         }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) b_o[i] = n_o[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) b_r[i] = n_r[i];
         __syncthreads();
+        k3 = kp;
     }
 
-    // density sum of the new state for the buoyancy of the next step
-    if (use_mass) {
-        double* red = reinterpret_cast<double*>(k3_smem);
-        for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(0xffffffffu, msum, o);
-        if ((tid & 31) == 0) red[tid >> 5] = msum;
-        __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-            for (int w = 0; w < NT / 32; ++w) s += red[w];
-            massq_add(&D.ctl->massq[(step + 1) % 3], s, massq_scale(D.inv_n));
+    if (err) atomicOr(&D.ctl->err, err);
+    // the last CTA ends the step
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(&D.ctl->done, 1) == (int)(gridDim.x * gridDim.y) - 1) {
+            __threadfence();
+            end_step(D.ctl, step, massq_scale(D.inv_n));
+            D.ctl->done = 0;
         }
     }
-    if (err) atomicOr(&D.ctl->err, err);
-}
-
-// psi of the ghost layers beyond the two walls (Section 3.3) from the current
-// state: rho_ghost = rho(layer 2) + tan(pi/2 - theta) |tangential difference of
-// rho at layer 1|, at the temperature of layer 1
-template <class R>
-__global__ void k3_ghost(Dom3 D, Phys<R> P) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int e = blockIdx.z;
-    if (x >= D.nx || y >= D.ny) return;
-    const int par = (int)(__ldcg(&D.ctl->step) & 1);
-    const R* fc = (const R*)D.f[par];
-    const R* gc = (const R*)D.g[par];
-    const int z1 = e == 0 ? 0 : D.nz - 1, z2 = e == 0 ? 1 : D.nz - 2;
-    auto rho_at = [&](int xx, int yy, int zz) {
-        const size_t n = nid<R>(D, xx, yy, zz);
-        R rd = 0;
-#pragma unroll
-        for (int i = 0; i < 19; ++i) rd += fc[i * D.plane + n];
-        return rd + (R)D.rho_ref;
-    };
-    const R dx = rho_at(wrapn(x + 1, D.nx), y, z1) - rho_at(wrapn(x - 1, D.nx), y, z1);
-    const R dy = rho_at(x, wrapn(y + 1, D.ny), z1) - rho_at(x, wrapn(y - 1, D.ny), z1);
-    const R rg = rho_at(x, y, z2) + (R)D.cot * rsq(dx * dx + dy * dy);
-    const size_t n1 = nid<R>(D, x, y, z1);
-    R Td = 0;
-#pragma unroll
-    for (int i = 0; i < 7; ++i) Td += gc[i * D.plane + n1];
-    const R q2 = psi2_of(P, rg, Td + (R)D.T_ref);
-    if (!(q2 >= R(0))) atomicOr(&D.ctl->err, (q2 != q2) ? ERR_NONFINITE : ERR_PSI);
-    ((R*)D.ghost)[((size_t)e * D.ny + y) * D.pitch + x] = f_sqrt(q2);
 }
 
 // populations f = f^eq(rho, u), g = w^ T as deviations; P = 0
@@ -1053,19 +1133,19 @@ __global__ void k3_init(Dom3 D, Lat3<R> L, const double* rho, const double* ux,
     const int z = blockIdx.z;
     if (x >= D.nx || y >= D.ny) return;
     const size_t h = ((size_t)z * D.ny + y) * D.nx + x, n = nid<R>(D, x, y, z);
-    R* f = (R*)D.f[0];
-    R* g = (R*)D.g[0];
+    R* f = (R*)D.f[0] + fofs(n);
+    R* g = (R*)D.g[0] + gofs(n);
     const double r = rho[h], a = ux[h], b = uy[h], c = uz[h], t = T[h];
     const double uu = a * a + b * b + c * c;
 #pragma unroll 19
     for (int i = 0; i < 19; ++i) {
         const double cu = qx(i) * a + qy(i) * b + qz(i) * c;
         const double fe = qw(i) * r * (1.0 + 3.0 * cu + 4.5 * cu * cu - 1.5 * uu);
-        f[i * D.plane + n] = (R)(fe - qw(i) * D.rho_ref);
+        f[i * XB] = (R)(fe - qw(i) * D.rho_ref);
     }
     const double w0 = (double)L.w7_0, w1 = (double)L.w7_1;
 #pragma unroll 19
-    for (int i = 0; i < 7; ++i) g[i * D.plane + n] = (R)((i == 0 ? w0 : w1) * (t - D.T_ref));
+    for (int i = 0; i < 7; ++i) g[i * XB] = (R)((i == 0 ? w0 : w1) * (t - D.T_ref));
     ((R*)D.P[0])[n] = R(0);
 }
 
@@ -1080,21 +1160,21 @@ __global__ void k3_export(Dom3 D, Lat3<R> L, int what, double* out) {
     const size_t h = ((size_t)z * D.ny + y) * D.nx + x, n = nid<R>(D, x, y, z);
     const int par = (int)(__ldcg(&D.ctl->step) & 1);
     if (what == 0) {
-        const R* A = (const R*)D.aux;
-        const R* B = (const R*)D.aux2;
-        out[0 * N + h] = (double)A[A_RHO * D.plane + n];
-        out[1 * N + h] = (double)B[B_UX * D.plane + n];
-        out[2 * N + h] = (double)B[B_UY * D.plane + n];
-        out[3 * N + h] = (double)B[B_UZ * D.plane + n];
-        out[4 * N + h] = (double)A[A_T * D.plane + n];
-        const double ux = out[1 * N + h], uy = out[2 * N + h], uz = out[3 * N + h];
+        const R* A = (const R*)D.aux + n;
+        const double ux = (double)A[Q_UX * D.plane], uy = (double)A[Q_UY * D.plane],
+                     uz = (double)A[Q_UZ * D.plane];
+        out[0 * N + h] = (double)A[Q_RHO * D.plane] + D.rho_ref;
+        out[1 * N + h] = ux;
+        out[2 * N + h] = uy;
+        out[3 * N + h] = uz;
+        out[4 * N + h] = (double)A[Q_T * D.plane];
         out[5 * N + h] = sqrt(ux * ux + uy * uy + uz * uz);
     } else {
-        const R* f = (const R*)D.f[par];
-        const R* g = (const R*)D.g[par];
-        for (int i = 0; i < 19; ++i) out[i * N + h] = (double)f[i * D.plane + n] + qw(i) * D.rho_ref;
+        const R* f = (const R*)D.f[par] + fofs(n);
+        const R* g = (const R*)D.g[par] + gofs(n);
+        for (int i = 0; i < 19; ++i) out[i * N + h] = (double)f[i * XB] + qw(i) * D.rho_ref;
         for (int i = 0; i < 7; ++i)
-            out[(19 + i) * N + h] = (double)g[i * D.plane + n] +
+            out[(19 + i) * N + h] = (double)g[i * XB] +
                                     (double)(i == 0 ? L.w7_0 : L.w7_1) * D.T_ref;
         out[26 * N + h] = (double)((const R*)D.P[par])[n];
     }
@@ -1115,9 +1195,8 @@ struct lbm3d_ctx {
     Ctl* ctl = nullptr;
     Dom3 D;
     cudaGraphExec_t graph = nullptr;
-    bool fused = true;       // one fused kernel per step (else three kernels)
-    int zseg = 0;            // planes per CTA of the fused step
-    bool aux_stale = false;  // the per-node planes lag the state (fused steps)
+    bool fused = true;       // marching step (else the step over nodes)
+    int zseg = 0;            // planes per CTA of the marching step
     long long step = 0;
     bool initialized = false;
     int sticky = LBM_OK;
@@ -1135,12 +1214,16 @@ size_t pitch_for(int nx) { return ((size_t)nx + 31) / 32 * 32; }
 size_t bytes_for(int nx, int ny, int nz, int prec) {
     const size_t es = prec == LBM_FP64 ? 8 : 4;
     const size_t plane = pitch_for(nx) * ny * nz;
-    // f 2 x 19, g 2 x 7, P 2, aux 8, aux2 7, two ghost-layer planes
-    return plane * es * (38 + 14 + 2 + A_N + B_N) + 2 * pitch_for(nx) * ny * es;
+    // f 2 x 19, g 2 x 7, P 2, the per-node planes 15, two layers in reserve
+    return plane * es * (38 + 14 + 2 + Q_N) + 2 * pitch_for(nx) * ny * es;
 }
 
-// planes per CTA of the fused step: enough (tile, segment) units for about
-// three per resident CTA, segments of 16 to 48 planes
+// planes per CTA of the marching step.  A segment costs about three planes
+// beyond its own, so a domain whose tiles leave room takes the shortest segments
+// that still fit the resident CTAs in one round (64^3 FP32: 4 planes 23.4 us per
+// step, 2 planes 27.9, 8 planes 26.4; 128^3: 32 planes 136 us, 16 planes 144; 72
+// x 50 x 61 between walls: 6 planes 37 us, 4 planes 44, 16 planes 47).  Larger
+// domains take 32 planes (256^3: 988 us; 48 planes 998, 64 planes 1039).
 int auto_zseg(int nx, int ny, int nz, int prec) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1150,11 +1233,9 @@ int auto_zseg(int nx, int ny, int nz, int prec) {
     const long long tiles = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
     const long long slots = (long long)sms * (prec == LBM_FP64 ? Tile3<double>::MIN_BLOCKS
                                                               : Tile3<float>::MIN_BLOCKS);
-    const long long nseg = (3 * slots + tiles - 1) / tiles;
-    int zs = (int)((nz + nseg - 1) / nseg);
-    if (zs < 16) zs = 16;
-    if (zs > 48) zs = 48;
-    return zs > nz ? nz : zs;
+    const long long nseg = slots / tiles;
+    const long long zs = nseg >= 1 ? (nz + nseg - 1) / nseg : nz;
+    return (int)(zs <= 48 ? zs : 32);
 }
 
 int set_err3(lbm3d_ctx* c, int code, const char* msg) {
@@ -1172,37 +1253,48 @@ int cuda_err3(lbm3d_ctx* c, cudaError_t e, const char* where) {
 dim3 blk3() { return dim3(32, 4, 1); }
 dim3 grd3(const lbm3d_ctx* c) { return dim3((c->nx + 31) / 32, (c->ny + 3) / 4, c->nz); }
 
+bool unit3(const lbm3d_ctx* c) { return unit_rates(phys_of(c->params)); }
+
+// the marching kernel addresses a plane's populations with 32-bit element offsets;
+// larger planes (more than 113 million nodes) take the step over nodes
+bool march_fits(const lbm3d_ctx* c) {
+    return (unsigned long long)c->ny * c->D.pitch * 19ull < (1ull << 31);
+}
+
 template <class R>
-int launch_fused(lbm3d_ctx* c) {
+int launch_march(lbm3d_ctx* c) {
     using G = Tile3<R>;
     Phys<R> P = make_phys<R>(phys_of(c->params));
-    Lat3<R> L = make_lat3<R>(c->params);
-    if (c->D.walls)
-        k3_ghost<R><<<dim3((c->nx + 31) / 32, (c->ny + 3) / 4, 2), blk3(), 0, c->stream>>>(c->D, P);
+    Lat3<R> L = make_lat3<R>(c->params, c->D);
     const dim3 grid((unsigned)(((c->nx + G::TX - 1) / G::TX) * ((c->ny + G::TY - 1) / G::TY)),
                     (unsigned)((c->nz + c->zseg - 1) / c->zseg));
-    k3_fused<R><<<grid, G::NT, G::BYTES, c->stream>>>(c->D, P, L, c->zseg, c->params.gravity != 0.0);
-    k3_advance<<<1, 1, 0, c->stream>>>(c->ctl, massq_scale(c->D.inv_n));
+    const bool unit = unit3(c);
+    k3_macro<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, c->params.gravity != 0.0, unit ? W_STRESS : 0);
+    if (unit) k3_march<R, true><<<grid, G::NT, G::BYTES, c->stream>>>(c->D, P, L, c->zseg);
+    else k3_march<R, false><<<grid, G::NT, G::BYTES, c->stream>>>(c->D, P, L, c->zseg);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// the per-node planes (rho, T, psi, T dp/dT, j) of the current state
+// the fields of the current state that the read-out needs (rho, u, T)
 template <class R>
-void launch_macro(lbm3d_ctx* c) {
-    k3_macro<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, make_phys<R>(phys_of(c->params)),
-                                                   (R)c->params.cv, 0, 0);
+void launch_fields(lbm3d_ctx* c) {
+    const Phys<R> P = make_phys<R>(phys_of(c->params));
+    const Lat3<R> L = make_lat3<R>(c->params, c->D);
+    k3_macro<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0, W_T);
+    k3_force<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0);
+    k3_export<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, L, 0, c->host_buf);
 }
 
 template <class R>
 int launch_step(lbm3d_ctx* c) {
-    if (c->fused) return launch_fused<R>(c);
+    if (c->fused && march_fits(c)) return launch_march<R>(c);
     Phys<R> P = make_phys<R>(phys_of(c->params));
-    Lat3<R> L = make_lat3<R>(c->params);
+    Lat3<R> L = make_lat3<R>(c->params, c->D);
     const dim3 b = blk3(), g = grd3(c);
-    k3_force<R><<<g, b, 0, c->stream>>>(c->D, P, L);
-    k3_collide<R><<<g, b, 0, c->stream>>>(c->D, P, L);
-    k3_macro<R><<<g, b, 0, c->stream>>>(c->D, make_phys<R>(phys_of(c->params)), (R)c->params.cv,
-                                        c->params.gravity != 0.0, 1);
+    k3_macro<R><<<g, b, 0, c->stream>>>(c->D, P, L, c->params.gravity != 0.0, W_IC);
+    k3_force<R><<<g, b, 0, c->stream>>>(c->D, P, L, 1);
+    if (unit3(c)) k3_collide<R, true><<<g, b, 0, c->stream>>>(c->D, P, L);
+    else k3_collide<R, false><<<g, b, 0, c->stream>>>(c->D, P, L);
     k3_advance<<<1, 1, 0, c->stream>>>(c->ctl, massq_scale(c->D.inv_n));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -1237,18 +1329,8 @@ int ensure_buf(lbm3d_ctx* c) {
 int export_fields(lbm3d_ctx* c) {
     int rc = ensure_buf(c);
     if (rc) return rc;
-    const dim3 b = blk3(), g = grd3(c);
-    if (c->prec == LBM_FP64) {
-        launch_macro<double>(c);
-        k3_force<double><<<g, b, 0, c->stream>>>(c->D, make_phys<double>(phys_of(c->params)),
-                                                   make_lat3<double>(c->params));
-        k3_export<double><<<g, b, 0, c->stream>>>(c->D, make_lat3<double>(c->params), 0, c->host_buf);
-    } else {
-        launch_macro<float>(c);
-        k3_force<float><<<g, b, 0, c->stream>>>(c->D, make_phys<float>(phys_of(c->params)),
-                                                  make_lat3<float>(c->params));
-        k3_export<float><<<g, b, 0, c->stream>>>(c->D, make_lat3<float>(c->params), 0, c->host_buf);
-    }
+    if (c->prec == LBM_FP64) launch_fields<double>(c);
+    else launch_fields<float>(c);
     return cuda_err3(c, cudaGetLastError(), "field export");
 }
 
@@ -1311,9 +1393,7 @@ int lbm3d_create(int nx, int ny, int nz, const lbm_params* params, const lbm3d_b
     for (int p = 0; p < 2; ++p) { D.f[p] = m + off; off += 19 * plane * es; }
     for (int p = 0; p < 2; ++p) { D.g[p] = m + off; off += 7 * plane * es; }
     for (int p = 0; p < 2; ++p) { D.P[p] = m + off; off += plane * es; }
-    D.aux = m + off; off += A_N * plane * es;
-    D.aux2 = m + off; off += B_N * plane * es;
-    D.ghost = m + off;
+    D.aux = m + off;
     D.ctl = c->ctl;
     D.nx = nx;
     D.ny = ny;
@@ -1330,15 +1410,21 @@ int lbm3d_create(int nx, int ny, int nz, const lbm_params* params, const lbm3d_b
     D.T_ref = 0.0;
     D.inv_n = 1.0 / ((double)nx * ny * nz);
     c->zseg = auto_zseg(nx, ny, nz, prec);
-    // the fused step is the faster in FP32; in FP64 (bound by the FP64 pipe)
-    // its recomputed halos cost more than the traffic it saves
+    // the marching step is the faster in FP32 (64^3 23.4 against 25.6 us, 256^3
+    // 988 against 1429); in FP64, bound by the FP64 pipe, its one CTA per SM
+    // keeps that pipe less busy (96^3 757 against 601 us)
     c->fused = prec == LBM_FP32;
-    if (prec == LBM_FP64)
-        e = cudaFuncSetAttribute(k3_fused<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)Tile3<double>::BYTES);
-    else
-        e = cudaFuncSetAttribute(k3_fused<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)Tile3<float>::BYTES);
+    auto smem = [&](auto kernel, size_t bytes) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    if (prec == LBM_FP64) {
+        smem(k3_march<double, true>, Tile3<double>::BYTES);
+        smem(k3_march<double, false>, Tile3<double>::BYTES);
+    } else {
+        smem(k3_march<float, true>, Tile3<float>::BYTES);
+        smem(k3_march<float, false>, Tile3<float>::BYTES);
+    }
     // the pitch padding is never read, but keep it defined
     if (e == cudaSuccess) e = cudaMemset(c->mem, 0, total);
     if (e != cudaSuccess) {
@@ -1378,34 +1464,33 @@ int lbm3d_init_fields(lbm3d_ctx* c, const double* rho, const double* ux, const d
     const dim3 b = blk3(), g = grd3(c);
     const int um = c->params.gravity != 0.0;
     if (c->prec == LBM_FP64) {
-        k3_init<double><<<g, b, 0, c->stream>>>(c->D, make_lat3<double>(c->params), c->host_buf,
+        k3_init<double><<<g, b, 0, c->stream>>>(c->D, make_lat3<double>(c->params, c->D), c->host_buf,
                                                 c->host_buf + N, c->host_buf + 2 * N,
                                                 c->host_buf + 3 * N, c->host_buf + 4 * N);
         k3_macro<double><<<g, b, 0, c->stream>>>(c->D, make_phys<double>(phys_of(c->params)),
-                                                 c->params.cv, um, 0);
+                                                 make_lat3<double>(c->params, c->D), um, 0);
     } else {
-        k3_init<float><<<g, b, 0, c->stream>>>(c->D, make_lat3<float>(c->params), c->host_buf,
+        k3_init<float><<<g, b, 0, c->stream>>>(c->D, make_lat3<float>(c->params, c->D), c->host_buf,
                                                c->host_buf + N, c->host_buf + 2 * N,
                                                c->host_buf + 3 * N, c->host_buf + 4 * N);
         k3_macro<float><<<g, b, 0, c->stream>>>(c->D, make_phys<float>(phys_of(c->params)),
-                                                (float)c->params.cv, um, 0);
+                                                make_lat3<float>(c->params, c->D), um, 0);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_err3(c, e, "init kernels");
-    // the initial density sum (accumulated into massq[0]) is read by step 0
-    // from slot 2 ((0 - 1) mod 3) and by step 1 from slot 0
+    // the initial density sum (accumulated into massq[0], which step 0 adds to
+    // again) is read by step 0 from slot 2 ((0 - 1) mod 3)
     e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess && um) {
         long long q0 = 0;
         e = cudaMemcpy(&q0, &c->ctl->massq[0], sizeof(q0), cudaMemcpyDeviceToHost);
         const double m0 = massq_value(q0, massq_scale(c->D.inv_n));
-        if (e == cudaSuccess) e = cudaMemcpy(&c->ctl->mass[0], &m0, sizeof(double), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemset(&c->ctl->massq[0], 0, sizeof(q0));
         if (e == cudaSuccess) e = cudaMemcpy(&c->ctl->mass[2], &m0, sizeof(double), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) return cuda_err3(c, e, "lbm3d_init_fields");
     if (c->graph) cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;   // the launch arguments carry rho_ref / T_ref
     c->step = 0;
-    c->aux_stale = false;
     c->sticky = LBM_OK;
     c->initialized = true;
     c->err.clear();
@@ -1417,11 +1502,6 @@ int lbm3d_step(lbm3d_ctx* c, int n) {
     if (!c->initialized) return set_err3(c, LBM_ESTATE, "lbm3d_step before lbm3d_init_fields");
     if (c->sticky) return c->sticky;
     if (n == 0) return LBM_OK;
-    if (!c->fused && c->aux_stale) {   // the three-kernel step starts from these planes
-        if (c->prec == LBM_FP64) launch_macro<double>(c);
-        else launch_macro<float>(c);
-    }
-    c->aux_stale = c->fused;
     const int kLen = 32;
     int left = n;
     if (left >= kLen) {
@@ -1474,9 +1554,9 @@ int lbm3d_get_populations(lbm3d_ctx* c, double* f, double* g, double* P) {
     const size_t N = (size_t)c->nx * c->ny * c->nz;
     const dim3 b = blk3(), gr = grd3(c);
     if (c->prec == LBM_FP64)
-        k3_export<double><<<gr, b, 0, c->stream>>>(c->D, make_lat3<double>(c->params), 1, c->host_buf);
+        k3_export<double><<<gr, b, 0, c->stream>>>(c->D, make_lat3<double>(c->params, c->D), 1, c->host_buf);
     else
-        k3_export<float><<<gr, b, 0, c->stream>>>(c->D, make_lat3<float>(c->params), 1, c->host_buf);
+        k3_export<float><<<gr, b, 0, c->stream>>>(c->D, make_lat3<float>(c->params, c->D), 1, c->host_buf);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && f)
         e = cudaMemcpyAsync(f, c->host_buf, 19 * N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
