@@ -357,7 +357,7 @@ void lbm_batch_destroy(lbm_batch* b);
  * device memory as the members, for the duration of the call).  The choice
  * is kept while members attach and detach (staging drops out while some
  * member cannot take it).  Without it a batch uses the lbm_create defaults
- * with 64-row segments.  lbm_batch_get_tile reports the tile in use. */
+ * with a segment height chosen from the members' sizes.  lbm_batch_get_tile reports the tile in use. */
 int lbm_batch_autotune(lbm_batch* b, int steps_per_trial);
 int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged);
 

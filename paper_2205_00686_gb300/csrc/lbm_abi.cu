@@ -134,8 +134,13 @@ int num_sms() {
     return n;
 }
 
-void build_units(const Inst& I, int inst_index, int threads, int rows, std::vector<Unit>& out) {
+// even: as few segments as rows allow, of equal height (else the last is what is left)
+void build_units(const Inst& I, int inst_index, int threads, int rows, bool even, std::vector<Unit>& out) {
     const int W = threads - 8;
+    if (even) {
+        const int n = (I.ny + rows - 1) / rows;
+        rows = (I.ny + n - 1) / n;
+    }
     for (int y0 = 0; y0 < I.ny; y0 += rows)
         for (int x0 = 0; x0 < I.nx; x0 += W) {
             Unit u;
@@ -157,21 +162,22 @@ bool has_walls(const Inst& I) {
 // have no walls (the wall rings would leave one CTA per SM) and are wide
 // enough that 216-column strips need no more thread columns than 120-column
 // ones (a 64-wide domain fills 29 % of a 224-thread strip, 50 % of a
-// 128-thread one; on the 512-domain mix with sides 64..512, 9 % more thread
-// columns already made the staged tile 12 % slower); otherwise the
-// register-prefetch form on 128 threads (four CTAs per SM).  lbm_autotune /
-// lbm_batch_autotune replace this guess by timed trials.
+// 128-thread one); otherwise the register-prefetch form on 128 threads (four
+// CTAs per SM).  A batch, whose segment heights follow its work (batch_rows),
+// takes staging up to 15 % more thread columns: sides 64..512 need 9 % more and
+// run at 203 us per step against 209 for the register tile's best height.
+// lbm_autotune / lbm_batch_autotune replace this guess by timed trials.
 long long strip_columns(int nx, int threads) {
     return (long long)((nx + threads - 9) / (threads - 8)) * threads;
 }
-bool default_staged(const Inst* const* I, size_t n, int prec) {
+bool default_staged(const Inst* const* I, size_t n, int prec, int more_percent = 0) {
     long long c224 = 0, c128 = 0;
     for (size_t i = 0; i < n; ++i) {
         if (!stage_eligible(*I[i], prec) || has_walls(*I[i])) return false;
         c224 += strip_columns(I[i]->nx, 224) * I[i]->ny;
         c128 += strip_columns(I[i]->nx, 128) * I[i]->ny;
     }
-    return n > 0 && c224 <= c128;
+    return n > 0 && c224 * 100 <= c128 * (100 + more_percent);
 }
 int default_threads(int staged) { return staged ? 224 : 128; }
 
@@ -289,7 +295,7 @@ static void drop_graph(cudaGraphExec_t* g) {
 static int ctx_apply_tile(lbm_ctx* c, int threads, int rows, int staged) {
     staged = staged && stage_eligible(c->inst, c->prec) ? 1 : 0;
     std::vector<Unit> us;
-    build_units(c->inst, 0, threads, rows, us);
+    build_units(c->inst, 0, threads, rows, false, us);
     int ctas = 1;
     size_t smem = 0;
     if (step_occupancy(c->prec, threads, has_walls(c->inst), staged, &ctas, &smem))
@@ -1222,6 +1228,48 @@ int lbm_autotune(lbm_ctx* c, int steps) {
 // new ones allocated and filled, on the batch stream (cudaFreeAsync,
 // cudaMallocAsync, copies from a pinned staging slot), so launches already
 // queued keep their own arrays and the host does not wait for them.
+// Segment height of a batch without a tuned tile: the domains' strips are cut
+// into segments of at most R rows, even within a domain, and the CTAs take them
+// from one list, longest first, so a launch lasts about w (R + 8) iterations
+// where w rounds of resident CTAs take all segments (a segment's sweep runs 6
+// iterations beyond its rows and starts up in about 2).  For each w the smallest
+// R that fits, then the w that gives the shortest launch.  FP32 open domains,
+// us per step: 64 of sides 64-512, the former 64 rows on the register tile 222,
+// this (73 rows, staged) 203, the tuner's best fixed height 208; 20 of sides
+// 64-300 45 (19 rows), 8 of sides 64-200 30 (8 rows).
+static int batch_rows(const std::vector<const Inst*>& ip, int threads, long long slots) {
+    const int W = threads - 8;
+    long long strip_rows = 0;
+    int most = 1;
+    for (const Inst* I : ip) {
+        strip_rows += (long long)((I->nx + W - 1) / W) * I->ny;
+        most = std::max(most, I->ny);
+    }
+    auto segments = [&](int R) {
+        long long n = 0;
+        for (const Inst* I : ip) n += (long long)((I->nx + W - 1) / W) * ((I->ny + R - 1) / R);
+        return n;
+    };
+    const long long w0 = std::max<long long>(1, (strip_rows + slots * most - 1) / (slots * most));
+    long long best = 0;
+    int rows = most;
+    for (long long w = w0; w < w0 + 12; ++w) {
+        if (segments(most) > w * slots) continue;
+        int lo = std::min(8, most), hi = most;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if (segments(mid) <= w * slots) hi = mid;
+            else lo = mid + 1;
+        }
+        const long long t = w * (lo + 8);
+        if (best == 0 || t < best) {
+            best = t;
+            rows = lo;
+        }
+    }
+    return rows;
+}
+
 static int batch_rebuild(lbm_batch* b) {
     drop_graph(&b->graph);
     if (b->insts) cudaFreeAsync(b->insts, b->stream);
@@ -1250,12 +1298,16 @@ static int batch_rebuild(lbm_batch* b) {
         b->staged = b->t_staged && all ? 1 : 0;
     } else {
         // bulk-copy staging (224-thread tile) when the members as a whole take it
-        b->staged = default_staged(ip.data(), ip.size(), b->prec) ? 1 : 0;
+        b->staged = default_staged(ip.data(), ip.size(), b->prec, 15) ? 1 : 0;
         b->threads = default_threads(b->staged);
     }
-    for (size_t i = 0; i < b->members.size(); ++i) {
-        build_units(b->members[i]->inst, (int)i, b->threads, std::min(b->rows, b->members[i]->ny), us);
-    }
+    int ctas = 1;
+    size_t smem = 0;
+    step_occupancy(b->prec, b->threads, b->walls, b->staged, &ctas, &smem);
+    const long long slots = (long long)std::max(ctas, 1) * num_sms();
+    if (!b->tuned) b->rows = batch_rows(ip, b->threads, slots);
+    for (size_t i = 0; i < b->members.size(); ++i)
+        build_units(b->members[i]->inst, (int)i, b->threads, std::min(b->rows, b->members[i]->ny), true, us);
     // longest first: a unit's sweep takes (rows + 6) iterations whatever its
     // width, and the persistent CTAs take units in list order, so the tall
     // units go first and the short ones fill the tail; units of equal height
@@ -1292,10 +1344,7 @@ static int batch_rebuild(lbm_batch* b) {
     if (e == cudaSuccess) e = cudaEventRecord(b->stage_ev[slot], b->stream);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
     b->n_units = (int)us.size();
-    int ctas = 1;
-    size_t smem = 0;
-    step_occupancy(b->prec, b->threads, b->walls, b->staged, &ctas, &smem);
-    b->grid = (int)std::min<long long>((long long)b->n_units, (long long)std::max(ctas, 1) * num_sms());
+    b->grid = (int)std::min<long long>((long long)b->n_units, slots);
     return LBM_OK;
 }
 
