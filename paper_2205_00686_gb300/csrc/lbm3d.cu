@@ -537,7 +537,8 @@ __device__ R psi_nb(const Dom3& D, const Phys<R>& P, int x, int y, int z, int* e
     const R dy = rho[nid<R>(D, x, wrapn(y + 1, D.ny), z1)] - rho[nid<R>(D, x, wrapn(y - 1, D.ny), z1)];
     const R rg = (rho[nid<R>(D, x, y, z2)] + (R)D.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy);
     const R tg = A[Q_T * D.plane + nid<R>(D, x, y, z1)];   // the fluid node's temperature
-    const R q2 = psi2_of(P, rg, tg);
+    R q2, tdp;
+    eos_node(P, rg, tg, &q2, &tdp);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
     return f_sqrt(q2);
 }
@@ -1149,7 +1150,8 @@ __global__ void k3_init(Dom3 D, Lat3<R> L, const double* rho, const double* ux,
     ((R*)D.P[0])[n] = R(0);
 }
 
-// state -> host-layout doubles: fields (rho, u, T) or absolute populations
+// state -> host-layout doubles: fields (what 0: rho, u, T; 2: and |u|) or, what 1,
+// absolute populations
 template <class R>
 __global__ void k3_export(Dom3 D, Lat3<R> L, int what, double* out) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1159,16 +1161,16 @@ __global__ void k3_export(Dom3 D, Lat3<R> L, int what, double* out) {
     const size_t N = (size_t)D.nx * D.ny * D.nz;
     const size_t h = ((size_t)z * D.ny + y) * D.nx + x, n = nid<R>(D, x, y, z);
     const int par = (int)(__ldcg(&D.ctl->step) & 1);
-    if (what == 0) {
+    if (what != 1) {
         const R* A = (const R*)D.aux + n;
-        const double ux = (double)A[Q_UX * D.plane], uy = (double)A[Q_UY * D.plane],
-                     uz = (double)A[Q_UZ * D.plane];
-        out[0 * N + h] = (double)A[Q_RHO * D.plane] + D.rho_ref;
+        const double ux = widen(A[Q_UX * D.plane]), uy = widen(A[Q_UY * D.plane]),
+                     uz = widen(A[Q_UZ * D.plane]);
+        out[0 * N + h] = widen(A[Q_RHO * D.plane]) + D.rho_ref;
         out[1 * N + h] = ux;
         out[2 * N + h] = uy;
         out[3 * N + h] = uz;
-        out[4 * N + h] = (double)A[Q_T * D.plane];
-        out[5 * N + h] = sqrt(ux * ux + uy * uy + uz * uz);
+        out[4 * N + h] = widen(A[Q_T * D.plane]);
+        if (what == 2) out[5 * N + h] = sqrt(ux * ux + uy * uy + uz * uz);   // for the diagnostics
     } else {
         const R* f = (const R*)D.f[par] + fofs(n);
         const R* g = (const R*)D.g[par] + gofs(n);
@@ -1277,12 +1279,12 @@ int launch_march(lbm3d_ctx* c) {
 
 // the fields of the current state that the read-out needs (rho, u, T)
 template <class R>
-void launch_fields(lbm3d_ctx* c) {
+void launch_fields(lbm3d_ctx* c, int what) {
     const Phys<R> P = make_phys<R>(phys_of(c->params));
     const Lat3<R> L = make_lat3<R>(c->params, c->D);
     k3_macro<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0, W_T);
     k3_force<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0);
-    k3_export<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, L, 0, c->host_buf);
+    k3_export<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, L, what, c->host_buf);
 }
 
 template <class R>
@@ -1325,12 +1327,12 @@ int ensure_buf(lbm3d_ctx* c) {
     return cuda_err3(c, e, "cudaMalloc(export buffers)");
 }
 
-// current fields (rho, u, T, |u|) into host_buf[0 .. 6N)
-int export_fields(lbm3d_ctx* c) {
+// current fields (rho, u, T; what = 2: |u| too) into host_buf[0 .. 6N)
+int export_fields(lbm3d_ctx* c, int what) {
     int rc = ensure_buf(c);
     if (rc) return rc;
-    if (c->prec == LBM_FP64) launch_fields<double>(c);
-    else launch_fields<float>(c);
+    if (c->prec == LBM_FP64) launch_fields<double>(c, what);
+    else launch_fields<float>(c, what);
     return cuda_err3(c, cudaGetLastError(), "field export");
 }
 
@@ -1533,7 +1535,7 @@ int lbm3d_step(lbm3d_ctx* c, int n) {
 int lbm3d_get_fields(lbm3d_ctx* c, double* rho, double* ux, double* uy, double* uz, double* T) {
     if (!c) return LBM_EINVAL;
     if (!c->initialized) return set_err3(c, LBM_ESTATE, "no state yet");
-    int rc = export_fields(c);
+    int rc = export_fields(c, 0);
     if (rc) return rc;
     const size_t N = (size_t)c->nx * c->ny * c->nz;
     double* dst[5] = {rho, ux, uy, uz, T};
@@ -1571,7 +1573,7 @@ int lbm3d_get_populations(lbm3d_ctx* c, double* f, double* g, double* P) {
 int lbm3d_diagnostics(lbm3d_ctx* c, double rho_l, double rho_g, int sessile, lbm_diag* out) {
     if (!c || !out || !(rho_l > rho_g)) return LBM_EINVAL;
     if (!c->initialized) return set_err3(c, LBM_ESTATE, "no state yet");
-    int rc = export_fields(c);
+    int rc = export_fields(c, 2);
     if (rc) return rc;
     const size_t N = (size_t)c->nx * c->ny * c->nz;
     // the reduction takes |u| in place of u_x and zeros for u_y

@@ -228,7 +228,7 @@ struct lbm_ctx {
     bool initialized = false;
     int sticky = LBM_OK;
     std::string err;
-    double* fields = nullptr;  // 5 N doubles (rho, ux, uy, T, psi scratch), lazily allocated
+    double* fields = nullptr;  // 4 N doubles (rho, ux, uy, T), lazily allocated
     void* diag_scratch = nullptr;
     double* diag_out = nullptr;
     void* iface_scratch = nullptr;   // contact-angle partial sums + 12 results
@@ -402,7 +402,7 @@ static int ctx_check(lbm_ctx* c) {
 static int ensure_fields(lbm_ctx* c) {
     if (c->fields) return LBM_OK;
     const size_t N = (size_t)c->nx * c->ny;
-    cudaError_t e = cudaMalloc(&c->fields, 5 * N * sizeof(double));
+    cudaError_t e = cudaMalloc(&c->fields, 4 * N * sizeof(double));
     if (e != cudaSuccess) {
         c->fields = nullptr;
         return cuda_err(c, e, "cudaMalloc(fields)");
@@ -642,8 +642,8 @@ int lbm_get_rho_u_T(lbm_ctx* c, double* rho, double* ux, double* uy, double* T) 
     int rc = ensure_fields(c);
     if (rc) return rc;
     const size_t N = (size_t)c->nx * c->ny;
-    if (fields_launch(c->prec, c->inst_dev, c->inst, c->phys, c->fields, c->fields + N,
-                      c->fields + 2 * N, c->fields + 3 * N, c->fields + 4 * N, c->stream))
+    if (fields_launch(c->prec, c->inst, c->phys, c->fields, c->fields + N, c->fields + 2 * N,
+                      c->fields + 3 * N, c->stream))
         return cuda_err(c, cudaGetLastError(), "fields kernel");
     double* dst[4] = {rho, ux, uy, T};
     cudaError_t e = cudaSuccess;
@@ -661,8 +661,8 @@ int lbm_diagnostics(lbm_ctx* c, double rho_l, double rho_g, int sessile, lbm_dia
     int rc = ensure_fields(c);
     if (rc) return rc;
     const size_t N = (size_t)c->nx * c->ny;
-    if (fields_launch(c->prec, c->inst_dev, c->inst, c->phys, c->fields, c->fields + N,
-                      c->fields + 2 * N, c->fields + 3 * N, c->fields + 4 * N, c->stream))
+    if (fields_launch(c->prec, c->inst, c->phys, c->fields, c->fields + N, c->fields + 2 * N,
+                      c->fields + 3 * N, c->stream))
         return cuda_err(c, cudaGetLastError(), "fields kernel");
     if (diag_launch(c->fields, c->fields + N, c->fields + 2 * N, c->fields + 3 * N, (long long)N,
                     c->params.cv, rho_l, rho_g, c->diag_out, c->diag_scratch, c->stream))
@@ -991,8 +991,8 @@ int lbm_contact_angle(lbm_ctx* c, double rho_l, double rho_g, int skip_rows, lbm
     }
     const size_t N = (size_t)c->nx * c->ny;
     double* res = (double*)((char*)c->iface_scratch + iface_scratch_bytes());
-    if (fields_launch(c->prec, c->inst_dev, c->inst, c->phys, c->fields, c->fields + N,
-                      c->fields + 2 * N, c->fields + 3 * N, c->fields + 4 * N, c->stream) ||
+    if (fields_launch(c->prec, c->inst, c->phys, c->fields, c->fields + N, c->fields + 2 * N,
+                      c->fields + 3 * N, c->stream) ||
         iface_launch(c->fields, c->nx, c->ny, 0.5 * (rho_l + rho_g), skip_rows, res,
                      c->iface_scratch, c->stream))
         return cuda_err(c, cudaGetLastError(), "contact-angle kernels");
@@ -1060,8 +1060,8 @@ int lbm_regions(lbm_ctx* c, double threshold, int below, int* labels, lbm_region
         }
     }
     int *parent = nullptr, *roots = nullptr, *count = nullptr;
-    if (fields_launch(c->prec, c->inst_dev, c->inst, c->phys, c->fields, c->fields + N,
-                      c->fields + 2 * N, c->fields + 3 * N, c->fields + 4 * N, c->stream) ||
+    if (fields_launch(c->prec, c->inst, c->phys, c->fields, c->fields + N, c->fields + 2 * N,
+                      c->fields + 3 * N, c->stream) ||
         regions_launch(c->fields, c->nx, c->ny, c->bc.flow[LBM_EDGE_W] == LBM_PERIODIC,
                        c->bc.flow[LBM_EDGE_S] == LBM_PERIODIC, threshold, below,
                        c->region_scratch, (int)N, &parent, &roots, &count, c->stream))

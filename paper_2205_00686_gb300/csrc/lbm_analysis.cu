@@ -17,16 +17,20 @@
 // not depend on scheduling.
 //
 // Regions.  A union-find over node indices: every node in the phase starts
-// as its own root; for each pair of 4-neighbours in the phase (across the
-// seams of periodic axes) the two roots are merged by an atomicMin that
+// with the first node of its run within 32 columns as parent; runs that touch
+// (across the seams of periodic axes too) have their roots merged by an atomicMin that
 // makes the larger root point to the smaller one, so a parent index is never
 // above its node's index and every region ends with its smallest node index
 // as root.  Loops that chase parents or retry a merge strictly decrease an
 // index, so they end within n iterations; they are still capped and report
 // an error word instead of running on.  A flattening pass then writes each
 // node's root, and a statistics pass accumulates per-root area, row sums,
-// row range and edge contacts with atomics (integers only: the result is
-// exact and independent of order).
+// row range and edge contacts with atomics, one lane for all lanes of a warp
+// that share a root (integers only: the result is exact and independent of
+// order).  2048^2 with 440 bubbles: merging 254 -> 71 us, the
+// other passes 103 -> 68.
+#include <algorithm>
+
 #include "lbm_internal.cuh"
 
 namespace lbm {
@@ -101,15 +105,20 @@ __global__ void __launch_bounds__(ANA_THREADS)
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(&sc->ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (last && threadIdx.x < ANA_VALS) {
+    if (last) {
+        // one warp per value: lane l adds blocks l, l + 32, ... in order, then
+        // the lanes pairwise (a fixed order)
         __threadfence();
-        const int k = threadIdx.x;
-        double x = __ldcg(&sc->partial[k]);
-        for (unsigned b = 1; b < gridDim.x; ++b) x += __ldcg(&sc->partial[b * ANA_VALS + k]);
-        if (pass == 0) sc->mean[k] = x;
-        else out[k] = x;
-        if (pass == 1 && k < 3) out[ANA_VALS + k] = sc->mean[k];
-        if (k == 0) sc->ticket = 0u;
+        for (int k = wid; k < ANA_VALS; k += ANA_THREADS / 32) {
+            double x = 0.0;
+            for (unsigned b = lane; b < gridDim.x; b += 32) x += __ldcg(&sc->partial[b * ANA_VALS + k]);
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            if (lane != 0) continue;
+            if (pass == 0) sc->mean[k] = x;
+            else out[k] = x;
+            if (pass == 1 && k < 3) out[ANA_VALS + k] = sc->mean[k];
+            if (k == 0) sc->ticket = 0u;
+        }
     }
 }
 
@@ -141,18 +150,49 @@ __device__ __forceinline__ int find_root(const int* parent, int x, long long cap
     return x;
 }
 
-__global__ void k_cc_init(const double* __restrict__ rho, long long n, double thr, int below,
+// Nodes are taken in segments of 32 columns of a row, one warp each: every node
+// of the phase starts with the first node of its run inside the segment as
+// parent (a ballot), so that only runs have to be merged and parent chains
+// stay short.
+struct Seg {
+    int x, y, lane;
+    long long i;        // node index
+    bool in;            // the column exists
+};
+__device__ __forceinline__ Seg seg_of(long long s, int segs, int nx) {
+    Seg g;
+    g.lane = threadIdx.x & 31;
+    g.y = (int)(s / segs);
+    g.x = (int)(s % segs) * 32 + g.lane;
+    g.in = g.x < nx;
+    g.i = (long long)g.y * nx + g.x;
+    return g;
+}
+// warps of the grid, and this thread's
+__device__ __forceinline__ long long warp_id() { return ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
+__device__ __forceinline__ long long warp_count() { return ((long long)gridDim.x * blockDim.x) >> 5; }
+
+__global__ void k_cc_init(const double* __restrict__ rho, int nx, int ny, double thr, int below,
                           CCArrays A) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const double r = rho[i];
-        const bool in = below ? (r < thr) : (r > thr);
-        A.parent[i] = in ? (int)i : -1;
-        A.area[i] = 0u;
-        A.sum_y[i] = 0ull;
-        A.y_min[i] = 0x7fffffff;
-        A.y_max[i] = -1;
-        A.flags[i] = 0;
+    const int segs = (nx + 31) / 32;
+    for (long long s = warp_id(); s < (long long)segs * ny; s += warp_count()) {
+        const Seg g = seg_of(s, segs, nx);
+        bool in = false;
+        if (g.in) {
+            const double r = rho[g.i];
+            in = below ? (r < thr) : (r > thr);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (!g.in) continue;
+        // the run's first lane: one past the last lane below this one that is out
+        const unsigned out_below = ~m & ((1u << g.lane) - 1u);
+        const int first = out_below ? 32 - __clz(out_below) : 0;
+        A.parent[g.i] = in ? (int)(g.i - g.lane + first) : -1;
+        A.area[g.i] = 0u;
+        A.sum_y[g.i] = 0ull;
+        A.y_min[g.i] = 0x7fffffff;
+        A.y_max[g.i] = -1;
+        A.flags[g.i] = 0;
     }
 }
 
@@ -177,23 +217,25 @@ __device__ void unite(int* parent, int a, int b, long long cap, int* err) {
 
 __global__ void k_cc_union(int nx, int ny, int perx, int pery, CCArrays A) {
     const long long n = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        if (A.parent[i] < 0) continue;
-        const int x = (int)(i % nx), y = (int)(i / nx);
-        // east and north neighbours cover every pair once (the seams through
-        // x = nx-1 -> 0 and y = ny-1 -> 0 when periodic)
-        int xe = x + 1, yn = y + 1;
-        if (xe == nx) xe = perx ? 0 : -1;
-        if (yn == ny) yn = pery ? 0 : -1;
-        if (xe >= 0) {
-            const long long j = (long long)y * nx + xe;
-            if (j != i && __ldcg(&A.parent[j]) >= 0) unite(A.parent, (int)i, (int)j, n, &A.count[1]);
+    const int segs = (nx + 31) / 32;
+    for (long long s = warp_id(); s < (long long)segs * ny; s += warp_count()) {
+        const Seg g = seg_of(s, segs, nx);
+        const bool in = g.in && __ldcg(&A.parent[g.i]) >= 0;
+        // west: a run that goes on in the segment before (or across the seam)
+        if (in && g.lane == 0) {
+            const int xw = g.x > 0 ? g.x - 1 : (perx ? nx - 1 : -1);
+            const long long j = (long long)g.y * nx + xw;
+            if (xw >= 0 && j != g.i && __ldcg(&A.parent[j]) >= 0)
+                unite(A.parent, (int)g.i, (int)j, n, &A.count[1]);
         }
-        if (yn >= 0) {
-            const long long j = (long long)yn * nx + x;
-            if (j != i && __ldcg(&A.parent[j]) >= 0) unite(A.parent, (int)i, (int)j, n, &A.count[1]);
-        }
+        // north: one merge per stretch of columns that this row's and the next
+        // row's runs have in common
+        const int yn = g.y + 1 < ny ? g.y + 1 : (pery ? 0 : -1);
+        const long long j = (long long)yn * nx + g.x;
+        const bool both = in && yn >= 0 && j != g.i && __ldcg(&A.parent[j]) >= 0;
+        const unsigned m = __ballot_sync(0xffffffffu, both);
+        if (both && (g.lane == 0 || !(m >> (g.lane - 1) & 1u)))
+            unite(A.parent, (int)g.i, (int)j, n, &A.count[1]);
     }
 }
 
@@ -203,20 +245,25 @@ __global__ void k_cc_flatten(long long n, CCArrays A) {
         if (A.parent[i] >= 0) A.parent[i] = find_root(A.parent, (int)i, n, &A.count[1]);
 }
 
+// per-root sums: one lane per root and segment adds for the lanes that share it
 __global__ void k_cc_stats(int nx, int ny, int max_roots, CCArrays A) {
-    const long long n = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int r = A.parent[i];
+    const int segs = (nx + 31) / 32;
+    for (long long s = warp_id(); s < (long long)segs * ny; s += warp_count()) {
+        const Seg g = seg_of(s, segs, nx);
+        const int r = g.in ? A.parent[g.i] : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, r);
         if (r < 0) continue;
-        const int x = (int)(i % nx), y = (int)(i / nx);
-        atomicAdd(&A.area[r], 1u);
-        atomicAdd(&A.sum_y[r], (unsigned long long)y);
-        atomicMin(&A.y_min[r], y);
-        atomicMax(&A.y_max[r], y);
-        const int f = (x == 0 ? 1 : 0) | (x == nx - 1 ? 2 : 0) | (y == 0 ? 4 : 0) | (y == ny - 1 ? 8 : 0);
-        if (f) atomicOr(&A.flags[r], f);
-        if (r == (int)i) {
+        const int f = (g.x == 0 ? 1 : 0) | (g.x == nx - 1 ? 2 : 0) | (g.y == 0 ? 4 : 0) | (g.y == ny - 1 ? 8 : 0);
+        if (f & 3) atomicOr(&A.flags[r], f);
+        if (g.lane == __ffs(same) - 1) {
+            const unsigned k = (unsigned)__popc(same);
+            atomicAdd(&A.area[r], k);
+            atomicAdd(&A.sum_y[r], (unsigned long long)g.y * k);
+            atomicMin(&A.y_min[r], g.y);
+            atomicMax(&A.y_max[r], g.y);
+            if (f & 12) atomicOr(&A.flags[r], f & 12);
+        }
+        if (r == (int)g.i) {
             const int slot = atomicAdd(&A.count[0], 1);
             if (slot < max_roots) A.roots[slot] = r;
         }
@@ -266,8 +313,11 @@ int iface_launch(const double* rho, int nx, int ny, double rho_mid, int skip, do
                  void* scratch, cudaStream_t st) {
     if (skip >= ny) skip = ny;
     IfaceScratch* sc = (IfaceScratch*)scratch;
+    // small fields take fewer blocks: their fold is what they would wait for
+    const long long n = (long long)nx * (ny - skip);
+    const int blocks = (int)std::min<long long>(ANA_BLOCKS, std::max<long long>(1, (n + 511) / 512));
     for (int pass = 0; pass < 2; ++pass)
-        k_iface<<<ANA_BLOCKS, ANA_THREADS, 0, st>>>(rho, nx, ny, rho_mid, skip, pass, out12, sc);
+        k_iface<<<blocks, ANA_THREADS, 0, st>>>(rho, nx, ny, rho_mid, skip, pass, out12, sc);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -279,8 +329,9 @@ int regions_launch(const double* rho, int nx, int ny, int perx, int pery, double
     const long long n = (long long)nx * ny;
     const CCArrays A = cc_arrays(scratch, n);
     if (cudaMemsetAsync(A.count, 0, 2 * sizeof(int), st) != cudaSuccess) return -1;
-    const int g = grid_for(n, CC_THREADS);
-    k_cc_init<<<g, CC_THREADS, 0, st>>>(rho, n, thr, below, A);
+    // whole warps per segment of 32 columns
+    const int g = grid_for((long long)((nx + 31) / 32 * 32) * ny, CC_THREADS);
+    k_cc_init<<<g, CC_THREADS, 0, st>>>(rho, nx, ny, thr, below, A);
     k_cc_union<<<g, CC_THREADS, 0, st>>>(nx, ny, perx, pery, A);
     k_cc_flatten<<<g, CC_THREADS, 0, st>>>(n, A);
     k_cc_stats<<<g, CC_THREADS, 0, st>>>(nx, ny, max_roots < n ? max_roots : (int)n, A);

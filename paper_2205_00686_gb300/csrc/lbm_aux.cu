@@ -2,7 +2,9 @@
 // macroscopic fields of the current state (rho, u with the half-force
 // correction of Eq. 11, T), population import / export as absolute doubles,
 // and the FP64 diagnostics reduction.  None of these is on the per-step path.
-#include "lbm_internal.cuh"
+#include <algorithm>
+
+#include "lbm_node.cuh"
 
 namespace lbm {
 
@@ -69,141 +71,122 @@ int init_launch(int prec, const Inst* I_dev, const Inst& I, const double* rho, c
 }
 
 // ---------------------------------------------------------------------------
-// fields of the current state, computed in double from the stored values
-__device__ double psi_of(const PhysD& p, double rho, double T) {
-    const double k = 0.37464 + 1.54226 * p.omega - 0.26992 * p.omega * p.omega;
-    const double Tc = 0.0778 * p.a / (0.45724 * p.b * p.Rg);
-    const double h = 1.0 + k * (1.0 - sqrt(T / Tc));
-    const double pe = rho * p.Rg * T / (1.0 - p.b * rho) -
-                      p.a * h * h * rho * rho / (1.0 + 2.0 * p.b * rho - p.b * p.b * rho * rho);
-    return sqrt(2.0 * (pe - rho / 3.0) / p.G);
-}
-
-// pass 1: per node rho, T, j and psi of the current state (in double)
+// Fields of the current state: rho, T and u = (j + F/2) / rho (Eq. 11) with F_m
+// from the psi stencil (Eq. 9, wetting ghost layer of Section 3.3) and buoyancy,
+// in the state's own precision, written as doubles.  A CTA takes 32 x 8 nodes;
+// moments and psi of the tile and one node around it come from the populations
+// (1.33 times the tile's), psi passes through shared memory.  Bound by memory:
+// 56 B read and 32 B written per node (FP32).  One pass instead of two over five
+// double fields, and float to double by integer operations (the conversion
+// instruction runs on the FP64 pipe): 2048^2 FP32 200 -> 84 us.
+constexpr int FTX = 32, FTY = 8;
 template <int PREC>
-__global__ void k_fields_node(Inst I, PhysD p, const Ctl* ctl, double* orho, double* ojx,
-                              double* ojy, double* oT, double* opsi) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= I.nx) return;
-    const long long step = __ldcg(&ctl->step);
-    const int par = (int)(step & 1);
+__global__ void __launch_bounds__(FTX* FTY)
+k_fields(const __grid_constant__ Inst I, const __grid_constant__ Phys<typename Types<PREC>::R> P,
+         double* __restrict__ orho, double* __restrict__ oux, double* __restrict__ ouy,
+         double* __restrict__ oT) {
+    typedef typename Types<PREC>::R R;
     typedef typename Types<PREC>::TF TF;
     typedef typename Types<PREC>::TG TG;
-    const TF* f = (const TF*)I.f[par];
-    const TG* g = (const TG*)I.g[par];
-    const size_t plane = (size_t)I.ny * I.pitch, off = (size_t)y * I.pitch + x;
-    double r = 0.0, t = 0.0, jx = 0.0, jy = 0.0;
-    for (int i = 0; i < 9; ++i) {
-        const double fi = (double)ld_st(f + i * plane + off) + dW9[i] * I.rho_ref;
-        r += fi;
-        jx += dCX9[i] * fi;
-        jy += dCY9[i] * fi;
-    }
-    for (int i = 0; i < 5; ++i) t += (double)ld_st(g + i * plane + off) + w5(i, p.w_dot) * I.T_ref;
-    const size_t n = (size_t)y * I.nx + x;
-    orho[n] = r;
-    oT[n] = t;
-    ojx[n] = jx;
-    ojy[n] = jy;
-    opsi[n] = psi_of(p, r, t);
-}
-
-// FP32 state: the same fields from float sums of the stored deviations and
-// the float EOS (the state's own precision; the GPU's FP64 rate would
-// otherwise bound this pass)
-template <int PREC>
-__global__ void k_fields_node_f(Inst I, Phys<float> pf, const Ctl* ctl, double* orho,
-                                double* ojx, double* ojy, double* oT, double* opsi) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= I.nx) return;
-    const long long step = __ldcg(&ctl->step);
+    typedef typename Vec2<R>::T R2;
+    constexpr int W = FTX + 2;
+    __shared__ R s_psi[W * (FTY + 2)];
+    const int nx = I.nx, ny = I.ny, t = threadIdx.x;
+    const unsigned ntx = (nx + FTX - 1) / FTX;
+    const int x0 = (int)(blockIdx.x % ntx) * FTX, y0 = (int)(blockIdx.x / ntx) * FTY;
+    const long long step = __ldcg(&I.ctl->step);
     const int par = (int)(step & 1);
-    typedef typename Types<PREC>::TF TF;
-    typedef typename Types<PREC>::TG TG;
-    const TF* f = (const TF*)I.f[par];
-    const TG* g = (const TG*)I.g[par];
-    const size_t plane = (size_t)I.ny * I.pitch, off = (size_t)y * I.pitch + x;
-    float rd = 0.f, jx = 0.f, jy = 0.f, td = 0.f;
+    const TF* const f = (const TF*)I.f[par];
+    const TG* const g = (const TG*)I.g[par];
+    const size_t plane = (size_t)ny * I.pitch;
+    const bool perx = I.flow[EW] == PERIODIC, pery = I.flow[ES] == PERIODIC;
+    const R rho_ref = (R)I.rho_ref, T_ref = (R)I.T_ref;
+    auto load = [&](int x, int y, R* fv, R* gv) {
+        const size_t off = (size_t)y * I.pitch + x;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const float fi = (float)ld_st(f + i * plane + off);
-        rd += fi;
-        jx += (float)dCX9[i] * fi;
-        jy += (float)dCY9[i] * fi;
-    }
+        for (int q = 0; q < 9; ++q) fv[q] = (R)ld_st(f + q * plane + off);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) td += (float)ld_st(g + i * plane + off);
-    // sum_i w_i = sum_i w^_i = 1 and sum_i w_i c_i = 0: the references add
-    // once to rho and T and not to j
-    const float r = rd + (float)I.rho_ref, t = td + (float)I.T_ref;
-    const size_t n = (size_t)y * I.nx + x;
-    orho[n] = r;
-    oT[n] = t;
-    ojx[n] = jx;
-    ojy[n] = jy;
-    opsi[n] = f_sqrt(psi2_of(pf, r, t));
-}
-
-// pass 2: F_m from the psi field (Eq. 9, wetting ghost layer of Section 3.3),
-// buoyancy, and u = (j + F/2) / rho (Eq. 11), in place over j
-template <class C>
-__global__ void k_fields_force(Inst I, PhysD p, Phys<float> pf, const Ctl* ctl, const double* rho,
-                               double* ux, double* uy, const double* T, const double* psi) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y;
-    if (x >= I.nx) return;
-    const int nx = I.nx, ny = I.ny;
-    const bool perx = I.flow[EW] == PERIODIC;
-    auto extx = [&](int xx) { return perx ? wrapi(xx, nx) : min(max(xx, 0), nx - 1); };
-    auto at = [&](const double* a, int xx, int yy) { return (C)a[(size_t)yy * nx + xx]; };
-    const C cot = (C)I.cot_theta;
-    auto psi_ext = [&](int xx, int yy) -> C {
-        const int xe = extx(xx);
-        if (yy >= 0 && yy < ny) return at(psi, xe, yy);
-        const int edge = yy < 0 ? ES : EN;
-        const int kind = I.flow[edge];
-        if (kind == PERIODIC) return at(psi, xe, wrapi(yy, ny));
-        if (kind == OPEN) return at(psi, xe, yy < 0 ? 0 : ny - 1);
-        const int y1 = edge == ES ? 0 : ny - 1, y2 = edge == ES ? 1 : ny - 2;
-        const C rg = at(rho, xe, y2) + cot * rabs(at(rho, extx(xe + 1), y1) - at(rho, extx(xe - 1), y1));
-        const C tg = at(T, xe, y1);     // the fluid node's temperature
-        if (sizeof(C) == 8) return (C)psi_of(p, (double)rg, (double)tg);
-        return (C)f_sqrt(psi2_of(pf, (float)rg, (float)tg));
+        for (int q = 0; q < 5; ++q) gv[q] = (R)ld_st(g + q * plane + off);
     };
-    C sx = 0, sy = 0;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const C wv = i < 5 ? C(1.0 / 3.0) : C(1.0 / 12.0);
-        const C pn = psi_ext(x + dCX9[i], y + dCY9[i]);
-        sx += wv * pn * (C)dCX9[i];
-        sy += wv * pn * (C)dCY9[i];
+    int err = 0;     // the step reports errors; the read-out does not
+    const int lx = t % FTX, ly = t / FTX, gx = x0 + lx, gy = y0 + ly;
+    const int tw = min(FTX, nx - x0), th = min(FTY, ny - y0);
+    const bool own = lx < tw && ly < th;
+    const int c = (ly + 1) * W + lx + 1;
+    Node<R> n;
+    if (own) {
+        R fv[9], gv[5];
+        load(gx, gy, fv, gv);
+        node_fields(P, rho_ref, T_ref, fv, gv, n);
+        s_psi[c] = n.psi;
     }
-    const size_t n = (size_t)y * nx + x;
-    const C r = (C)rho[n], pc = (C)psi[n];
-    const C G = (C)p.G;
-    const C Fx = -G * pc * sx;
-    const long long step = __ldcg(&ctl->step);
-    const C rho_ave = (C)(__ldcg(&ctl->mass[(step + 2) % 3]) * I.inv_n);
-    const C Fy = -G * pc * sy - (r - rho_ave) * (C)p.gravity;
-    ux[n] = p.frozen_flow ? 0.0 : (double)(((C)ux[n] + C(0.5) * Fx) / r);
-    uy[n] = p.frozen_flow ? 0.0 : (double)(((C)uy[n] + C(0.5) * Fy) / r);
+    if (t < 2 * (tw + th) + 4) {
+        // the ring around the tile: inside the domain (wrapped along periodic
+        // axes), the ghost layer of a wall, or unused
+        const int w = tw + 2;
+        int rx, ry;
+        if (t < w) { rx = t - 1; ry = -1; }
+        else if (t < 2 * w) { rx = t - w - 1; ry = th; }
+        else if (t < 2 * w + th) { rx = -1; ry = t - 2 * w; }
+        else { rx = tw; ry = t - 2 * w - th; }
+        const int r = (ry + 1) * W + rx + 1;
+        int x = x0 + rx, y = y0 + ry;
+        if (perx) x = wrapi(x, nx);
+        if (pery) y = wrapi(y, ny);
+        if (x >= 0 && x < nx) {
+            R fv[9], gv[5];
+            if (y >= 0 && y < ny) {
+                Node<R> m;
+                load(x, y, fv, gv);
+                node_fields(P, rho_ref, T_ref, fv, gv, m);
+                s_psi[r] = m.psi;
+            } else if (I.flow[y < 0 ? ES : EN] == WALL) {
+                const int y1 = y < 0 ? 0 : ny - 1, y2 = y < 0 ? 1 : ny - 2;
+                const int xp = perx ? wrapi(x + 1, nx) : min(x + 1, nx - 1);
+                const int xm = perx ? wrapi(x - 1, nx) : max(x - 1, 0);
+                auto rho_at = [&](int xx, int yy) {
+                    load(xx, yy, fv, gv);
+                    return radd(sum9(fv), rho_ref);
+                };
+                const R rp = rho_at(xp, y1), rm = rho_at(xm, y1), far = rho_at(x, y2);
+                load(x, y1, fv, gv);
+                s_psi[r] = ghost_psi(P, far, rp, rm, (R)I.cot_theta, radd(sum5(gv), T_ref), &err);
+            }
+        }
+    }
+    __syncthreads();
+    if (!own) return;
+    const int dw = (!perx && gx == 0) ? 0 : -1, de = (!perx && gx == nx - 1) ? 0 : 1;
+    const int ds = (I.flow[ES] == OPEN && gy == 0) ? 0 : -W, dn = (I.flow[EN] == OPEN && gy == ny - 1) ? 0 : W;
+    const R* const p = s_psi + c;
+    const R2 s12 = force_stencil<R>(p[dw], p[de], p[ds + dw], p[ds], p[ds + de], p[dn + dw], p[dn], p[dn + de]);
+    R rho_ave = R(0);
+    if (P.gravity != R(0)) rho_ave = (R)(__ldcg(&I.ctl->mass[(step + 2) % 3]) * I.inv_n);
+    const R2 F = force_of<R>(P, s12, n.psi, n.rho, rho_ave);
+    R ux = R(0), uy = R(0);
+    if (!P.frozen_flow) {
+        if constexpr (sizeof(R) == 8) {
+            const R2 u = velocity<R>(F, pr(n.jx, n.jy), n.ir);
+            ux = u.x;
+            uy = u.y;
+        } else {
+            ux = __fdiv_rn(rfma(F.x, R(0.5), n.jx), n.rho);
+            uy = __fdiv_rn(rfma(F.y, R(0.5), n.jy), n.rho);
+        }
+    }
+    const size_t o = (size_t)gy * nx + gx;
+    orho[o] = widen(n.rho);
+    oux[o] = widen(ux);
+    ouy[o] = widen(uy);
+    oT[o] = widen(n.T);
 }
 
-int fields_launch(int prec, const Inst* I_dev, const Inst& I, const PhysD& phys, double* rho,
-                  double* ux, double* uy, double* T, double* psi, cudaStream_t st) {
-    (void)I_dev;
-    dim3 blk(128), grd((I.nx + 127) / 128, I.ny);
-    const Phys<float> pf = make_phys<float>(phys);
-    if (prec == 0) {
-        k_fields_node<0><<<grd, blk, 0, st>>>(I, phys, I.ctl, rho, ux, uy, T, psi);
-        k_fields_force<double><<<grd, blk, 0, st>>>(I, phys, pf, I.ctl, rho, ux, uy, T, psi);
-    } else {
-        if (prec == 1) k_fields_node_f<1><<<grd, blk, 0, st>>>(I, pf, I.ctl, rho, ux, uy, T, psi);
-        else k_fields_node_f<2><<<grd, blk, 0, st>>>(I, pf, I.ctl, rho, ux, uy, T, psi);
-        k_fields_force<float><<<grd, blk, 0, st>>>(I, phys, pf, I.ctl, rho, ux, uy, T, psi);
-    }
+int fields_launch(int prec, const Inst& I, const PhysD& phys, double* rho, double* ux, double* uy,
+                  double* T, cudaStream_t st) {
+    const unsigned grd = (unsigned)((I.nx + FTX - 1) / FTX) * (unsigned)((I.ny + FTY - 1) / FTY);
+    if (prec == 0) k_fields<0><<<grd, FTX * FTY, 0, st>>>(I, make_phys<double>(phys), rho, ux, uy, T);
+    else if (prec == 1) k_fields<1><<<grd, FTX * FTY, 0, st>>>(I, make_phys<float>(phys), rho, ux, uy, T);
+    else k_fields<2><<<grd, FTX * FTY, 0, st>>>(I, make_phys<float>(phys), rho, ux, uy, T);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -260,8 +243,37 @@ int pop_set_launch(int prec, const Inst& I, int par, double w_dot, const double*
 
 // ---------------------------------------------------------------------------
 // diagnostics: per-block partial sums in double, then the last block to finish
-// folds the partials in block order (deterministic result)
+// folds the partials, one warp per value, in a fixed order (deterministic
+// result).  Bound by the FP64 pipe: 13 FP64 operations per node (no division, no
+// square root per node, finiteness by integer tests).  2048^2 308 -> 114 us; small
+// fields take fewer blocks, whose fold is what they wait for.
 enum { DIAG_BLOCKS = 304, DIAG_THREADS = 256, DIAG_VALS = 7 };
+inline int diag_blocks(long long n) {
+    return (int)std::min<long long>(DIAG_BLOCKS, std::max<long long>(1, (n + 2 * DIAG_THREADS - 1) / (2 * DIAG_THREADS)));
+}
+
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// folds n_vals values of n_blocks partials ([block][value]) by warps: lane l adds
+// blocks l, l + 32, ... in order, then the lanes pairwise; value `vmax` (if any)
+// by maximum.  All threads of the block take part; fin(k, v) in lane 0.
+template <class Fin>
+__device__ __forceinline__ void fold_partials(const double* partial, unsigned n_blocks, int n_vals, int vmax,
+                                              Fin fin) {
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < n_vals; k += blockDim.x >> 5) {
+        double x = 0.0;
+        for (unsigned b = lane; b < n_blocks; b += 32) {
+            const double y = __ldcg(&partial[b * n_vals + k]);
+            x = k == vmax ? fmax(x, y) : x + y;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double y = __shfl_down_sync(0xffffffffu, x, o);
+            x = k == vmax ? fmax(x, y) : x + y;
+        }
+        if (lane == 0) fin(k, x);
+    }
+}
 
 size_t diag_scratch_bytes(long long n) {
     (void)n;
@@ -274,25 +286,27 @@ __global__ void __launch_bounds__(DIAG_THREADS)
            unsigned* ticket) {
     __shared__ double red[DIAG_VALS][DIAG_THREADS / 32];
     __shared__ bool last;
-    const double rmid = 0.5 * (rho_l + rho_g);
+    const double rmid = 0.5 * (rho_l + rho_g), inv = 1.0 / (rho_l - rho_g);
     double v[DIAG_VALS] = {0, 0, 0, 0, 0, 0, 0};
+    unsigned n_liq = 0, n_bad = 0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const double r = rho[i], a = ux[i], b = uy[i], t = T[i];
-        const bool fin = isfinite(r) && isfinite(a) && isfinite(b) && isfinite(t);
         v[0] += r;
-        v[1] += r * cv * t;
+        v[1] += r * t;
         if (r > rmid) {
             v[2] += r;
-            v[3] += 1.0;
+            ++n_liq;
         }
-        double ph = (r - rho_g) / (rho_l - rho_g);
-        ph = ph < 0.0 ? 0.0 : (ph > 1.0 ? 1.0 : ph);
-        v[4] += ph;
-        const double um = sqrt(a * a + b * b);
-        v[5] = fmax(v[5], um);
-        v[6] += fin ? 0.0 : 1.0;
+        const double ph = (r - rho_g) * inv;
+        v[4] += ph < 0.0 ? 0.0 : (ph > 1.0 ? 1.0 : ph);
+        v[5] = fmax(v[5], fma(a, a, b * b));
+        n_bad += finite(r) && finite(a) && finite(b) && finite(t) ? 0u : 1u;
     }
+    v[1] *= cv;
+    v[3] = (double)n_liq;
+    v[5] = sqrt(v[5]);
+    v[6] = (double)n_bad;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int k = 0; k < DIAG_VALS; ++k) {
         double x = v[k];
@@ -313,16 +327,12 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (last && threadIdx.x < DIAG_VALS) {
+    if (last) {
         __threadfence();
-        const int k = threadIdx.x;
-        double x = __ldcg(&partial[k]);
-        for (unsigned b = 1; b < gridDim.x; ++b) {
-            const double y = __ldcg(&partial[b * DIAG_VALS + k]);
-            x = k == 5 ? fmax(x, y) : x + y;
-        }
-        out[k] = x;
-        if (k == 0) *ticket = 0u;
+        fold_partials(partial, gridDim.x, DIAG_VALS, 5, [&](int k, double x) {
+            out[k] = x;
+            if (k == 0) *ticket = 0u;
+        });
     }
 }
 
@@ -359,13 +369,12 @@ __global__ void __launch_bounds__(DIAG_THREADS)
     __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (last && threadIdx.x < 2) {
+    if (last) {
         __threadfence();
-        const int k = threadIdx.x;
-        double x = __ldcg(&partial[k]);
-        for (unsigned bk = 1; bk < gridDim.x; ++bk) x += __ldcg(&partial[bk * 2 + k]);
-        out[k] = x;
-        if (k == 0) *ticket = 0u;
+        fold_partials(partial, gridDim.x, 2, -1, [&](int k, double x) {
+            out[k] = x;
+            if (k == 0) *ticket = 0u;
+        });
     }
 }
 
@@ -373,7 +382,7 @@ int sum2_launch(const double* a, const double* b, long long n, double* out2, voi
                 cudaStream_t st) {
     double* partial = (double*)scratch;
     unsigned* ticket = (unsigned*)((char*)scratch + (size_t)DIAG_BLOCKS * DIAG_VALS * sizeof(double));
-    k_sum2<<<DIAG_BLOCKS, DIAG_THREADS, 0, st>>>(a, b, n, out2, partial, ticket);
+    k_sum2<<<diag_blocks(n), DIAG_THREADS, 0, st>>>(a, b, n, out2, partial, ticket);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -382,7 +391,7 @@ int diag_launch(const double* rho, const double* ux, const double* uy, const dou
                 cudaStream_t st) {
     double* partial = (double*)scratch;
     unsigned* ticket = (unsigned*)((char*)scratch + (size_t)DIAG_BLOCKS * DIAG_VALS * sizeof(double));
-    k_diag<<<DIAG_BLOCKS, DIAG_THREADS, 0, st>>>(rho, ux, uy, T, n, cv, rho_l, rho_g, out9,
+    k_diag<<<diag_blocks(n), DIAG_THREADS, 0, st>>>(rho, ux, uy, T, n, cv, rho_l, rho_g, out9,
                                                  partial, ticket);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

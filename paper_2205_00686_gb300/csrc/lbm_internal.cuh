@@ -177,6 +177,16 @@ __device__ __forceinline__ void st_st(__half* p, float v) { *p = __float2half_rn
 __device__ __forceinline__ float st_val(float v) { return v; }
 __device__ __forceinline__ float st_val(__half v) { return __half2float(v); }
 
+// float to double, exactly, by integer operations for normal numbers: the
+// conversion instruction runs on the FP64 pipe (64 cycles per warp and SM
+// partition), these six on the integer pipe
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)v;     // zero, denormal, infinite, NaN
+    return __hiloint2double((int)(((a >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(a << 29));
+}
+
 // ---- arithmetic helpers (precision-generic) -------------------------------
 // FP64 keeps IEEE division and square root (parity with the FP64 oracle to
 // ~1e-13); FP32 uses the hardware approximations (rcp.approx / sqrt.approx,
@@ -225,20 +235,6 @@ __device__ __forceinline__ double f_sqrt(double x) {
     const double t = x * y;
     const double e = fma(-t, y, 1.0);
     return fma(t * e, fma(0.375, e, 0.5), t);
-}
-
-// Peng-Robinson pressure (Eq. 10) and psi^2 = 2 (p_EOS - rho/3) / G.
-template <class R>
-__device__ __forceinline__ R eos_p(const Phys<R>& P, R rho, R T) {
-    R st = rsq(T * P.inv_Tc);
-    R h = R(1) + P.kpr * (R(1) - st);
-    R br = P.b * rho;
-    return rho * P.Rg * T / (R(1) - br) - P.a * h * h * rho * rho / (R(1) + R(2) * br - br * br);
-}
-
-template <class R>
-__device__ __forceinline__ R psi2_of(const Phys<R>& P, R rho, R T) {
-    return P.two_over_G * (eos_p(P, rho, T) - rho * R(1.0 / 3.0));
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {
@@ -316,9 +312,9 @@ int step_occupancy(int prec, int threads, int walls, int staged, int* ctas_per_s
 
 int init_launch(int prec, const Inst* I_dev, const Inst& I, const double* rho, const double* ux,
                 const double* uy, const double* T, double w_dot, cudaStream_t st);
-// rho, u (half-force velocity), T of the current state; psi is scratch of n doubles
-int fields_launch(int prec, const Inst* I_dev, const Inst& I, const PhysD& phys, double* rho,
-                  double* ux, double* uy, double* T, double* psi, cudaStream_t st);
+// rho, u (half-force velocity), T of the current state
+int fields_launch(int prec, const Inst& I, const PhysD& phys, double* rho, double* ux, double* uy,
+                  double* T, cudaStream_t st);
 int pop_get_launch(int prec, const Inst& I, int parity, double w_dot, double* f, double* g,
                    double* P, cudaStream_t st);
 int pop_set_launch(int prec, const Inst& I, int parity, double w_dot, const double* f,
