@@ -44,12 +44,11 @@ __device__ __forceinline__ float ld_l2(const __half* p) {
     return __half2float(__ushort_as_half(__ldcg(reinterpret_cast<const unsigned short*>(p))));
 }
 
-// Most threads per CTA and CTAs per SM.  FP32: two CTAs of 256 threads at 128
-// registers (three at 80 registers spill: 300 x 600 15.3 -> 18.5 us per step,
-// 256^2 5.1 -> 6.5).  FP64: one CTA of up to 288 threads (20 x 14 nodes, 168
+// Most threads per CTA.  FP32: up to 512, so that 128 registers are left (two CTAs
+// of 256 threads per SM; at 80 registers three fit but spill: 300 x 600 15.3 ->
+// 18.5 us per step, 256^2 5.1 -> 6.5).  FP64: up to 288 (20 x 14 nodes, 168
 // registers), so that 200 x 200 fits one round of 152 SMs.
-constexpr int TILE_MAX(int prec) { return prec == 0 ? 288 : 256; }
-constexpr int TILE_MIN(int prec) { return prec == 0 ? 1 : 2; }
+constexpr int TILE_MAX(int prec) { return prec == 0 ? 288 : 512; }
 
 // release / acquire on the grid counter
 __device__ __forceinline__ unsigned bar_load(const unsigned* p) {
@@ -70,7 +69,7 @@ __host__ __device__ inline size_t tile_bytes(size_t es, int tx, int ty) {
 }
 
 template <int PREC, bool UNIT>
-__global__ void __launch_bounds__(TILE_MAX(PREC), TILE_MIN(PREC))
+__global__ void __launch_bounds__(TILE_MAX(PREC))
 k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typename Types<PREC>::R> P) {
     typedef typename Types<PREC>::R R;
     typedef typename Types<PREC>::TF TF;
@@ -483,14 +482,17 @@ int tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int threads, 
 
 // Which tile, and whether the domain takes this form at all.
 //
-// FP32 / FP16-g: a step is bound by latency (barrier 1.3-1.7 us, loads, two
-// barriers of the CTA), about 3.4 us per round of resident tiles.  32 x 8 nodes
-// (256 threads, full rows of 128 bytes) beat 16 x 16, 16 x 8, 8 x 8 and 64 x 4
-// everywhere except where 8 x 8 tiles with their surrounding nodes on threads
-// of their own (one pass of stage A instead of two) leave at most one per SM:
-// 64^2 4.0 -> 3.35 us.  Against the sweep with its best tile, 512^2 is 15.4 us
-// against 23.5, 768^2 (8 rounds) 28.7 against 28.7 and 1024^2 48.5 against
-// 40.6: up to 7 rounds.
+// FP32 / FP16-g: a step is bound by latency (grid barrier 1.3-1.7 us, loads, three
+// barriers of the CTA per tile): about 1.6 us and, per round of resident tiles,
+// 3.45 us for 32 x 8 nodes (two CTAs per SM), 2.4 for 32 x 10 and 2.75 for 32 x
+// 12 (one).  Which one wastes least of its last round decides (us per step, 32
+// x 8 / 32 x 10 / 32 x 12): 256^2 5.1 / 6.8 / 7.2, 400 x 200 FP16-g 8.7 / 7.8 / 7.9,
+// 300 x 600 15.3 / 14.9 / 15.6, 512^2 15.2 / 16.0 / 15.1, 700^2 22.9 / 27.1 / 25.2.
+// Full rows of 128 bytes beat 16 x 16, 16 x 8 and 8 x 8 everywhere except where 8
+// x 8 tiles with their surrounding nodes on threads of their own (one pass of
+// stage A instead of two) leave at most one per SM: 64^2 4.0 -> 3.35 us.  Against
+// the sweep with its best tile, 512^2 is 15.1 us against 23.5, 768^2 28.7 (8
+// rounds of 32 x 8) against 28.7 and 1024^2 48.5 against 40.6: up to 26 us here.
 //
 // FP64: each of an SM's four partitions takes 64 cycles per FP64 warp
 // instruction, so the time is that of the busiest partition: about 170
@@ -505,10 +507,10 @@ int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out
     out->tx = 0;
     if ((long long)I.nx * I.ny > (1 << 20)) return 0;   // far beyond either limit below
     struct Cand { int tx, ty, sep; };
-    static const Cand c32[2] = {{8, 8, 1}, {32, 8, 0}};
+    static const Cand c32[4] = {{8, 8, 1}, {32, 8, 0}, {32, 10, 0}, {32, 12, 0}};
     static const Cand c64[5] = {{8, 4, 1}, {8, 8, 1}, {32, 8, 0}, {16, 8, 0}, {20, 14, 0}};
     const Cand* const cand = prec == 0 ? c64 : c32;
-    const int n_cand = prec == 0 ? 5 : 2;
+    const int n_cand = prec == 0 ? 5 : 4;
     const size_t es = prec == 0 ? 8 : 4;
     double best = 1e30;
     for (int k = 0; k < n_cand; ++k) {
@@ -530,8 +532,9 @@ int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out
         double us;
         if (prec != 0) {
             if (cand[k].sep && nt > sms) continue;
-            if (rounds > 7) continue;
-            us = 3.4 * (double)rounds + k;   // 8 x 8 first where it applies
+            static const double per_round[4] = {1.75, 3.45, 2.4, 2.75};
+            us = 1.6 + per_round[k] * (double)rounds;
+            if (us > 26.0) continue;
         } else {
             const double ring_cost = 65.0 + 25.0 * n_ring1 / n_ring;
             // the busiest partition of one CTA, and all partitions of the CTAs
