@@ -467,7 +467,7 @@ def bench_3d(lbm, stream, torch, peak, n=256, steps=200, warmup=20, zseg=None):
                          "kernels": "k3_fused (+ k3_advance)"},
             "three_kernels": {"mlups": round(N * s3 / t3 / 1e6, 1), "steps": s3,
                               "hbm_frac_of_measured": round(ach3 / peak, 4),
-                              "kernels": "k3_force + k3_collide + k3_macro (+ k3_advance)"},
+                              "kernels": "k3_macro + k3_flow + k3_thermal (+ k3_advance)"},
             "max_u_after": round(dg["max_u"], 5), "nonfinite": dg["nonfinite"]}
 
 

@@ -9,13 +9,13 @@
 // Then k3_march (below; the default in FP32) does the rest of the step in one
 // kernel over z-marching tiles.  The other form (the default in FP64) is two
 // more kernels over the nodes plus a one-thread counter update:
-//   k3_force    psi of the 18 neighbours (ghost layer at walls) -> F_m, F,
-//               u = (j + F/2)/rho, |F_m|^2/psi^2                (Eqs. 9, 11)
-//   k3_collide  div u (neighbour u), grad T (local moments), Q, P^n, S;
-//               D3Q19 and D3Q7 collisions; f* pushed to its destination
-//               (bounce-back at walls); g*_i blended into the destination's
+//   k3_flow     psi of the 18 neighbours (ghost layer at walls) -> F_m, F,
+//               u = (j + F/2)/rho, |F_m|^2/psi^2; D3Q19 collision, f* pushed
+//               to its destination (bounce-back at walls)    (Eqs. 5, 9, 11)
+//   k3_thermal  div u (neighbour u), grad T (local moments), Q, P^n, S;
+//               D3Q7 collision; g*_i blended into the destination's
 //               g(t+1) = g + (g* - g)/(rho c_v) (anti-bounce-back at walls),
-//               P^n stored                          (Eqs. 5, 20, 24, 39)
+//               P^n stored                             (Eqs. 20, 24, 39)
 //
 // Populations are stored as deviations f_i - w_i rho_ref and g_i - w^_i T_ref,
 // in blocks of 32 nodes along x: a block holds its 19 (or 7) populations one
@@ -28,7 +28,7 @@
 // paper's setting) the collision needs of f only rho, j and the five stress
 // moments (collide19_unit): about 310 operations per node and step instead
 // of 770, which is what bounds the FP64 step, and no moment matrices (96^3
-// FP64 in the step over nodes: 1080 -> 601 us).
+// FP64 in the step over nodes: 1080 -> 540 us).
 #include <math.h>
 #include <string.h>
 
@@ -180,10 +180,11 @@ __host__ __device__ constexpr int hy(int i) { return i == 3 ? 1 : (i == 4 ? -1 :
 __host__ __device__ constexpr int hz(int i) { return i == 5 ? 1 : (i == 6 ? -1 : 0); }
 
 // per-node planes: the fields of the current state (rho as its deviation from
-// rho_ref, which keeps the precision of the populations) and, for the step over
-// nodes and the read-out, T, u and F (which share planes with the stresses)
+// rho_ref, which keeps the precision of the populations), E = T dp/dT / (12 rho
+// c_v), and, for the step over nodes and the read-out, T, u and IC = 1/(rho c_v)
+// (k3_flow, once it has read the node's j_x)
 enum { Q_RHO = 0, Q_PSI, Q_E, Q_JX, Q_JY, Q_JZ, Q_S, Q_T = Q_S + 5, Q_UX, Q_UY, Q_UZ, Q_N,
-       Q_FX = Q_S, Q_FY, Q_FZ, Q_F2, Q_IC };   // E = T dp/dT / (12 rho c_v), IC = 1/(rho c_v)
+       Q_IC = Q_JX };
 
 // Blocks of XB nodes along x: population i of node n at fofs(n) + i XB, gofs(n)
 // + i XB (the pitch is a multiple of 32)
@@ -568,8 +569,9 @@ __device__ __forceinline__ void force_at(const Dom3& D, const Phys<R>& P, const 
     *S = s[0] * s[0] + s[1] * s[1] + s[2] * s[2];
 }
 
+// u of the read-out
 template <class R>
-__global__ void __launch_bounds__(128) k3_force(Dom3 D, Phys<R> P, Lat3<R> L, int want_F) {
+__global__ void __launch_bounds__(128) k3_force(Dom3 D, Phys<R> P, Lat3<R> L) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -588,17 +590,78 @@ __global__ void __launch_bounds__(128) k3_force(Dom3 D, Phys<R> P, Lat3<R> L, in
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) A[(Q_UX + a) * D.plane + n] = u[a];
-    if (want_F) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) A[(Q_FX + a) * D.plane + n] = F[a];
-        A[Q_F2 * D.plane + n] = S;
-    }
     if (err) atomicOr(&D.ctl->err, err);
 }
 
 // ---------------------------------------------------------------------------
+// Step over nodes (the default in FP64), after k3_macro: k3_flow has the force,
+// u and the flow collision, k3_thermal what needs the neighbours' u and 1/(rho
+// c_v).  In FP64 both are bound by the FP64 pipe (84 % busy).  At unit rates
+// the collision takes rho, j and the stresses k3_macro has formed, so that
+// neither the moments are formed again from f (a collision kernel that did both
+// lattices after a kernel for the force spent 49 of 353 FP64 operations per
+// node on that) nor F passes through memory: 96^3 FP64 605 -> 540 us per step
+// (FP32 on the same path, 128^3: 189 -> 163).
 template <class R, bool UNIT>
-__global__ void __launch_bounds__(128) k3_collide(Dom3 D, Phys<R> P, Lat3<R> L) {
+__global__ void __launch_bounds__(128) k3_flow(Dom3 D, Phys<R> P, Lat3<R> L) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int z = blockIdx.z;
+    if (x >= D.nx || y >= D.ny) return;
+    const long long step = __ldcg(&D.ctl->step);
+    const int par = (int)(step & 1);
+    R* A = (R*)D.aux;
+    const size_t n = nid<R>(D, x, y, z);
+    const Nbr nb = nbr_offsets(D, x, y, z);
+    int err = 0;
+    Mom3<R> m;
+    m.rhod = A[Q_RHO * D.plane + n];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m.j[a] = A[(Q_JX + a) * D.plane + n];
+    R F[3], S;
+    force_at<R>(D, P, L, x, y, z, n, nb, step, &err, F, &S);
+    const R rho = m.rhod + L.rho_ref, ir = f_rcp(rho);
+    R u[3] = {0, 0, 0};
+    if (!L.frozen_flow) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[a] = (m.j[a] + R(0.5) * F[a]) * ir;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) A[(Q_UX + a) * D.plane + n] = u[a];
+    A[Q_IC * D.plane + n] = ir * P.inv_cv;
+    if (err) atomicOr(&D.ctl->err, err);
+
+    // ---- D3Q19 MRT collision, pushed to x + c_i (bounce-back through walls)
+    const R* fc = (const R*)D.f[par] + fofs(n);
+    R* fn = (R*)D.f[par ^ 1];
+    R f[19];
+    if (!UNIT || L.frozen_flow) {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) f[i] = fc[i * XB];
+    }
+    if (L.frozen_flow) {
+#pragma unroll
+        for (int i = 0; i < 19; ++i) fn[fofs(n) + i * XB] = f[i];
+        return;
+    }
+    if constexpr (UNIT) {
+#pragma unroll
+        for (int a = 0; a < 5; ++a) m.st[a] = A[(Q_S + a) * D.plane + n];
+        collide19_unit(L, rho, m, u, F, S, f);
+    } else {
+        collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
+    }
+    static_for<19>([&](auto icn) {
+        constexpr int i = decltype(icn)::value;
+        if (nbr_solid(nb, qz(i)))
+            fn[fofs(n) + qopp(i) * XB] = f[i];
+        else
+            fn[fofs((size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)))) + i * XB] = f[i];
+    });
+}
+
+template <class R, bool UNIT>
+__global__ void __launch_bounds__(128) k3_thermal(Dom3 D, Phys<R> P, Lat3<R> L) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -606,15 +669,11 @@ __global__ void __launch_bounds__(128) k3_collide(Dom3 D, Phys<R> P, Lat3<R> L) 
     const long long step = __ldcg(&D.ctl->step);
     const int par = (int)(step & 1);
     const size_t n = nid<R>(D, x, y, z);
-    const R* fc = (const R*)D.f[par] + fofs(n);
-    R* fn = (R*)D.f[par ^ 1];
     const R* gc = (const R*)D.g[par];
     R* gn = (R*)D.g[par ^ 1];
     const R* A = (const R*)D.aux;
     const R rho = A[Q_RHO * D.plane + n] + L.rho_ref;
     const R u[3] = {A[Q_UX * D.plane + n], A[Q_UY * D.plane + n], A[Q_UZ * D.plane + n]};
-    const R F[3] = {A[Q_FX * D.plane + n], A[Q_FY * D.plane + n], A[Q_FZ * D.plane + n]};
-    const R S = A[Q_F2 * D.plane + n];
     const size_t gno = gofs(n);
     R g[7];
 #pragma unroll
@@ -636,30 +695,6 @@ __global__ void __launch_bounds__(128) k3_collide(Dom3 D, Phys<R> P, Lat3<R> L) 
     const R Pn = thermal7<UNIT>(L, g, C, A[Q_E * D.plane + n], u[0], u[1], u[2], R(2) * dva + dvd,
                                 ((const R*)D.P[par])[n], step == 0, gs);
     ((R*)D.P[par ^ 1])[n] = Pn;
-
-    // ---- D3Q19 MRT collision, pushed to x + c_i (bounce-back through walls)
-    R f[19];
-#pragma unroll
-    for (int i = 0; i < 19; ++i) f[i] = fc[i * XB];
-    if (L.frozen_flow) {
-#pragma unroll
-        for (int i = 0; i < 19; ++i) fn[fofs(n) + i * XB] = f[i];
-    } else {
-        if constexpr (UNIT) {
-            Mom3<R> m;
-            moments3<true>(f, m);
-            collide19_unit(L, rho, m, u, F, S, f);
-        } else {
-            collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
-        }
-        static_for<19>([&](auto icn) {
-            constexpr int i = decltype(icn)::value;
-            if (nbr_solid(nb, qz(i)))
-                fn[fofs(n) + qopp(i) * XB] = f[i];
-            else
-                fn[fofs((size_t)((long long)n + nbr_off(nb, qx(i), qy(i), qz(i)))) + i * XB] = f[i];
-        });
-    }
 
     // weighted streaming (Eq. 39) from this node's side: g*_i lands on
     // x = y + c_i as g_i(x) + (g*_i - g_i(x)) / (rho(x) c_v), with g_i(x)
@@ -723,10 +758,10 @@ __device__ __forceinline__ void add_mass(const Dom3& D, double v, int slot) {
 
 // Fields of the current state from its populations, into the planes, with
 // its density sum into slot step % 3 for buoyancy.  want: W_STRESS the stress
-// moments (for k3_march at unit rates), W_IC 1/(rho c_v) (k3_collide), W_T the
+// moments (which the collision at unit rates takes), W_T the
 // temperature everywhere (else only next to the walls, for the ghost layer).
 // Bound by its traffic, 26 populations read and 6 to 11 fields written.
-enum { W_STRESS = 1, W_IC = 2, W_T = 4 };
+enum { W_STRESS = 1, W_T = 2 };
 template <class R>
 __global__ void __launch_bounds__(128) k3_macro(Dom3 D, Phys<R> P, Lat3<R> L, int use_mass, int want) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -760,7 +795,6 @@ __global__ void __launch_bounds__(128) k3_macro(Dom3 D, Phys<R> P, Lat3<R> L, in
 #pragma unroll
             for (int a = 0; a < 5; ++a) A[(Q_S + a) * D.plane] = m.st[a];
         }
-        if (want & W_IC) A[Q_IC * D.plane] = o.ic;
         if ((want & W_T) || (D.walls && (z == 0 || z == D.nz - 1))) A[Q_T * D.plane] = o.T;
         if (err) atomicOr(&D.ctl->err, err);
         if (use_mass) msum = (double)o.rho;
@@ -1283,7 +1317,7 @@ void launch_fields(lbm3d_ctx* c, int what) {
     const Phys<R> P = make_phys<R>(phys_of(c->params));
     const Lat3<R> L = make_lat3<R>(c->params, c->D);
     k3_macro<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0, W_T);
-    k3_force<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L, 0);
+    k3_force<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, P, L);
     k3_export<R><<<grd3(c), blk3(), 0, c->stream>>>(c->D, L, what, c->host_buf);
 }
 
@@ -1293,10 +1327,15 @@ int launch_step(lbm3d_ctx* c) {
     Phys<R> P = make_phys<R>(phys_of(c->params));
     Lat3<R> L = make_lat3<R>(c->params, c->D);
     const dim3 b = blk3(), g = grd3(c);
-    k3_macro<R><<<g, b, 0, c->stream>>>(c->D, P, L, c->params.gravity != 0.0, W_IC);
-    k3_force<R><<<g, b, 0, c->stream>>>(c->D, P, L, 1);
-    if (unit3(c)) k3_collide<R, true><<<g, b, 0, c->stream>>>(c->D, P, L);
-    else k3_collide<R, false><<<g, b, 0, c->stream>>>(c->D, P, L);
+    const bool unit = unit3(c);
+    k3_macro<R><<<g, b, 0, c->stream>>>(c->D, P, L, c->params.gravity != 0.0, unit ? W_STRESS : 0);
+    if (unit) {
+        k3_flow<R, true><<<g, b, 0, c->stream>>>(c->D, P, L);
+        k3_thermal<R, true><<<g, b, 0, c->stream>>>(c->D, P, L);
+    } else {
+        k3_flow<R, false><<<g, b, 0, c->stream>>>(c->D, P, L);
+        k3_thermal<R, false><<<g, b, 0, c->stream>>>(c->D, P, L);
+    }
     k3_advance<<<1, 1, 0, c->stream>>>(c->ctl, massq_scale(c->D.inv_n));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -1414,7 +1453,7 @@ int lbm3d_create(int nx, int ny, int nz, const lbm_params* params, const lbm3d_b
     c->zseg = auto_zseg(nx, ny, nz, prec);
     // the marching step is the faster in FP32 (64^3 23.4 against 25.6 us, 256^3
     // 988 against 1429); in FP64, bound by the FP64 pipe, its one CTA per SM
-    // keeps that pipe less busy (96^3 757 against 601 us)
+    // keeps that pipe less busy (96^3 609 against 540 us)
     c->fused = prec == LBM_FP32;
     auto smem = [&](auto kernel, size_t bytes) {
         if (e == cudaSuccess)
