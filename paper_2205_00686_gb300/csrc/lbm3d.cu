@@ -26,9 +26,9 @@
 //
 // At unit rates (s_e = s_eps = s_q = 1 and varsigma_3 = varsigma_4 = 1, the
 // paper's setting) the collision needs of f only rho, j and the five stress
-// moments (collide19_unit): about 310 operations per node and step instead
+// moments (collide19_unit): about 300 operations per node and step instead
 // of 770, which is what bounds the FP64 step, and no moment matrices (96^3
-// FP64 in the step over nodes: 1080 -> 540 us).
+// FP64 in the step over nodes: 1080 -> 514 us).
 #include <math.h>
 #include <string.h>
 
@@ -209,9 +209,9 @@ struct Lat3 {
     R s_e, s_eps, s_q, s_p;
     R sig_e3;            // (19/2) sigma / (1/s_e - 1/2), the sigma term of e
     R vs0, vs1, vs3, vs4, w7_0, w7_1, cs2h, cv, inv_cv, gravity;
-    // unit rates: 1 - s_p, 2 - s_p; the sigma term's factors of |12 s|^2 in the
+    // unit rates: 1 - s_p, a quarter of it, 2 - s_p/2; the sigma term's factors of |12 s|^2 in the
     // axis and diagonal populations; (1 - vs1)/2; vs1 / cs2h
-    R c_m, c_f, h_ax, h_dg, h_m, vs1_cs2h;
+    R c_m, c_m4, c_w, h_ax, h_dg, h_m, vs1_cs2h;
     R rho_ref, T_ref;
     R tw2[2];            // 2 w^_i (T_wall - T_ref) of the bottom and the top
     int frozen_flow, frozen_thermal;
@@ -227,7 +227,8 @@ Lat3<R> make_lat3(const lbm_params& p, const Dom3& D) {
     L.s_p = (R)s_p;
     L.sig_e3 = (R)(9.5 * p.sigma / (1.0 / p.s_e - 0.5));
     L.c_m = (R)(1.0 - s_p);
-    L.c_f = (R)(2.0 - s_p);
+    L.c_m4 = (R)(0.25 * (1.0 - s_p));
+    L.c_w = (R)(2.0 - 0.5 * s_p);
     {
         // half the sigma source of e, as a factor of |12 s|^2 = 144 |F_m|^2 / (G psi)^2,
         // times the row entries over the row's norm
@@ -323,34 +324,38 @@ __device__ __forceinline__ void moments3(const R* f, Mom3<R>& m) {
 // equilibrium + F/2).  The rest population is what the others leave of rho and
 // 1/6 is rounded down, 1/12 up, so that 2/6 + 8/12 is 1: with each weight
 // rounded by itself mass and momentum grow by 3e-8 a step in FP32 (256^3 after
-// 100 steps: fields 1.4e-6 off the FP64 ones).
+// 100 steps: fields 1.4e-6 off the FP64 ones).  With the products with u grouped
+// as below and E without a reciprocal of its own the step has 16 operations fewer
+// than with each moment by itself (96^3 FP64 540 -> 514 us).
 template <class R>
-__device__ __forceinline__ void collide19_unit(const Lat3<R>& L, R rho, const Mom3<R>& m, const R* u,
+__device__ __forceinline__ void collide19_unit(const Lat3<R>& L, const Mom3<R>& m, const R* u,
                                                const R* F, R S, R* f) {
-    const R rx = rho * u[0], ry = rho * u[1], rz = rho * u[2];
-    const R exx = rx * u[0], eyy = ry * u[1], ezz = rz * u[2];
-    const R fxx = u[0] * F[0], fyy = u[1] * F[1], fzz = u[2] * F[2];
-    const R eyz = eyy + ezz, fyz = fyy + fzz;
-    const R K = (exx + eyz) + (fxx + fyz);
-    // equilibrium and force of 3p_xx (half: the force row is 2 axx) and p_ww
-    const R pxx = R(2) * exx - eyz, axx = R(2) * fxx - fyz;
-    const R pww = eyy - ezz, aww = fyy - fzz;
-    const R n9 = L.c_m * m.st[0] + (L.s_p * pxx + L.c_f * axx);
-    const R n11 = L.c_m * m.st[1] + (L.s_p * pww + L.c_f * aww);
-    const R hf = R(0.5) * L.c_f;
-    const R n13 = L.c_m * m.st[2] + (L.s_p * (rx * u[1]) + hf * (u[0] * F[1] + u[1] * F[0]));
-    const R n14 = L.c_m * m.st[3] + (L.s_p * (ry * u[2]) + hf * (u[1] * F[2] + u[2] * F[1]));
-    const R n15 = L.c_m * m.st[4] + (L.s_p * (rx * u[2]) + hf * (u[0] * F[2] + u[2] * F[0]));
-    // stress parts: a = N/36 (or N/12), b = (m^eq + F/2)/72 (or /24)
-    const R b9 = (pxx + axx) * R(1.0 / 72.0), b11 = (pww + aww) * R(1.0 / 24.0);
-    const R pa = n9 * R(1.0 / 36.0) + b9, pd = n9 * R(1.0 / 36.0) - R(0.5) * b9;
-    const R qa = n11 * R(1.0 / 12.0) + b11, qd = n11 * R(1.0 / 12.0) - R(0.5) * b11;
+    // equilibrium + force as products with u (rho u = j + F/2): g = u_a (rho u + F)_a
+    // gives K and m^eq + F/2 of 3p_xx and p_ww (their force rows are twice u_a F_a's),
+    // w = s_p rho u + (2 - s_p) F the relaxed stresses
+    const R gx = u[0] * (m.j[0] + R(1.5) * F[0]), gy = u[1] * (m.j[1] + R(1.5) * F[1]),
+            gz = u[2] * (m.j[2] + R(1.5) * F[2]);
+    const R gyz = gy + gz, K = gx + gyz;
+    const R pxx = R(2) * gx - gyz, pww = gy - gz;
+    const R wx = L.s_p * m.j[0] + L.c_w * F[0], wy = L.s_p * m.j[1] + L.c_w * F[1],
+            wz = L.s_p * m.j[2] + L.c_w * F[2];
+    const R ty = u[1] * wy, tz = u[2] * wz;
+    const R n9 = L.c_m * m.st[0] + (R(2) * (u[0] * wx) - (ty + tz));
+    const R n11 = L.c_m * m.st[1] + (ty - tz);
+    // N_ab / 4
+    const R q13 = L.c_m4 * m.st[2] + R(0.125) * (u[0] * wy + u[1] * wx);
+    const R q14 = L.c_m4 * m.st[3] + R(0.125) * (u[1] * wz + u[2] * wy);
+    const R q15 = L.c_m4 * m.st[4] + R(0.125) * (u[0] * wz + u[2] * wx);
+    // stress parts: N/36 (or N/12) and (m^eq + F/2)/72 (or /24)
+    const R p9 = n9 * R(1.0 / 36.0), p11 = n11 * R(1.0 / 12.0);
+    const R pa = pxx * R(1.0 / 72.0) + p9, pd = pxx * R(-1.0 / 144.0) + p9;
+    const R qa = pww * R(1.0 / 24.0) + p11, qd = pww * R(-1.0 / 48.0) + p11;
     const R ax = m.rhod * R(1.0 / 18.0) + L.h_ax * S;
     const R dg = m.rhod * R(1.0 / 36.0) + (K * R(1.0 / 24.0) + L.h_dg * S);
     const R jx = m.j[0] + F[0], jy = m.j[1] + F[1], jz = m.j[2] + F[2];
     const R a0 = ax + R(2) * pa, a1 = (ax - pa) + qa, a2 = (ax - pa) - qa;
     const R dxy = (dg + pd) + qd, dxz = (dg + pd) - qd, dyz = dg - R(2) * pd;
-    const R c6 = sizeof(R) == 4 ? R(0x1.555554p-3) : R(1.0 / 6.0), c12 = R(1.0 / 12.0), q = R(0.25);
+    const R c6 = sizeof(R) == 4 ? R(0x1.555554p-3) : R(1.0 / 6.0), c12 = R(1.0 / 12.0);
     f[0] = (m.rhod - R(6) * ax) - R(12) * dg;
     f[1] = a0 + c6 * jx;
     f[2] = a0 - c6 * jx;
@@ -358,8 +363,8 @@ __device__ __forceinline__ void collide19_unit(const Lat3<R>& L, R rho, const Mo
     f[4] = a1 - c6 * jy;
     f[5] = a2 + c6 * jz;
     f[6] = a2 - c6 * jz;
-    const R e7 = dxy + q * n13, e9 = dxy - q * n13, e11 = dxz + q * n15, e13 = dxz - q * n15;
-    const R e15 = dyz + q * n14, e17 = dyz - q * n14;
+    const R e7 = dxy + q13, e9 = dxy - q13, e11 = dxz + q15, e13 = dxz - q15;
+    const R e15 = dyz + q14, e17 = dyz - q14;
     const R o7 = jx + jy, o9 = jx - jy, o11 = jx + jz, o13 = jx - jz, o15 = jy + jz, o17 = jy - jz;
     f[7] = e7 + c12 * o7;
     f[8] = e7 - c12 * o7;
@@ -538,8 +543,8 @@ __device__ R psi_nb(const Dom3& D, const Phys<R>& P, int x, int y, int z, int* e
     const R dy = rho[nid<R>(D, x, wrapn(y + 1, D.ny), z1)] - rho[nid<R>(D, x, wrapn(y - 1, D.ny), z1)];
     const R rg = (rho[nid<R>(D, x, y, z2)] + (R)D.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy);
     const R tg = A[Q_T * D.plane + nid<R>(D, x, y, z1)];   // the fluid node's temperature
-    R q2, tdp;
-    eos_node(P, rg, tg, &q2, &tdp);
+    R q2, E;
+    eos_node(P, rg, tg, &q2, &E);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
     return f_sqrt(q2);
 }
@@ -647,7 +652,7 @@ __global__ void __launch_bounds__(128) k3_flow(Dom3 D, Phys<R> P, Lat3<R> L) {
     if constexpr (UNIT) {
 #pragma unroll
         for (int a = 0; a < 5; ++a) m.st[a] = A[(Q_S + a) * D.plane + n];
-        collide19_unit(L, rho, m, u, F, S, f);
+        collide19_unit(L, m, u, F, S, f);
     } else {
         collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
     }
@@ -725,20 +730,17 @@ __global__ void __launch_bounds__(128) k3_thermal(Dom3 D, Phys<R> P, Lat3<R> L) 
 // macroscopic fields of a node from its (deviation) populations
 template <class R>
 struct Fld3 {
-    R rho, T, psi, C, ic, E;
+    R rho, T, psi, E;
 };
 template <class R>
 __device__ __forceinline__ void fields3(const Phys<R>& P, const Lat3<R>& L, R rhod, R Td, Fld3<R>& o,
                                         int* err) {
     o.rho = rhod + L.rho_ref;
     o.T = Td + L.T_ref;
-    R q2, tdp;
-    eos_node(P, o.rho, o.T, &q2, &tdp);
+    R q2;
+    eos_node(P, o.rho, o.T, &q2, &o.E);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
     o.psi = f_sqrt(q2);
-    o.C = o.rho * L.cv;
-    o.ic = f_rcp(o.C);
-    o.E = tdp * (o.ic * R(1.0 / 12.0));
 }
 template <class R>
 __device__ __forceinline__ R sum7(const R* g) {
@@ -926,8 +928,8 @@ k3_march(const __grid_constant__ Dom3 D, const __grid_constant__ Phys<R> P, cons
         const R dx = rho[row + (x == D.nx - 1 ? 0 : x + 1)] - rho[row + (x == 0 ? D.nx - 1 : x - 1)];
         const R dy = rho[za + (size_t)(y == D.ny - 1 ? 0 : y + 1) * D.pitch + x] -
                      rho[za + (size_t)(y == 0 ? D.ny - 1 : y - 1) * D.pitch + x];
-        R q2, tdp;
-        eos_node(P, (rho[zb + n] + L.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy), A[Q_T * PL + za + n], &q2, &tdp);
+        R q2, E;
+        eos_node(P, (rho[zb + n] + L.rho_ref) + (R)D.cot * rsq(dx * dx + dy * dy), A[Q_T * PL + za + n], &q2, &E);
         if (!(q2 >= R(0))) err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
         return f_sqrt(q2);
     };
@@ -1117,7 +1119,7 @@ k3_march(const __grid_constant__ Dom3 D, const __grid_constant__ Phys<R> P, cons
                             for (int a = 0; a < 3; ++a) m.j[a] = b_o[1 + a];
 #pragma unroll
                             for (int a = 0; a < 5; ++a) m.st[a] = b_o[4 + a];
-                            collide19_unit(L, rho, m, u, F, S, f);
+                            collide19_unit(L, m, u, F, S, f);
                         } else {
                             collide19(L, rho, u, F, P.negG_12 * P.negG_12 * S, f);
                         }
@@ -1453,7 +1455,7 @@ int lbm3d_create(int nx, int ny, int nz, const lbm_params* params, const lbm3d_b
     c->zseg = auto_zseg(nx, ny, nz, prec);
     // the marching step is the faster in FP32 (64^3 23.4 against 25.6 us, 256^3
     // 988 against 1429); in FP64, bound by the FP64 pipe, its one CTA per SM
-    // keeps that pipe less busy (96^3 609 against 540 us)
+    // keeps that pipe less busy (96^3 583 against 514 us)
     c->fused = prec == LBM_FP32;
     auto smem = [&](auto kernel, size_t bytes) {
         if (e == cudaSuccess)

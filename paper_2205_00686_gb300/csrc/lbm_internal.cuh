@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 namespace lbm {
 
 // flow / thermal boundary kinds (same values as the public header)
@@ -91,17 +93,17 @@ struct Phys {
     // EOS: p = rho Rg T/(1 - b rho) - a h^2 rho^2/(1 + 2 b rho - b^2 rho^2),
     // h = 1 + kpr (1 - sqrt(T/Tc))
     R a, b, Rg, kpr, inv_Tc;
-    R one_p_kpr;
+    R k_sa, k1_sa, m_third;          // k sqrt(a), (1 + k) sqrt(a), -1/3: see eos_node
     R two_over_G, negG, negG_12;
     // D2Q9 MRT rates and Li forcing
     R s_e, s_eps, s_q, s_p;
     R hs_e, hs_eps, hs_q, hs_p;      // 1 - s/2
     R sig_e, sig_eps;                // sigma / (1/s - 1/2)
     // unit rates: the collision's combined factors (collide9_unit)
-    R u_m, u_d, u_g7, u_g8;          // (1 - s_p)/4, s_p/4, hs_p/2, hs_p/4
-    R u_ax, u_dg;                    // the sigma terms' factors of |12 s|^2
+    R u_m, u_d, u_w;                 // (1 - s_p)/4, s_p/4, 1/2 - s_p/8
+    R u_ax, u_dg, u_0;               // the sigma terms' factors of |12 s|^2
     // D2Q5
-    R cv, inv_cv, w_dot, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
+    R cv, inv_cv, inv_12cv, w_dot, w5_0, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
     R h_m, one_m_vs4;               // h_m = (1 - vs1) / 2
     R gravity;
     int frozen_flow, frozen_thermal;
@@ -122,11 +124,15 @@ inline Phys<R> make_phys(const PhysD& d) {
     double Tc = 0.0778 * d.a / (0.45724 * d.b * d.Rg);
     p.a = (R)d.a;
     p.b = (R)d.b;
-    p.Rg = (R)d.Rg;
+    p.Rg = (R)(d.a < 0 ? -d.Rg : d.Rg);
     p.kpr = (R)kpr;
     p.inv_Tc = (R)(1.0 / Tc);
-    p.one_p_kpr = (R)(1.0 + kpr);
-    p.two_over_G = (R)(2.0 / d.G);
+    // eos_node works with |a| and p times the sign of a
+    const double sgn = d.a < 0 ? -1.0 : 1.0, sa = std::sqrt(std::fabs(d.a));
+    p.k_sa = (R)(kpr * sa);
+    p.k1_sa = (R)((1.0 + kpr) * sa);
+    p.m_third = (R)(-sgn / 3.0);
+    p.two_over_G = (R)(sgn * 2.0 / d.G);
     p.negG = (R)(-d.G);
     p.negG_12 = (R)(-d.G / 12.0);
     p.s_e = (R)d.s_e;
@@ -141,8 +147,7 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.sig_eps = (R)(d.sigma / (1.0 / d.s_eps - 0.5));
     p.u_m = (R)(0.25 * (1.0 - d.s_p));
     p.u_d = (R)(0.25 * d.s_p);
-    p.u_g7 = (R)(0.5 * (1.0 - 0.5 * d.s_p));
-    p.u_g8 = (R)(0.25 * (1.0 - 0.5 * d.s_p));
+    p.u_w = (R)(0.5 - 0.125 * d.s_p);
     {
         // |F_m|^2 / psi^2 = G^2 |12 s|^2 / 144; e and epsilon get +-half of
         // sigma / (1/s - 1/2) times it (s_e = s_eps = 1)
@@ -150,10 +155,13 @@ inline Phys<R> make_phys(const PhysD& d) {
                      sp = 0.5 * d.sigma / (1.0 / d.s_eps - 0.5);
         p.u_ax = (R)(k * (2.0 * sp - se) / 36.0);
         p.u_dg = (R)(k * (2.0 * se - sp) / 36.0);
+        p.u_0 = (R)(-k * (se + sp) / 9.0);
     }
     p.cv = (R)d.cv;
     p.inv_cv = (R)(1.0 / d.cv);
+    p.inv_12cv = (R)(sgn / (12.0 * d.cv));
     p.w_dot = (R)d.w_dot;
+    p.w5_0 = (R)(1.0 - d.w_dot);
     p.w5_1 = (R)(0.25 * d.w_dot);
     p.vs1_cs2h = (R)(d.vs1 / (0.5 * d.w_dot));
     p.vs3 = (R)d.vs3;
@@ -208,10 +216,12 @@ __device__ __forceinline__ float f_rcp(float x) {
 // is left out is of order e^3 ~ 2^-60, below the FP64 rounding, so the result
 // is within about one ulp (not always the correctly rounded value).  Three
 // and five FP64 instructions, against four for two Newton-Raphson steps and
-// about ten for the IEEE square root.  With the node arithmetic of lbm_node.cuh, which count FP64 operations the
-// same way (about 168 per node instead of 220), the FP64 step on 1999 x 1501
-// went from 1.355 to 1.067 ms; in FP32 the same forms took the 4096^2 step
-// from 340.3 to 336.1 us.  A zero, infinite or NaN reciprocal
+// about ten for the IEEE square root.  With the node arithmetic of
+// lbm_node.cuh, which counts FP64 operations the same way (about 162 per node
+// instead of 220), the FP64 step on 1999 x 1501 went from 1.355 to 1.043 ms; in
+// FP32 the same forms took the 4096^2 step from 340.3 to 334.4 us.  (With the
+// IEEE operations instead the fields' distance from the FP64 oracle's is the
+// same, 2.3e-15 on 1999 x 1501.)  A zero, infinite or NaN reciprocal
 // operand gives a non-finite result, which the step reports; a square-root
 // operand outside the normal range (zero, negative, NaN among them) takes
 // the IEEE square root.

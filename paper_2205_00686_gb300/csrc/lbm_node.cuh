@@ -49,24 +49,25 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b) {
 }
 __device__ __forceinline__ double2 psub(double2 a, double2 b) { return pr(rsub(a.x, b.x), rsub(a.y, b.y)); }
 
-// psi^2 and T (dp/dT)_rho of one node, with D1 = 1 - b rho and
-// D2 = 1 + 2 b rho - b^2 rho^2 = 2 - D1^2 over one common reciprocal:
+// psi^2 and E = T (dp/dT)_rho / (12 rho c_v) of one node, with D1 = 1 - b rho
+// and D2 = 1 + 2 b rho - b^2 rho^2 = 2 - D1^2 over one common reciprocal:
 //   p = rho (Rg T D2 - a h^2 rho D1) / (D1 D2)
 //   T (dp/dT)_rho = rho (Rg T D2 + a k h sqrt(T/Tc) rho D1) / (D1 D2)
-// (T / sqrt(T/Tc) = Tc sqrt(T/Tc), so no second reciprocal).  One square
-// root and one reciprocal, 20 other operations.
+// (T / sqrt(T/Tc) = Tc sqrt(T/Tc), so no second reciprocal, and E needs none of
+// rho).  One square root and one reciprocal, 18 other operations with sqrt(a)
+// taken into h.  (For a < 0, which needs R < 0, p and the constants that meet it
+// carry the other sign.)
 template <class R>
-__device__ __forceinline__ void eos_node(const Phys<R>& P, R rho, R T, R* psi2, R* TdpdT) {
+__device__ __forceinline__ void eos_node(const Phys<R>& P, R rho, R T, R* psi2, R* E) {
     const R st = f_sqrt(rmul(T, P.inv_Tc));
-    const R h = rfma(-P.kpr, st, P.one_p_kpr);
-    const R ah = rmul(P.a, h);
+    const R h = rfma(-P.k_sa, st, P.k1_sa);      // sqrt(a) h
     const R d1 = rfma(-P.b, rho, R(1));
     const R d2 = rfma(-d1, d1, R(2));
-    const R s = rmul(rho, f_rcp(rmul(d1, d2)));
+    const R rc = f_rcp(rmul(d1, d2));
     const R u = rmul(rmul(P.Rg, T), d2), w = rmul(rho, d1);
-    const R p = rmul(s, rfma(-rmul(ah, h), w, u));
-    *psi2 = rmul(P.two_over_G, rfma(rho, R(-1.0 / 3.0), p));
-    *TdpdT = rmul(s, rfma(rmul(rmul(P.kpr, ah), st), w, u));
+    const R p = rmul(rmul(rho, rc), rfma(-rmul(h, h), w, u));
+    *psi2 = rmul(P.two_over_G, rfma(rho, P.m_third, p));
+    *E = rmul(rmul(P.inv_12cv, rc), rfma(rmul(rmul(P.k_sa, st), h), w, u));
 }
 
 // What the later stages take of a node's populations and EOS
@@ -122,12 +123,10 @@ __device__ __forceinline__ void node_fields(const Phys<R>& P, R rho_ref, R T_ref
     n.jy = radd(dA.y, radd(dB.x, dB.y));    // (f2 - f4) + (f5 - f7) + (f6 - f8)
     n.m7 = rsub(sA.x, sA.y);
     n.m8 = rsub(sB.x, sB.y);
-    R tdp;
-    eos_node(P, n.rho, n.T, &n.q2, &tdp);
+    eos_node(P, n.rho, n.T, &n.q2, &n.E);
     n.psi = f_sqrt(n.q2);
     n.C = rmul(n.rho, P.cv);
     n.iC = rmul(n.ir, P.inv_cv);
-    n.E = rmul(tdp, rmul(n.iC, R(1.0 / 12.0)));
 }
 
 // ghost-layer psi of a wall (Section 3.3): rho_ghost = rho(layer 2) +
@@ -137,8 +136,8 @@ template <class R>
 __device__ __forceinline__ R ghost_psi(const Phys<R>& P, R rho_far, R rho_p, R rho_m, R cot, R Tg,
                                        int* err) {
     const R rg = rfma(cot, rabs(rsub(rho_p, rho_m)), rho_far);
-    R q2, tdp;
-    eos_node(P, rg, Tg, &q2, &tdp);
+    R q2, E;
+    eos_node(P, rg, Tg, &q2, &E);
     if (!(q2 >= R(0))) *err |= (q2 != q2) ? ERR_NONFINITE : ERR_PSI;
     return f_sqrt(q2);
 }
@@ -158,7 +157,8 @@ __device__ __forceinline__ typename Vec2<R>::T force_of(const Phys<R>& P, typena
                                                         R psi, R rho, R rho_ave) {
     const R gp = rmul(P.negG_12, psi);
     typename Vec2<R>::T F = pmul(pr(gp, gp), s12);
-    F.y = rfma(-P.gravity, rsub(rho, rho_ave), F.y);
+    // (without gravity FP64 spares its two operations)
+    if (sizeof(R) == 4 || P.gravity != R(0)) F.y = rfma(-P.gravity, rsub(rho, rho_ave), F.y);
     return F;
 }
 
@@ -178,21 +178,22 @@ __device__ __forceinline__ R2 velocity(R2 F, R2 j, R ir) {
 //                   +- ((j + F)_x +- (j + F)_y)/12
 // With f*_0 as the remainder and the float 1/12 rounded down, so that 2/3 + 4/12
 // is 1, mass and momentum are kept to the rounding of the populations (each
-// weight rounded by itself adds 3e-8 of them every step in FP32).
-// rhod: deviation of rho from the storage reference (f is stored as
-// deviations); rho: the density itself.
+// weight rounded by itself adds 3e-8 of them every step in FP32).  In FP64, where
+// that is 1e-16, it is formed from its own weight as the oracle does (fields of
+// 1999 x 1501 after 10 steps 2.3e-15 off the oracle's, as remainder 2.8e-15).
+// With rho u = j + F/2 the products with u come in two groups: u_a (j + 3/2 F)_a
+// sums to K, and u_a w_b with w = s_p/4 rho u + (1 - s_p/2)/2 F is what the
+// stresses take.  rhod: deviation of rho from the storage reference (f is stored
+// as deviations).
 template <class R, class R2>
-__device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rho, R rhod, R2 j, R m7, R m8,
+__device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rhod, R2 j, R m7, R m8,
                                               R2 u, R2 F, R2 s12, R* f, int stride) {
-    const R2 ru = pmul(pr(rho, rho), u);
-    const R2 uu = pmul(ru, u);      // rho (ux^2, uy^2)
-    const R2 uF = pmul(u, F);       // (ux Fx, uy Fy)
-    const R2 K2 = padd(uu, uF);
-    const R K = radd(K2.x, K2.y);
+    const R2 v = pfma(F, pr(R(1.5), R(1.5)), j);
+    const R2 w = pfma(F, pr(P.u_w, P.u_w), pmul(j, pr(P.u_d, P.u_d)));
+    const R K = rfma(u.x, v.x, rmul(u.y, v.y));
     const R S = rfma(s12.x, s12.x, rmul(s12.y, s12.y));
-    const R b7 = rfma(P.u_m, m7, rfma(P.u_d, rsub(uu.x, uu.y), rmul(P.u_g7, rsub(uF.x, uF.y))));
-    const R b8 = rfma(P.u_m, m8, rfma(P.u_d, rmul(ru.x, u.y),
-                                      rmul(P.u_g8, rfma(u.x, F.y, rmul(u.y, F.x)))));
+    const R b7 = rfma(P.u_m, m7, rfma(u.x, w.x, -rmul(u.y, w.y)));
+    const R b8 = rfma(P.u_m, m8, rmul(R(0.5), rfma(u.x, w.y, rmul(u.y, w.x))));
     const R K12 = rmul(K, R(1.0 / 12.0));
     const R2 cc = pfma(pr(rhod, rhod), pr(R(1.0 / 9.0), R(1.0 / 36.0)),
                        pfma(pr(S, S), pr(P.u_ax, P.u_dg), pr(K12, K12)));
@@ -206,7 +207,8 @@ __device__ __forceinline__ void collide9_unit(const Phys<R>& P, R rho, R rhod, R
     const R2 t3 = pr(R(1.0 / 3.0), R(1.0 / 3.0)), t12 = pr(w12, w12);
     const R2 f12 = pfma(js, t3, cb), f58 = pfma(sd, t12, db);
     const R2 f34 = pnfma(js, t3, cb), f76 = pnfma(sd, t12, db);
-    f[0] = rfma(R(-4), radd(cc.x, cc.y), rhod);
+    f[0] = sizeof(R) == 4 ? rfma(R(-4), radd(cc.x, cc.y), rhod)
+                          : rfma(R(4.0 / 9.0), rhod, rfma(R(-2.0 / 3.0), K, rmul(P.u_0, S)));
     f[1 * stride] = f12.x;
     f[2 * stride] = f12.y;
     f[3 * stride] = f34.x;
@@ -296,7 +298,8 @@ __device__ __forceinline__ R thermal5(const Phys<R>& P, const R* g, R Td, R C, R
         // varsigma_3 = varsigma_4 = 1: m3* = w_dot (T + Q + S), m4* = 0
         const R TQ = rfma(C, dP, Td);
         const R a = rmul(P.w5_1, TQ);
-        gs[0] = rfma(R(-4), a, TQ);     // what the others leave of T
+        // FP32: what the others leave of T (see collide9_unit)
+        gs[0] = sizeof(R) == 4 ? rfma(R(-4), a, TQ) : rmul(P.w5_0, TQ);
         const R2 g12 = padd(pr(a, a), h12), g34 = psub(pr(a, a), h12);
         gs[1] = g12.x;
         gs[2] = g12.y;

@@ -783,7 +783,7 @@ struct Sweep {
                             for (int q = 0; q < 9; ++q) fsw[q * NT] = fp[q];
                         }
                     } else if (UNIT) {
-                        collide9_unit(P, rhop, rhodp, pr(jxp, jyp), m7p, m8p, uv, F, s12, fsw, NT);
+                        collide9_unit(P, rhodp, pr(jxp, jyp), m7p, m8p, uv, F, s12, fsw, NT);
                     } else {
                         collide9(P, rhop, rhodp, fp, uv, F, s12, fsw, NT);
                     }

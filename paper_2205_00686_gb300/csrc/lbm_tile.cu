@@ -290,7 +290,7 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
                 } else {
                     R fs[9];
                     if constexpr (UNIT)
-                        collide9_unit(P, no.rho, no.rhod, pr(no.jx, no.jy), no.m7, no.m8, u, F, s12, fs, 1);
+                        collide9_unit(P, no.rhod, pr(no.jx, no.jy), no.m7, no.m8, u, F, s12, fs, 1);
                     else
                         collide9(P, no.rho, no.rhod, fo, u, F, s12, fs, 1);
                     st_st(fw, (TF)fs[0]);
