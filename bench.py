@@ -464,7 +464,7 @@ def bench_3d(lbm, stream, torch, peak, n=256, steps=200, warmup=20, zseg=None):
             "ms_per_step": round(t / steps * 1e3, 4), "zseg": zseg, "zseg_tried_mlups": tried,
             "roofline": {"bound": "hbm", "achieved": round(ach, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(ach / peak, 4), "algorithmic_bytes_per_node": 216,
-                         "kernels": "k3_fused (+ k3_advance)"},
+                         "kernels": "k3_macro + k3_march"},
             "three_kernels": {"mlups": round(N * s3 / t3 / 1e6, 1), "steps": s3,
                               "hbm_frac_of_measured": round(ach3 / peak, 4),
                               "kernels": "k3_macro + k3_flow + k3_thermal (+ k3_advance)"},

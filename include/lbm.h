@@ -40,7 +40,7 @@ extern "C" {
 #define LBM_EIO (-6)         /* checkpoint file could not be read or written  */
 #define LBM_ESTATE (-7)      /* call out of order (e.g. step before init)     */
 #define LBM_ETOOBIG (-8)     /* size beyond a fixed capacity (no-alloc entry)  */
-#define LBM_ETIMEOUT (-9)    /* a bounded device wait ran out (staged rows)    */
+#define LBM_ETIMEOUT (-9)    /* a bounded device wait ran out: staged row, grid barrier */
 
 /* ---- precision of storage and arithmetic ------------------------------- */
 typedef enum {

@@ -1453,8 +1453,8 @@ int lbm3d_create(int nx, int ny, int nz, const lbm_params* params, const lbm3d_b
     D.T_ref = 0.0;
     D.inv_n = 1.0 / ((double)nx * ny * nz);
     c->zseg = auto_zseg(nx, ny, nz, prec);
-    // the marching step is the faster in FP32 (64^3 23.4 against 25.6 us, 256^3
-    // 988 against 1429); in FP64, bound by the FP64 pipe, its one CTA per SM
+    // the marching step is the faster in FP32 (72 x 50 x 61 34.5 against 36.6 us,
+    // 128^3 136 against 162, 256^3 983 against 1256); in FP64, bound by the FP64 pipe, its one CTA per SM
     // keeps that pipe less busy (96^3 583 against 514 us)
     c->fused = prec == LBM_FP32;
     auto smem = [&](auto kernel, size_t bytes) {

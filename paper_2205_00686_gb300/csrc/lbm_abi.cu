@@ -392,7 +392,7 @@ static int ctx_check(lbm_ctx* c) {
     if (rc) return rc;
     if (h.err && c->sticky == LBM_OK) {
         c->sticky = map_device_err(h.err);
-        c->err = c->sticky == LBM_ETIMEOUT ? "a bounded wait for a staged row ran out"
+        c->err = c->sticky == LBM_ETIMEOUT ? "a bounded wait for a staged row or the grid barrier ran out"
                  : c->sticky == LBM_EPSI ? "psi^2 < 0 at some node (density above the EOS range)"
                                          : "non-finite density or temperature";
     }
