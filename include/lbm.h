@@ -374,9 +374,14 @@ int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged)
  * runs up to 1024 steps in one cooperative launch over tiles of nodes.  The
  * state is bit for bit the sweep's (with buoyancy, up to the rounding of the
  * density sum).  lbm_set_tile and lbm_set_staging select the sweep,
- * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile. */
+ * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile.  Where
+ * the cooperative launch is refused (a process or stream that may use only part
+ * of the SMs), the context takes the sweep from that step on.
+ * lbm_get_small_form: the tile (tx x ty nodes), tiles and CTAs per launch of the
+ * form lbm_step takes next; all 0 when it is the sweep. */
 int lbm_set_tile(lbm_ctx* ctx, int threads, int rows);
 int lbm_get_tile(const lbm_ctx* ctx, int* threads, int* rows);
+int lbm_get_small_form(const lbm_ctx* ctx, int* tx, int* ty, int* tiles, int* grid);
 int lbm_autotune(lbm_ctx* ctx, int steps_per_trial);
 
 /* Load path of the fused FP32 / FP32_G16 step (no counterpart in the paper, which
@@ -408,7 +413,8 @@ int lbm_get_staging(const lbm_ctx* ctx);
  * records LBM_ETIMEOUT in the sticky error word.  The row pipeline keeps its
  * own waits, so the step's results are unchanged and no copy is left in
  * flight; the GPU is never faulted.  No effect on the register-prefetch path
- * or on batches.  Returns LBM_EINVAL for NULL, LBM_ESTATE in a batch. */
+ * or on batches.  on = 2: the cooperative launches of the small-domain form are
+ * answered as if the device had refused them (nothing is launched).  Returns LBM_EINVAL for NULL, LBM_ESTATE in a batch. */
 int lbm_set_wait_probe(lbm_ctx* ctx, int on);
 
 /* ---- diagnostics without any allocation -------------------------------- *

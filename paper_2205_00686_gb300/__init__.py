@@ -40,7 +40,7 @@ ABI_FUNCTIONS = (
     "lbm_batch_create", "lbm_batch_attach", "lbm_batch_detach", "lbm_batch_size",
     "lbm_batch_step", "lbm_batch_sync", "lbm_batch_destroy", "lbm_batch_autotune",
     "lbm_batch_errors_async",
-    "lbm_batch_get_tile", "lbm_set_tile", "lbm_get_tile",
+    "lbm_batch_get_tile", "lbm_set_tile", "lbm_get_tile", "lbm_get_small_form",
     "lbm_autotune", "lbm_set_staging", "lbm_get_staging", "lbm_set_wait_probe",
     "lbm_diag_reduce_noalloc", "lbm_reconfigure", "lbm_contact_angle",
     "lbm_regions", "lbm_rows_bytes", "lbm_pack_rows", "lbm_unpack_rows", "lbm_set_partition",
@@ -146,6 +146,7 @@ def lib():
             "lbm_set_tile": ([_vp, ctypes.c_int, ctypes.c_int], ctypes.c_int),
             "lbm_get_tile": ([_vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)],
                              ctypes.c_int),
+            "lbm_get_small_form": ([_vp] + [ctypes.POINTER(ctypes.c_int)] * 4, ctypes.c_int),
             "lbm_autotune": ([_vp, ctypes.c_int], ctypes.c_int),
             "lbm_set_staging": ([_vp, ctypes.c_int], ctypes.c_int),
             "lbm_get_staging": ([_vp], ctypes.c_int),
@@ -325,6 +326,13 @@ class Domain:
         lib().lbm_get_tile(self._h, ctypes.byref(t), ctypes.byref(r))
         return t.value, r.value
 
+    def small_form(self):
+        """(tx, ty, tiles, CTAs) of the small-domain form step() takes next,
+        zeros when it is the sweep; see lbm_get_small_form."""
+        v = [ctypes.c_int() for _ in range(4)]
+        _check(lib().lbm_get_small_form(self._h, *[ctypes.byref(x) for x in v]), self._h)
+        return tuple(x.value for x in v)
+
     def autotune(self, steps_per_trial: int = 10):
         _check(lib().lbm_autotune(self._h, steps_per_trial), self._h)
         return self.tile()
@@ -339,10 +347,11 @@ class Domain:
     def staged(self, on: bool):
         _check(lib().lbm_set_staging(self._h, 1 if on else 0), self._h)
 
-    def set_wait_probe(self, on: bool):
-        """Test hook: staged launches also wait on an mbarrier nothing arms,
-        so each CTA's bounded wait runs out and LBM_ETIMEOUT is reported."""
-        _check(lib().lbm_set_wait_probe(self._h, 1 if on else 0), self._h)
+    def set_wait_probe(self, on: int):
+        """Test hook: with 1 (True) staged launches also wait on an mbarrier
+        nothing arms, so each CTA's bounded wait runs out and LBM_ETIMEOUT is
+        reported; with 2 cooperative launches are answered as refused."""
+        _check(lib().lbm_set_wait_probe(self._h, int(on)), self._h)
 
     @property
     def last_error(self) -> str:

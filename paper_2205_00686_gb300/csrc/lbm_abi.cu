@@ -327,7 +327,7 @@ static StepLaunch ctx_launch(const lbm_ctx* c) {
     L.grid = c->grid;
     L.walls = has_walls(c->inst) ? 1 : 0;
     L.staged = c->staged;
-    L.wait_probe = c->wait_probe;
+    L.wait_probe = c->wait_probe == 1 ? 1 : 0;
     L.targets = c->target > 0 ? 1 : 0;
     L.phys = c->phys;
     return L;
@@ -361,7 +361,10 @@ static int enqueue_steps(cudaStream_t st, cudaGraphExec_t* graph, const StepLaun
     return LBM_OK;
 }
 
-// queues n steps of the small-domain form
+// Queues n steps of the small-domain form.  Its grid is made for all SMs of the
+// device and has to be resident at once, so a launch is refused where the
+// process or the stream may use fewer of them (an MPS share, a green context);
+// the context then goes on with the sweep, from the step it has reached.
 static int enqueue_tiled(lbm_ctx* c, int n) {
     TileLaunch L;
     L.inst = c->inst;
@@ -374,8 +377,16 @@ static int enqueue_tiled(lbm_ctx* c, int n) {
     L.targets = c->target > 0 ? 1 : 0;
     for (; n > 0; n -= L.steps) {
         L.steps = std::min(n, kTileSteps);
-        if (tile_launch(c->prec, c->tile, L, c->phys, c->stream))
-            return cuda_err(c, cudaGetLastError(), "step launch");
+        // (one step has no barrier and is launched without that condition)
+        const cudaError_t e = c->wait_probe == 2 && L.steps > 1
+                                  ? cudaErrorCooperativeLaunchTooLarge
+                                  : tile_launch(c->prec, c->tile, L, c->phys, c->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+            e == cudaErrorNotSupported) {
+            c->tiled = false;
+            return enqueue_steps(c->stream, &c->graph, ctx_launch(c), c->prec, c->threads, n, c);
+        }
+        if (e != cudaSuccess) return cuda_err(c, e, "step launch");
     }
     return LBM_OK;
 }
@@ -1130,7 +1141,7 @@ int lbm_get_staging(const lbm_ctx* c) { return c ? c->staged : LBM_EINVAL; }
 int lbm_set_wait_probe(lbm_ctx* c, int on) {
     if (!c) return LBM_EINVAL;
     if (c->batch) return set_err(c, LBM_ESTATE, "context is attached to a batch");
-    c->wait_probe = on ? 1 : 0;
+    c->wait_probe = on == 2 ? 2 : (on ? 1 : 0);
     drop_graph(&c->graph);
     return LBM_OK;
 }
@@ -1139,6 +1150,15 @@ int lbm_get_tile(const lbm_ctx* c, int* threads, int* rows) {
     if (!c) return LBM_EINVAL;
     if (threads) *threads = c->threads;
     if (rows) *rows = c->rows;
+    return LBM_OK;
+}
+
+int lbm_get_small_form(const lbm_ctx* c, int* tx, int* ty, int* tiles, int* grid) {
+    if (!c) return LBM_EINVAL;
+    if (tx) *tx = c->tiled ? c->tile.tx : 0;
+    if (ty) *ty = c->tiled ? c->tile.ty : 0;
+    if (tiles) *tiles = c->tiled ? c->tile.n_tiles : 0;
+    if (grid) *grid = c->tiled ? c->tile.grid : 0;
     return LBM_OK;
 }
 

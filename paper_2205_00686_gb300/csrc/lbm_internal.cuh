@@ -308,7 +308,8 @@ struct TileLaunch {
     int targets;       // the domain has a target step (lbm_set_target)
 };
 int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out);
-int tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys, cudaStream_t st);
+cudaError_t tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys,
+                        cudaStream_t st);
 
 // The unit-rate form applies when every non-hydrodynamic rate is exactly 1
 // (s_e = s_eps = s_q = 1 and varsigma_3 = varsigma_4 = 1, the paper's choice).

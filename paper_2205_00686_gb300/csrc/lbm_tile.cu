@@ -451,7 +451,8 @@ int tile_occ(int threads, size_t smem, int* ctas) {
 }
 
 template <int PREC, bool UNIT>
-int tile_run(const TileLaunch& L, const PhysD& phys, int grid, int threads, size_t smem, cudaStream_t st) {
+cudaError_t tile_run(const TileLaunch& L, const PhysD& phys, int grid, int threads, size_t smem,
+                     cudaStream_t st) {
     Phys<typename Types<PREC>::R> P = make_phys<typename Types<PREC>::R>(phys);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -463,7 +464,9 @@ int tile_run(const TileLaunch& L, const PhysD& phys, int grid, int threads, size
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = L.steps > 1 ? 1 : 0;   // one step has no barrier
-    return cudaLaunchKernelEx(&cfg, k_tile<PREC, UNIT>, L, P) == cudaSuccess ? 0 : -1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_tile<PREC, UNIT>, L, P);
+    if (e != cudaSuccess) cudaGetLastError();   // the caller answers it
+    return e;
 }
 
 template <int PREC>
@@ -472,8 +475,8 @@ int tile_occ_any(const PhysD& phys, int threads, size_t smem, int* ctas) {
                             : tile_occ<PREC, false>(threads, smem, ctas);
 }
 template <int PREC>
-int tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int threads, size_t smem,
-                 cudaStream_t st) {
+cudaError_t tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int threads, size_t smem,
+                         cudaStream_t st) {
     return unit_rates(phys) ? tile_run<PREC, true>(L, phys, grid, threads, smem, st)
                             : tile_run<PREC, false>(L, phys, grid, threads, smem, st);
 }
@@ -561,7 +564,8 @@ int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out
     return 0;
 }
 
-int tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys, cudaStream_t st) {
+cudaError_t tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys,
+                        cudaStream_t st) {
     if (prec == 0) return tile_run_any<0>(L, phys, T.grid, T.threads, T.smem, st);
     if (prec == 1) return tile_run_any<1>(L, phys, T.grid, T.threads, T.smem, st);
     return tile_run_any<2>(L, phys, T.grid, T.threads, T.smem, st);

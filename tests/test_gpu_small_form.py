@@ -1,0 +1,39 @@
+"""Choice and failure paths of the small-domain form of the step."""
+import numpy as np
+import pytest
+
+import parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64", "fp32_g16"])
+def test_refused_cooperative_launch_goes_on_with_the_sweep(prec):
+    """A device that refuses the cooperative launch (answered by the test hook
+    on the host) costs the context the small-domain form and nothing else."""
+    import paper_2205_00686_gb300 as lbm
+    c = P.droplet_case(130, 70, P.bc_variants()["open_dirichlet"], seed=31)
+    ref = lbm.Domain(c.nx, c.ny, c.params, c.bc, prec=prec)
+    ref.init_fields(*c.fields())
+    d = lbm.Domain(c.nx, c.ny, c.params, c.bc, prec=prec)
+    d.init_fields(*c.fields())
+    d.step(5)
+    assert d.small_form()[0] > 0
+    d.set_wait_probe(2)
+    d.step(40)
+    assert d.small_form() == (0, 0, 0, 0)
+    d.set_wait_probe(0)
+    d.step(3)
+    ref.step(48)
+    assert ref.small_form()[0] > 0
+    assert d.step_count == ref.step_count == 48
+    for a, b in zip(d.populations(), ref.populations()):
+        assert np.array_equal(a, b)
+    ref.close()
+    d.close()
