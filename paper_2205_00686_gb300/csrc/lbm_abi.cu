@@ -541,7 +541,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, const lbm_bc* bc, int p
                             staged, nx, ny);
     }
     int rc = ctx_apply_tile(c, threads, rows, staged);
-    if (rc == LBM_OK && tile_plan(prec, I, c->phys, num_sms(), &c->tile))
+    if (rc == LBM_OK && tile_plan(prec, I, num_sms(), &c->tile))
         rc = set_err(c, LBM_ECUDA, "occupancy query failed");
     if (rc) {
         lbm_destroy(c);

@@ -307,7 +307,7 @@ struct TileLaunch {
     int tx, ty, ring0, ntx, n_tiles, steps;
     int targets;       // the domain has a target step (lbm_set_target)
 };
-int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out);
+int tile_plan(int prec, const Inst& I, int sms, TilePlan* out);
 cudaError_t tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys,
                         cudaStream_t st);
 

@@ -440,14 +440,18 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
     if (err) atomicOr(&I.ctl->err, err);
 }
 
-template <int PREC, bool UNIT>
+// CTAs per SM of both instantiations, the fewer: a plan outlives lbm_reconfigure,
+// which may change between unit and general rates
+template <int PREC>
 int tile_occ(int threads, size_t smem, int* ctas) {
-    // up to 227 KB a CTA (only FP64 tiles come near the 48 KB that need no attribute)
-    if (cudaFuncSetAttribute(k_tile<PREC, UNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) !=
-        cudaSuccess)
+    int unit = 0, general = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&unit, k_tile<PREC, true>, threads, smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&general, k_tile<PREC, false>, threads, smem) !=
+            cudaSuccess)
         return -1;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_tile<PREC, UNIT>, threads, smem) ==
-                   cudaSuccess ? 0 : -1;
+    *ctas = std::min(unit, general);
+    return 0;
 }
 
 template <int PREC, bool UNIT>
@@ -469,11 +473,6 @@ cudaError_t tile_run(const TileLaunch& L, const PhysD& phys, int grid, int threa
     return e;
 }
 
-template <int PREC>
-int tile_occ_any(const PhysD& phys, int threads, size_t smem, int* ctas) {
-    return unit_rates(phys) ? tile_occ<PREC, true>(threads, smem, ctas)
-                            : tile_occ<PREC, false>(threads, smem, ctas);
-}
 template <int PREC>
 cudaError_t tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int threads, size_t smem,
                          cudaStream_t st) {
@@ -506,7 +505,7 @@ cudaError_t tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int t
 // 32 x 8 73.8 / 74.6; the sweep needs 92 at 200^2, 154 at 384^2, 156 at 512^2
 // (this form 124) and 198 at 640^2 (11 rounds of 32 x 8, 203 modelled), so
 // domains up to 190 modelled microseconds come here.
-int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out) {
+int tile_plan(int prec, const Inst& I, int sms, TilePlan* out) {
     out->tx = 0;
     if ((long long)I.nx * I.ny > (1 << 20)) return 0;   // far beyond either limit below
     struct Cand { int tx, ty, sep; };
@@ -526,9 +525,9 @@ int tile_plan(int prec, const Inst& I, const PhysD& phys, int sms, TilePlan* out
         const long long ntx = (I.nx + tx - 1) / tx, nt = ntx * ((I.ny + ty - 1) / ty);
         const size_t smem = tile_bytes(es, tx, ty);
         int ctas = 0;
-        const int rc = prec == 0 ? tile_occ_any<0>(phys, threads, smem, &ctas)
-                       : prec == 1 ? tile_occ_any<1>(phys, threads, smem, &ctas)
-                                   : tile_occ_any<2>(phys, threads, smem, &ctas);
+        const int rc = prec == 0 ? tile_occ<0>(threads, smem, &ctas)
+                       : prec == 1 ? tile_occ<1>(threads, smem, &ctas)
+                                   : tile_occ<2>(threads, smem, &ctas);
         if (rc) return -1;
         if (ctas < 1) continue;
         const long long slots = (long long)ctas * sms, rounds = (nt + slots - 1) / slots;

@@ -37,3 +37,31 @@ def test_refused_cooperative_launch_goes_on_with_the_sweep(prec):
         assert np.array_equal(a, b)
     ref.close()
     d.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_rates_changed_after_the_plan(prec):
+    """The plan is made at creation; lbm_reconfigure may then switch between
+    unit and general rates, another kernel on the same grid.  A domain of
+    several rounds of tiles keeps agreeing with the sweep."""
+    import paper_2205_00686_gb300 as lbm
+    c = P.droplet_case(430, 410, P.bc_variants()["open_dirichlet"], seed=32)
+    general = dict(c.params, s_e=1.1, s_eps=0.9, s_q=1.2, vs3=0.8, vs4=1.3)
+    pops = []
+    for sweep in (False, True):
+        d = lbm.Domain(c.nx, c.ny, c.params, c.bc, prec=prec)
+        if sweep:
+            d.set_tile(128, 32)
+        d.init_fields(*c.fields())
+        d.step(7)
+        d.reconfigure(general, c.bc)
+        d.step(7)
+        tx, ty, tiles, ctas = d.small_form()
+        assert (tx > 0) != sweep and (sweep or tiles > ctas)
+        d.reconfigure(c.params, c.bc)
+        d.step(7)
+        d.sync()
+        pops.append(d.populations())
+        d.close()
+    for a, b in zip(*pops):
+        assert np.array_equal(a, b)
