@@ -114,13 +114,20 @@ uint32_t crc32_update(uint32_t crc, const void* data, size_t n) {
     return ~crc;
 }
 
-// tile autotuner cache: (prec, nx, ny) -> (threads, rows, staged, small form)
+// tile autotuner cache: (prec, nx, ny) -> (threads, rows, staged), and whether the
+// small-domain form beat that sweep, by flow kinds in y and rates (which decide how
+// the two compare)
 struct Tile {
-    int threads, rows, staged, tiled;
+    int threads, rows, staged;
+    signed char tiled[4];   // -1: not timed
 };
 std::map<std::tuple<int, int, int>, Tile>& tune_cache() {
     static std::map<std::tuple<int, int, int>, Tile> m;
     return m;
+}
+
+int form_key(const Inst& I, const PhysD& d) {
+    return (I.flow[ES] == WALL || I.flow[EN] == WALL ? 2 : 0) + (unit_rates(d) ? 1 : 0);
 }
 
 int num_sms() {
@@ -547,7 +554,8 @@ int lbm_create(int nx, int ny, const lbm_params* params, const lbm_bc* bc, int p
         lbm_destroy(c);
         return rc;
     }
-    c->tiled = c->tile.tx > 0 && (it == tune_cache().end() || it->second.tiled);
+    c->tiled = c->tile.tx > 0 &&
+               (it == tune_cache().end() || it->second.tiled[form_key(I, c->phys)] != 0);
     *out = c;
     return LBM_OK;
 }
@@ -1178,9 +1186,17 @@ int lbm_autotune(lbm_ctx* c, int steps) {
         lbm_destroy(s);
         return set_err(c, rc, "autotune: init failed");
     }
+    if (c->wait_probe == 2) s->wait_probe = 2;   // refused launches are refused here too
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
+    // time of a trial; a trial that fails is out of the comparison
+    auto trial = [&](float* ms) {
+        return lbm_step(s, 2) == LBM_OK && cudaEventRecord(e0, s->stream) == cudaSuccess &&
+               lbm_step(s, steps) == LBM_OK && cudaEventRecord(e1, s->stream) == cudaSuccess &&
+               cudaEventSynchronize(e1) == cudaSuccess &&
+               cudaEventElapsedTime(ms, e0, e1) == cudaSuccess;
+    };
     float best = 1e30f;
     int bt = c->threads, br = c->rows, bs = c->staged;
     const int thr_c[4] = {128, 192, 224, 256};
@@ -1207,14 +1223,8 @@ int lbm_autotune(lbm_ctx* c, int steps) {
             for (int rows : rows_c) {
                 if (ctx_apply_tile(s, thr_c[ti], rows, staged)) continue;
                 s->tiled = false;
-                lbm_step(s, 2);
-                cudaEventRecord(e0, s->stream);
-                lbm_step(s, steps);
-                cudaEventRecord(e1, s->stream);
-                if (cudaEventSynchronize(e1) != cudaSuccess) continue;
                 float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (ms < best) {
+                if (trial(&ms) && ms < best) {
                     best = ms;
                     bt = thr_c[ti];
                     br = rows;
@@ -1225,18 +1235,19 @@ int lbm_autotune(lbm_ctx* c, int steps) {
     bool tiled = false;
     if (s->tile.tx > 0) {
         s->tiled = true;
-        lbm_step(s, 2);
-        cudaEventRecord(e0, s->stream);
-        lbm_step(s, steps);
-        cudaEventRecord(e1, s->stream);
         float ms = 0.f;
-        if (cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
-            tiled = ms < best;
+        // (a refused launch leaves the trial on the sweep)
+        tiled = trial(&ms) && s->tiled && ms < best;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     lbm_destroy(s);
-    tune_cache()[std::make_tuple(c->prec, c->nx, c->ny)] = Tile{bt, br, bs, tiled ? 1 : 0};
+    Tile& kept = tune_cache().emplace(std::make_tuple(c->prec, c->nx, c->ny), Tile{0, 0, 0, {-1, -1, -1, -1}})
+                     .first->second;
+    kept.threads = bt;
+    kept.rows = br;
+    kept.staged = bs;
+    kept.tiled[form_key(c->inst, c->phys)] = tiled ? 1 : 0;
     rc = ctx_apply_tile(c, bt, br, bs);
     if (rc == LBM_OK) c->tiled = tiled;
     return rc;

@@ -65,3 +65,28 @@ def test_rates_changed_after_the_plan(prec):
         d.close()
     for a, b in zip(*pops):
         assert np.array_equal(a, b)
+
+
+def test_autotune_keeps_no_form_that_was_refused():
+    """A trial whose launch is refused is out of the comparison, and what the
+    autotuner learned for one set of boundaries and rates says nothing about
+    another."""
+    import paper_2205_00686_gb300 as lbm
+    v = P.bc_variants()
+    c = P.droplet_case(210, 150, v["open_dirichlet"], seed=33)
+
+    def fresh(bc="open_dirichlet", **over):
+        return lbm.Domain(c.nx, c.ny, dict(c.params, **over), v[bc], prec="fp32")
+
+    d = fresh()
+    d.init_fields(*c.fields())
+    d.set_wait_probe(2)
+    d.autotune(4)
+    assert d.small_form() == (0, 0, 0, 0)
+    assert fresh().small_form() == (0, 0, 0, 0)
+    assert fresh("two_walls_adiabatic").small_form()[0] > 0
+    assert fresh(s_q=1.2).small_form()[0] > 0
+    d.set_wait_probe(0)
+    d.autotune(4)
+    assert d.small_form()[0] > 0 and fresh().small_form() == d.small_form()
+    d.close()
