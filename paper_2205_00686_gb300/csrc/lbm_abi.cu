@@ -14,6 +14,7 @@
 
 #include "lbm.h"
 #include "lbm_internal.cuh"
+#include "lbm_rules.h"
 
 using namespace lbm;
 
@@ -1259,48 +1260,6 @@ int lbm_autotune(lbm_ctx* c, int steps) {
 // new ones allocated and filled, on the batch stream (cudaFreeAsync,
 // cudaMallocAsync, copies from a pinned staging slot), so launches already
 // queued keep their own arrays and the host does not wait for them.
-// Segment height of a batch without a tuned tile: the domains' strips are cut
-// into segments of at most R rows, even within a domain, and the CTAs take them
-// from one list, longest first, so a launch lasts about w (R + 8) iterations
-// where w rounds of resident CTAs take all segments (a segment's sweep runs 6
-// iterations beyond its rows and starts up in about 2).  For each w the smallest
-// R that fits, then the w that gives the shortest launch.  FP32 open domains,
-// us per step: 64 of sides 64-512, the former 64 rows on the register tile 222,
-// this (73 rows, staged) 203, the tuner's best fixed height 208; 20 of sides
-// 64-300 45 (19 rows), 8 of sides 64-200 30 (8 rows).
-static int batch_rows(const std::vector<const Inst*>& ip, int threads, long long slots) {
-    const int W = threads - 8;
-    long long strip_rows = 0;
-    int most = 1;
-    for (const Inst* I : ip) {
-        strip_rows += (long long)((I->nx + W - 1) / W) * I->ny;
-        most = std::max(most, I->ny);
-    }
-    auto segments = [&](int R) {
-        long long n = 0;
-        for (const Inst* I : ip) n += (long long)((I->nx + W - 1) / W) * ((I->ny + R - 1) / R);
-        return n;
-    };
-    const long long w0 = std::max<long long>(1, (strip_rows + slots * most - 1) / (slots * most));
-    long long best = 0;
-    int rows = most;
-    for (long long w = w0; w < w0 + 12; ++w) {
-        if (segments(most) > w * slots) continue;
-        int lo = std::min(8, most), hi = most;
-        while (lo < hi) {
-            const int mid = (lo + hi) / 2;
-            if (segments(mid) <= w * slots) hi = mid;
-            else lo = mid + 1;
-        }
-        const long long t = w * (lo + 8);
-        if (best == 0 || t < best) {
-            best = t;
-            rows = lo;
-        }
-    }
-    return rows;
-}
-
 static int batch_rebuild(lbm_batch* b) {
     drop_graph(&b->graph);
     if (b->insts) cudaFreeAsync(b->insts, b->stream);
@@ -1336,7 +1295,14 @@ static int batch_rebuild(lbm_batch* b) {
     size_t smem = 0;
     step_occupancy(b->prec, b->threads, b->walls, b->staged, &ctas, &smem);
     const long long slots = (long long)std::max(ctas, 1) * num_sms();
-    if (!b->tuned) b->rows = batch_rows(ip, b->threads, slots);
+    if (!b->tuned) {
+        std::vector<int> nx, ny;
+        for (const Inst* I : ip) {
+            nx.push_back(I->nx);
+            ny.push_back(I->ny);
+        }
+        b->rows = batch_rows(nx.data(), ny.data(), ip.size(), b->threads, slots);
+    }
     for (size_t i = 0; i < b->members.size(); ++i)
         build_units(b->members[i]->inst, (int)i, b->threads, std::min(b->rows, b->members[i]->ny), true, us);
     // longest first: a unit's sweep takes (rows + 6) iterations whatever its
