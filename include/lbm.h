@@ -372,8 +372,7 @@ int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged)
  * Small domains (up to about 740 x 740 in FP32, 600 x 600 in FP64) take another
  * form of the same arithmetic unless a tile or load path is asked for: lbm_step
  * runs up to 1024 steps in one cooperative launch over tiles of nodes.  The
- * state is bit for bit the sweep's (with buoyancy, up to the rounding of the
- * density sum).  lbm_set_tile and lbm_set_staging select the sweep,
+ * state is bit for bit the sweep's.  lbm_set_tile and lbm_set_staging select the sweep,
  * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile.  Where
  * the cooperative launch is refused (a process or stream that may use only part
  * of the SMs), the context takes the sweep from that step on.

@@ -24,13 +24,15 @@ enum { ERR_PSI = 1, ERR_NONFINITE = 2, ERR_TIMEOUT = 4 };
 // read by every launch, the three-slot ring of per-step density sums used by
 // the buoyancy force (step n accumulates sum rho(n) into slot n % 3 and reads
 // slot (n - 1) % 3), and the sticky error word.  The CTAs of a launch add
-// their block sums as fixed-point integers (massq, see massq_scale), so the
-// total does not depend on the order in which the CTAs finish; the launch's
-// last CTA converts the finished slot to mass[] for the next step to read.
+// their sums as fixed-point integers (massq and massh, see mass_bits; in three
+// dimensions massq alone, see massq_scale), so the total does not depend on the
+// order in which the CTAs finish; the launch's last CTA converts the finished
+// slot to mass[] for the next step to read.
 struct Ctl {
     long long step;
     double mass[3];
     long long massq[3];
+    long long massh[3];
     // the step count at which the domain stops (> 0), or 0 for none: a
     // launch skips the units of a domain that has reached it, so its state,
     // step counter and density ring stay as they are
@@ -44,7 +46,7 @@ __device__ __forceinline__ bool ctl_stopped(const Ctl* c) {
     return tg > 0 && __ldcg(&c->step) >= tg;
 }
 
-// fixed-point scale of Ctl::massq for a domain of N = 1 / inv_n nodes:
+// fixed-point scale of a three-dimensional domain's Ctl::massq, N = 1 / inv_n nodes:
 // 2^(58 - e) with N < 2^e.  Densities stay below 16 (the EOS ends at 1/b =
 // 10.5), so a domain total stays below 2^62 and no sum overflows, while a
 // block sum keeps at least 30 fraction bits (N < 2^28) and small domains keep
@@ -60,6 +62,26 @@ __device__ __forceinline__ void massq_add(long long* slot, double block_sum, dou
 }
 __host__ __device__ __forceinline__ double massq_value(long long q, double scale) {
     return (double)q / scale;
+}
+
+// Density sum of the two-dimensional step.  Every node's density is rounded to a
+// fixed-point number of mass_bits(b) fraction bits and the numbers are added as
+// integers, low 24 bits of a warp's sum into massq and the rest into massh: the
+// total is exact, so rho_ave is the same bit for bit whatever strips, segments or
+// tiles the domain is cut into, alone or in a batch.  (Sums in floating point over
+// a segment's rows changed with the segment's height, which a batch takes from
+// all of its members.)  Densities end at 1/b (EOS): with 1/b < 2^e the numbers
+// hold up to 2^(e+1), in FP32 as 32 bits without sign (the grid is 7.5e-9 at b =
+// 2/21: exact for a float density of 0.125 or more; a negative one counts as 0),
+// in FP64 to 2^-(50-e) (1.4e-14, where a floating-point sum of 64 rows rounds at
+// 3e-14).  It costs the 4096^2 FP32 step 334.5 -> 337.9 us, a batch of 64 192.8 ->
+// 194.7; the 300 x 600 pool, whose threads no longer convert the sum back with a
+// division each, went from 16.9 to 14.7.
+inline int mass_bits(double b, bool fp64) {
+    int e = 0;
+    frexp(1.0 / b, &e);
+    e = e < -60 ? -60 : (e > 60 ? 60 : e);
+    return (fp64 ? 50 : 31) - e;
 }
 
 // One domain as seen by the kernels.  Populations are stored as deviations
@@ -106,6 +128,8 @@ struct Phys {
     R cv, inv_cv, inv_12cv, w_dot, w5_0, w5_1, vs1_cs2h, vs3, vs4;   // vs1_cs2h = vs1 / cs2h
     R h_m, one_m_vs4;               // h_m = (1 - vs1) / 2
     R gravity;
+    R m_fix;              // density to fixed point, see mass_fix
+    double m_unit;        // and back
     int frozen_flow, frozen_thermal;
 };
 
@@ -169,6 +193,11 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.h_m = (R)(0.5 * (1.0 - d.vs1));
     p.one_m_vs4 = (R)(1.0 - d.vs4);
     p.gravity = (R)d.gravity;
+    // FP32 multiplies by 2^bits; FP64 adds 1.5 * 2^(52 - bits), which leaves the
+    // rounded density in the low bits of the sum
+    const int bits = mass_bits(d.b, sizeof(R) == 8);
+    p.m_fix = (R)(sizeof(R) == 8 ? std::ldexp(1.5, 52 - bits) : std::ldexp(1.0, bits));
+    p.m_unit = std::ldexp(1.0, -bits);
     p.frozen_flow = d.frozen_flow;
     p.frozen_thermal = d.frozen_thermal;
     return p;
@@ -245,6 +274,24 @@ __device__ __forceinline__ double f_sqrt(double x) {
     const double t = x * y;
     const double e = fma(-t, y, 1.0);
     return fma(t * e, fma(0.375, e, 0.5), t);
+}
+
+// density of a node as a fixed-point number (see mass_bits), one conversion in
+// FP32, in FP64 one addition on the FP64 pipe as a running sum would take
+// (0 where the node is not counted)
+__device__ __forceinline__ unsigned mass_fix(const Phys<float>& P, float rho, bool counted) {
+    return __float2uint_rn(__fmul_rn(rho, counted ? P.m_fix : 0.0f));
+}
+__device__ __forceinline__ long long mass_fix(const Phys<double>& P, double rho, bool counted) {
+    const long long q = __double_as_longlong(__dadd_rn(rho, P.m_fix)) - __double_as_longlong(P.m_fix);
+    return counted ? q : 0;
+}
+__device__ __forceinline__ void mass_add(Ctl* c, int slot, long long sum) {
+    atomicAdd(reinterpret_cast<unsigned long long*>(&c->massq[slot]), (unsigned long long)(sum & 0xffffff));
+    atomicAdd(reinterpret_cast<unsigned long long*>(&c->massh[slot]), (unsigned long long)(sum >> 24));
+}
+__device__ __forceinline__ double mass_total(const Ctl* c, int slot, double unit) {
+    return fma((double)__ldcg(&c->massh[slot]), 16777216.0, (double)__ldcg(&c->massq[slot])) * unit;
 }
 
 __device__ __forceinline__ int wrapi(int i, int n) {

@@ -213,7 +213,7 @@ struct Sweep {
     // the stress moments m_7 and m_8, formed in stage A (fp is then unused)
     R m7p, m8p;
     R fa[9], ga[5], pa;
-    R mass_acc;
+    long long mass_acc;     // sum of mass_fix
     int errbits;
     int ra0, ra1, ra2, b0, kw;
     // staged form: window start column, this column's index in a staged row,
@@ -323,7 +323,7 @@ struct Sweep {
         rhop = R(1);
         rhodp = jxp = jyp = psip = R(0);
         irp = R(1);
-        mass_acc = R(0);
+        mass_acc = 0;
         errbits = 0;
 #pragma unroll
         for (int q = 0; q < 5; ++q) cg[q] = dg[q] = R(0);
@@ -716,9 +716,6 @@ struct Sweep {
                 S.own[b0][1][t] = o1;
                 if constexpr (sizeof(R) == 8) S.own2[b0][t] = pr(nd.iC, nd.Td);
             }
-            // this unit's output rows only (steady iterations also load the
-            // three rows above the segment)
-            mass_acc += (inD && k >= my0 && k < my1) ? rho_a : R(0);
         }
         __syncthreads();
 
@@ -735,6 +732,11 @@ struct Sweep {
         if constexpr (STG) {
             if (k + DA + 1 <= y1 + 3) arm_row(k + DA + 1, NF == 3 ? a0 : fq);
         }
+
+        // density sum: this unit's output rows only (steady iterations also load
+        // the three rows above the segment).  Here rather than in stage A, whose
+        // barrier would wait for the conversion (4096^2 338.6 -> 337.9 us)
+        mass_acc += mass_fix(P, rhop, inD && k - 1 >= my0 && k - 1 < my1);
 
         // ---- B(k-1): interaction force, velocity, D2Q9 MRT collision
         {
@@ -927,12 +929,12 @@ __device__ __forceinline__ void process_unit(const Inst& I, const Unit& U,
         // fixed-point integers (order-free, so no barrier is needed); kept
         // with gravity off too, so that lbm_reconfigure can switch buoyancy on
         // with the previous step's density sum in place
-        double macc = (double)w.mass_acc;
+        long long macc = w.mass_acc;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) macc += __shfl_down_sync(0xffffffffu, macc, o);
         if ((w.t & 31) == 0) {
             const long long step = __ldcg(&I.ctl->step);
-            massq_add(&I.ctl->massq[step % 3], macc, massq_scale(I.inv_n));
+            mass_add(I.ctl, (int)(step % 3), macc);
         }
     }
 }
@@ -985,8 +987,9 @@ __global__ void __launch_bounds__(NT, (PREC == 0) ? 1 : (512 / NT))
             Ctl* c = L.insts[i].ctl;
             if (L.targets && ctl_stopped(c)) continue;
             const long long s = __ldcg(&c->step);
-            c->mass[s % 3] = massq_value(__ldcg(&c->massq[s % 3]), massq_scale(L.insts[i].inv_n));
+            c->mass[s % 3] = mass_total(c, (int)(s % 3), P.m_unit);
             c->massq[(s + 1) % 3] = 0;
+            c->massh[(s + 1) % 3] = 0;
             c->step = s + 1;
         }
         __syncthreads();

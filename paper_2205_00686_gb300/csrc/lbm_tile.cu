@@ -83,7 +83,7 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
     R2* const s_u = reinterpret_cast<R2*>(s_psi + ((N2 + 1) & ~1));         // [N1]
     R* const s_ic = reinterpret_cast<R*>(s_u + N1);                         // [N1]
     R* const s_g = s_ic + N1;                                               // [4][N1] g_1 .. g_4
-    __shared__ double s_mass[16];
+    __shared__ long long s_mass[16];
     __shared__ int s_abort;
 
     const int t = threadIdx.x, NT = blockDim.x;
@@ -151,15 +151,17 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
         R rho_ave = R(0);
         if (use_mass) {
             const int sl = (int)((step + 2) % 3);
-            const double m = s == 0 ? __ldcg(&I.ctl->mass[sl])
-                                    : massq_value(__ldcg(&I.ctl->massq[sl]), massq_scale(I.inv_n));
+            const double m = s == 0 ? __ldcg(&I.ctl->mass[sl]) : mass_total(I.ctl, sl, P.m_unit);
             rho_ave = (R)(m * I.inv_n);
         }
         // this step's sum: with buoyancy every step's is read by the next;
         // without, only the last one of the launch is kept
         const bool sum_mass = use_mass || s == steps - 1;
-        double msum = 0.0;
-        if (blockIdx.x == 0 && t == 0) I.ctl->massq[(step + 1) % 3] = 0;
+        long long msum = 0;
+        if (blockIdx.x == 0 && t == 0) {
+            I.ctl->massq[(step + 1) % 3] = 0;
+            I.ctl->massh[(step + 1) % 3] = 0;
+        }
 
         for (int tile = blockIdx.x; tile < L.n_tiles; tile += gridDim.x) {
             if (tile != set_up) {
@@ -226,7 +228,7 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
             if (own) {
                 node_fields(P, rho_ref, T_ref, fo, go, no);
                 keep(no, go, c2, c1, true);
-                if (sum_mass && gy >= I.own_y0 && gy < I.own_y1) msum += (double)no.rho;
+                if (sum_mass) msum += mass_fix(P, no.rho, gy >= I.own_y0 && gy < I.own_y1);
             }
             // ---- A: the nodes around the tile
             const bool near = kr < n_ring1;
@@ -397,7 +399,7 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
             }
         }
 
-        // ---- the step's density sum, fixed point (order-free)
+        // ---- the step's density sum (exact, order-free)
         if (sum_mass) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(0xffffffffu, msum, o);
@@ -406,9 +408,9 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
         __syncthreads();
         if (t == 0) {
             if (sum_mass) {
-                double m = 0.0;
+                long long m = 0;
                 for (int w = 0; w < (NT + 31) / 32; ++w) m += s_mass[w];
-                massq_add(&I.ctl->massq[step % 3], m, massq_scale(I.inv_n));
+                mass_add(I.ctl, (int)(step % 3), m);
             }
             __threadfence();
             const unsigned done = bar_add(L.bar);
@@ -417,8 +419,7 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
                 // the last CTA of the launch publishes the density sum, advances
                 // the step counter and clears the grid counter for the next launch
                 if (done == all - 1) {
-                    I.ctl->mass[step % 3] = massq_value(__ldcg(&I.ctl->massq[step % 3]),
-                                                        massq_scale(I.inv_n));
+                    I.ctl->mass[step % 3] = mass_total(I.ctl, (int)(step % 3), P.m_unit);
                     I.ctl->step = step + 1;
                     *L.bar = 0u;
                     __threadfence();
