@@ -376,10 +376,15 @@ int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged)
  * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile.  Where
  * the cooperative launch is refused (a process or stream that may use only part
  * of the SMs), the context takes the sweep from that step on.
+ * lbm_set_small_form: back from a sweep tile to that form, with the tile of its
+ * own choice (0, 0; a domain beyond its range stays with the sweep) or a given
+ * one: 8 x 8, 32 x 8, 32 x 10 or 32 x 12 nodes in FP32, 8 x 4, 8 x 8, 16 x 8, 32 x
+ * 8 or 20 x 14 in FP64 (LBM_EINVAL for others and beyond 2^20 nodes).
  * lbm_get_small_form: the tile (tx x ty nodes), tiles and CTAs per launch of the
  * form lbm_step takes next; all 0 when it is the sweep. */
 int lbm_set_tile(lbm_ctx* ctx, int threads, int rows);
 int lbm_get_tile(const lbm_ctx* ctx, int* threads, int* rows);
+int lbm_set_small_form(lbm_ctx* ctx, int tx, int ty);
 int lbm_get_small_form(const lbm_ctx* ctx, int* tx, int* ty, int* tiles, int* grid);
 int lbm_autotune(lbm_ctx* ctx, int steps_per_trial);
 
@@ -412,7 +417,10 @@ int lbm_get_staging(const lbm_ctx* ctx);
  * records LBM_ETIMEOUT in the sticky error word.  The row pipeline keeps its
  * own waits, so the step's results are unchanged and no copy is left in
  * flight; the GPU is never faulted.  No effect on the register-prefetch path
- * or on batches.  on = 2: the cooperative launches of the small-domain form are
+ * or on batches.  A launch of several steps of the small-domain form has its CTAs
+ * give up at once at the grid barrier: they leave, the launches queued behind it
+ * advance nothing, and the state is lost until lbm_init_fields, lbm_set_populations or
+ * lbm_load.  on = 2: the cooperative launches of the small-domain form are
  * answered as if the device had refused them (nothing is launched).  Returns LBM_EINVAL for NULL, LBM_ESTATE in a batch. */
 int lbm_set_wait_probe(lbm_ctx* ctx, int on);
 

@@ -40,7 +40,8 @@ ABI_FUNCTIONS = (
     "lbm_batch_create", "lbm_batch_attach", "lbm_batch_detach", "lbm_batch_size",
     "lbm_batch_step", "lbm_batch_sync", "lbm_batch_destroy", "lbm_batch_autotune",
     "lbm_batch_errors_async",
-    "lbm_batch_get_tile", "lbm_set_tile", "lbm_get_tile", "lbm_get_small_form",
+    "lbm_batch_get_tile", "lbm_set_tile", "lbm_get_tile", "lbm_set_small_form",
+    "lbm_get_small_form",
     "lbm_autotune", "lbm_set_staging", "lbm_get_staging", "lbm_set_wait_probe",
     "lbm_diag_reduce_noalloc", "lbm_reconfigure", "lbm_contact_angle",
     "lbm_regions", "lbm_rows_bytes", "lbm_pack_rows", "lbm_unpack_rows", "lbm_set_partition",
@@ -146,6 +147,7 @@ def lib():
             "lbm_set_tile": ([_vp, ctypes.c_int, ctypes.c_int], ctypes.c_int),
             "lbm_get_tile": ([_vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)],
                              ctypes.c_int),
+            "lbm_set_small_form": ([_vp, ctypes.c_int, ctypes.c_int], ctypes.c_int),
             "lbm_get_small_form": ([_vp] + [ctypes.POINTER(ctypes.c_int)] * 4, ctypes.c_int),
             "lbm_autotune": ([_vp, ctypes.c_int], ctypes.c_int),
             "lbm_set_staging": ([_vp, ctypes.c_int], ctypes.c_int),
@@ -326,6 +328,11 @@ class Domain:
         lib().lbm_get_tile(self._h, ctypes.byref(t), ctypes.byref(r))
         return t.value, r.value
 
+    def set_small_form(self, tx: int = 0, ty: int = 0):
+        """Take the small-domain form, with the given tile or (0, 0) its own
+        choice; see lbm_set_small_form."""
+        _check(lib().lbm_set_small_form(self._h, int(tx), int(ty)), self._h)
+
     def small_form(self):
         """(tx, ty, tiles, CTAs) of the small-domain form step() takes next,
         zeros when it is the sweep; see lbm_get_small_form."""
@@ -350,7 +357,8 @@ class Domain:
     def set_wait_probe(self, on: int):
         """Test hook: with 1 (True) staged launches also wait on an mbarrier
         nothing arms, so each CTA's bounded wait runs out and LBM_ETIMEOUT is
-        reported; with 2 cooperative launches are answered as refused."""
+        reported, and multi-step launches of the small-domain form give up
+        at their grid barrier; with 2 cooperative launches are answered as refused."""
         _check(lib().lbm_set_wait_probe(self._h, int(on)), self._h)
 
     @property

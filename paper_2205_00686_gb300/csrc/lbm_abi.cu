@@ -22,6 +22,7 @@ namespace {
 
 const int kGraphLen = 32;      // launches per captured graph
 const int kTileSteps = 1024;   // most steps per launch of the small-domain form
+const unsigned kTileWait = 1u << 31;   // clocks at its grid barrier, about a second
 const size_t kAlign = 256;
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -383,6 +384,7 @@ static int enqueue_tiled(lbm_ctx* c, int n) {
     L.ntx = c->tile.ntx;
     L.n_tiles = c->tile.n_tiles;
     L.targets = c->target > 0 ? 1 : 0;
+    L.wait = c->wait_probe == 1 ? 0 : kTileWait;
     for (; n > 0; n -= L.steps) {
         L.steps = std::min(n, kTileSteps);
         // (one step has no barrier and is launched without that condition)
@@ -549,7 +551,7 @@ int lbm_create(int nx, int ny, const lbm_params* params, const lbm_bc* bc, int p
                             staged, nx, ny);
     }
     int rc = ctx_apply_tile(c, threads, rows, staged);
-    if (rc == LBM_OK && tile_plan(prec, I, num_sms(), &c->tile))
+    if (rc == LBM_OK && tile_plan(prec, I, num_sms(), 0, 0, &c->tile))
         rc = set_err(c, LBM_ECUDA, "occupancy query failed");
     if (rc) {
         lbm_destroy(c);
@@ -1159,6 +1161,17 @@ int lbm_get_tile(const lbm_ctx* c, int* threads, int* rows) {
     if (!c) return LBM_EINVAL;
     if (threads) *threads = c->threads;
     if (rows) *rows = c->rows;
+    return LBM_OK;
+}
+
+int lbm_set_small_form(lbm_ctx* c, int tx, int ty) {
+    if (!c || tx < 0 || ty < 0) return LBM_EINVAL;
+    if (c->batch) return set_err(c, LBM_ESTATE, "context is attached to a batch");
+    TilePlan T;
+    if (tile_plan(c->prec, c->inst, num_sms(), tx, ty, &T)) return set_err(c, LBM_ECUDA, "occupancy query failed");
+    if (T.tx == 0 && tx > 0) return set_err(c, LBM_EINVAL, "no such tile of the small-domain form");
+    c->tile = T;
+    c->tiled = T.tx > 0;
     return LBM_OK;
 }
 

@@ -353,8 +353,11 @@ struct TileLaunch {
     unsigned* bar;     // grid counter, 0 between launches
     int tx, ty, ring0, ntx, n_tiles, steps;
     int targets;       // the domain has a target step (lbm_set_target)
+    unsigned wait;     // clocks (modulo 2^32) a CTA waits at the grid barrier before it gives up
 };
-int tile_plan(int prec, const Inst& I, int sms, TilePlan* out);
+// the plan of the form's own choice, or (want_tx > 0) for that tile: tx = 0 when
+// there is none
+int tile_plan(int prec, const Inst& I, int sms, int want_tx, int want_ty, TilePlan* out);
 cudaError_t tile_launch(int prec, const TilePlan& T, const TileLaunch& L, const PhysD& phys,
                         cudaStream_t st);
 

@@ -21,7 +21,8 @@
 //
 // Steps of one launch are separated by a barrier over the grid (a counter in
 // device memory; the launch is cooperative, so every CTA is resident).  The
-// wait is bounded: after about a second a CTA records ERR_TIMEOUT and leaves.
+// wait is bounded: after about a second a CTA records ERR_TIMEOUT and leaves, and
+// the others with it.
 // What a step reads that another CTA wrote goes through L2 (ld.global.cg).
 // The arithmetic is that of lbm_node.cuh, so the state is bit for bit the one
 // the sweep would give.
@@ -49,6 +50,12 @@ __device__ __forceinline__ float ld_l2(const __half* p) {
 // 18.5 us per step, 256^2 5.1 -> 6.5).  FP64: up to 288 (20 x 14 nodes, 168
 // registers), so that 200 x 200 fits one round of 152 SMs.
 constexpr int TILE_MAX(int prec) { return prec == 0 ? 288 : 512; }
+
+// Set in the grid counter by a CTA that gave up its wait: the others leave at
+// their next look at the counter, and so do the launches queued behind this one,
+// until lbm_init_fields, lbm_set_populations or lbm_load clears it.  (Counts stay
+// below 1024 steps times a few thousand CTAs.)
+constexpr unsigned BAR_LEFT = 1u << 30;
 
 // release / acquire on the grid counter
 __device__ __forceinline__ unsigned bar_load(const unsigned* p) {
@@ -415,7 +422,9 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
             __threadfence();
             const unsigned done = bar_add(L.bar);
             const unsigned all = (unsigned)(s + 1) * gridDim.x;
-            if (s == steps - 1) {
+            if (done >= BAR_LEFT) {
+                s_abort = 1;
+            } else if (s == steps - 1) {
                 // the last CTA of the launch publishes the density sum, advances
                 // the step counter and clears the grid counter for the next launch
                 if (done == all - 1) {
@@ -425,14 +434,17 @@ k_tile(const __grid_constant__ TileLaunch L, const __grid_constant__ Phys<typena
                     __threadfence();
                 }
             } else if (done != all - 1) {
-                const long long c0 = clock64();
-                while (bar_load(L.bar) < all) {
-                    if (clock64() - c0 > (1LL << 31)) {
+                const unsigned c0 = (unsigned)clock();
+                unsigned v;
+                while ((v = bar_load(L.bar)) < all) {
+                    if ((unsigned)clock() - c0 > L.wait) {
+                        atomicOr(L.bar, BAR_LEFT);
                         err |= ERR_TIMEOUT;
                         s_abort = 1;
                         break;
                     }
                 }
+                if (v >= BAR_LEFT) s_abort = 1;
             }
         }
         __syncthreads();
@@ -506,8 +518,9 @@ cudaError_t tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int t
 // 32 x 8 73.8 / 74.6; the sweep needs 92 at 200^2, 154 at 384^2, 156 at 512^2
 // (this form 124) and 198 at 640^2 (11 rounds of 32 x 8, 203 modelled), so
 // domains up to 190 modelled microseconds come here.
-int tile_plan(int prec, const Inst& I, int sms, TilePlan* out) {
+int tile_plan(int prec, const Inst& I, int sms, int want_tx, int want_ty, TilePlan* out) {
     out->tx = 0;
+    const bool any = want_tx > 0;
     if ((long long)I.nx * I.ny > (1 << 20)) return 0;   // far beyond either limit below
     struct Cand { int tx, ty, sep; };
     static const Cand c32[4] = {{8, 8, 1}, {32, 8, 0}, {32, 10, 0}, {32, 12, 0}};
@@ -518,6 +531,7 @@ int tile_plan(int prec, const Inst& I, int sms, TilePlan* out) {
     double best = 1e30;
     for (int k = 0; k < n_cand; ++k) {
         const int tx = cand[k].tx, ty = cand[k].ty;
+        if (any && (tx != want_tx || ty != want_ty)) continue;
         const int n_ring1 = 2 * (tx + ty) + 4, n_ring = n_ring1 + 2 * (tx + ty) + 12;
         const int own_w = (tx * ty + 31) / 32, ring_w = (n_ring + 31) / 32;
         // separate: the surrounding nodes have threads of their own
@@ -534,10 +548,10 @@ int tile_plan(int prec, const Inst& I, int sms, TilePlan* out) {
         const long long slots = (long long)ctas * sms, rounds = (nt + slots - 1) / slots;
         double us;
         if (prec != 0) {
-            if (cand[k].sep && nt > sms) continue;
+            if (cand[k].sep && nt > sms && !any) continue;
             static const double per_round[4] = {1.75, 3.45, 2.4, 2.75};
             us = 1.6 + per_round[k] * (double)rounds;
-            if (us > 26.0) continue;
+            if (us > 26.0 && !any) continue;
         } else {
             const double ring_cost = 65.0 + 25.0 * n_ring1 / n_ring;
             // the busiest partition of one CTA, and all partitions of the CTAs
@@ -548,7 +562,7 @@ int tile_plan(int prec, const Inst& I, int sms, TilePlan* out) {
             const double all = (double)share * (own_w * 170.0 + ring_w * ring_cost) / 4.0;
             us = (double)rounds * (3.4 + std::max(part, all) * 64.0 / 2070.0);
             if (tx * ty == 128) us *= 1.12;   // measured against modelled, 64^2 and 384^2
-            if (us > 190.0) continue;
+            if (us > 190.0 && !any) continue;
         }
         if (us >= best) continue;
         best = us;
