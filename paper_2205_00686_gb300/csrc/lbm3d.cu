@@ -1237,6 +1237,7 @@ struct lbm3d_ctx {
     int zseg = 0;            // planes per CTA of the marching step
     long long step = 0;
     bool initialized = false;
+    bool unseen = false;     // the step over nodes has made a state whose fields are not formed yet
     int sticky = LBM_OK;
     std::string err;
     double* host_buf = nullptr;   // device doubles: 27 N (export), reused
@@ -1356,6 +1357,24 @@ int check3(lbm3d_ctx* c) {
     return c->sticky;
 }
 
+// As check3, for the state the last step made.  The step over nodes forms and
+// checks the fields of a state when it starts from it; here they are formed for
+// the check alone.  (The marching step reports a state with the step after it.)
+int check_state(lbm3d_ctx* c) {
+    if (c->unseen && c->sticky == LBM_OK) {
+        if (c->prec == LBM_FP64)
+            k3_macro<double><<<grd3(c), blk3(), 0, c->stream>>>(c->D, make_phys<double>(phys_of(c->params)),
+                                                                make_lat3<double>(c->params, c->D), 0, 0);
+        else
+            k3_macro<float><<<grd3(c), blk3(), 0, c->stream>>>(c->D, make_phys<float>(phys_of(c->params)),
+                                                               make_lat3<float>(c->params, c->D), 0, 0);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_err3(c, e, "fields kernel");
+        c->unseen = false;
+    }
+    return check3(c);
+}
+
 int ensure_buf(lbm3d_ctx* c) {
     if (c->host_buf) return LBM_OK;
     const size_t N = (size_t)c->nx * c->ny * c->nz;
@@ -1374,6 +1393,7 @@ int export_fields(lbm3d_ctx* c, int what) {
     if (rc) return rc;
     if (c->prec == LBM_FP64) launch_fields<double>(c, what);
     else launch_fields<float>(c, what);
+    c->unseen = false;
     return cuda_err3(c, cudaGetLastError(), "field export");
 }
 
@@ -1534,6 +1554,7 @@ int lbm3d_init_fields(lbm3d_ctx* c, const double* rho, const double* ux, const d
     if (c->graph) cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;   // the launch arguments carry rho_ref / T_ref
     c->step = 0;
+    c->unseen = false;
     c->sticky = LBM_OK;
     c->initialized = true;
     c->err.clear();
@@ -1545,6 +1566,7 @@ int lbm3d_step(lbm3d_ctx* c, int n) {
     if (!c->initialized) return set_err3(c, LBM_ESTATE, "lbm3d_step before lbm3d_init_fields");
     if (c->sticky) return c->sticky;
     if (n == 0) return LBM_OK;
+    c->unseen = !(c->fused && march_fits(c));
     const int kLen = 32;
     int left = n;
     if (left >= kLen) {
@@ -1608,7 +1630,7 @@ int lbm3d_get_populations(lbm3d_ctx* c, double* f, double* g, double* P) {
     if (e == cudaSuccess && P)
         e = cudaMemcpyAsync(P, c->host_buf + 26 * N, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return cuda_err3(c, e, "copying populations to the host");
-    return check3(c);
+    return check_state(c);
 }
 
 int lbm3d_diagnostics(lbm3d_ctx* c, double rho_l, double rho_g, int sessile, lbm_diag* out) {
@@ -1664,7 +1686,7 @@ int lbm3d_get_path(const lbm3d_ctx* c, int* fused, int* zseg) {
 int lbm3d_sync(lbm3d_ctx* c) {
     if (!c) return LBM_EINVAL;
     if (!c->initialized) return LBM_OK;
-    return check3(c);
+    return check_state(c);
 }
 
 void lbm3d_destroy(lbm3d_ctx* c) {
