@@ -42,12 +42,13 @@ sys.path.insert(0, ROOT)
 NX = NY = 4096
 BYTES_PER_NODE = {"fp32": 120, "fp64": 240, "fp32_g16": 100}
 # FP64 FLOP per node update of the FP64 step (2 DFMA + DADD + DMUL thread
-# instructions per node, ncu on the same kernel: profiles/k_step_fp64_2048_alu.md)
+# instructions per node, from ncu's instruction counters on the same kernel)
 # and the nominal FP64 rate of the part (no measured FP64 peak on this machine)
 FP64_FLOP_PER_NODE = 239.0
 FP64_NOMINAL_GFLOPS = 1250.0
 METRIC = "coupled D2Q9+D2Q5 MLUPS and % of HBM roofline, FP32 vs FP64 at stated error"
 STEP_SOURCES = ["paper_2205_00686_gb300/csrc/lbm_step.cu",
+                "paper_2205_00686_gb300/csrc/lbm_node.cuh",
                 "paper_2205_00686_gb300/csrc/lbm_internal.cuh"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "step_kernel_traffic.json")
 
