@@ -48,7 +48,7 @@ typedef struct lbm3d_ctx lbm3d_ctx;
 /* Device bytes of the state of an nx x ny x nz domain at prec (LBM_FP64 or
  * LBM_FP32): two copies of f (19), g (7) and P, 15 per-node scalars (the
  * current state's rho, j, psi, T dp/dT/(rho c_v), stresses, T, u), plus two
- * layers in reserve.  0 for invalid arguments. */
+ * layers that are allocated and not used.  0 for invalid arguments. */
 size_t lbm3d_state_bytes(int nx, int ny, int nz, int prec);
 
 /* Creates a context; stream as in lbm_create (NULL: a library stream).

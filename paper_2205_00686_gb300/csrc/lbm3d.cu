@@ -208,7 +208,7 @@ template <class R>
 struct Lat3 {
     R s_e, s_eps, s_q, s_p;
     R sig_e3;            // (19/2) sigma / (1/s_e - 1/2), the sigma term of e
-    R vs0, vs1, vs3, vs4, w7_0, w7_1, cs2h, cv, inv_cv, gravity;
+    R vs3, vs4, w7_0, w7_1, cv, inv_cv, gravity;
     // unit rates: 1 - s_p, a quarter of it, 2 - s_p/2; the sigma term's factors of |12 s|^2 in the
     // axis and diagonal populations; (1 - vs1)/2; vs1 / cs2h
     R c_m, c_m4, c_w, h_ax, h_dg, h_m, vs1_cs2h;
@@ -239,9 +239,6 @@ Lat3<R> make_lat3(const lbm_params& p, const Dom3& D) {
     L.rho_ref = (R)D.rho_ref;
     L.T_ref = (R)D.T_ref;
     const double cs2h = p.w_dot / 3.0;
-    L.cs2h = (R)cs2h;
-    L.vs0 = (R)p.vs0;
-    L.vs1 = (R)(1.0 / (p.lambda / cs2h + 0.5));
     L.vs3 = (R)p.vs3;
     L.vs4 = (R)p.vs4;
     L.w7_0 = (R)(1.0 - p.w_dot);
@@ -527,15 +524,12 @@ __device__ __forceinline__ bool nbr_solid(const Nbr& d, int cz) {
 }
 
 // ---------------------------------------------------------------------------
-// psi of a node at most one layer beyond the domain: z wraps or, at walls,
-// comes from the ghost layer built from rho / T of layers 1 and 2
+// psi of a node beyond a wall: the ghost layer, from rho / T of layers 1 and 2
 template <class R>
-__device__ R psi_nb(const Dom3& D, const Phys<R>& P, int x, int y, int z, int* err) {
+__device__ R psi_ghost(const Dom3& D, const Phys<R>& P, int x, int y, int z, int* err) {
     const R* A = (const R*)D.aux;
     x = wrapn(x, D.nx);
     y = wrapn(y, D.ny);
-    if (z >= 0 && z < D.nz) return A[Q_PSI * D.plane + nid<R>(D, x, y, z)];
-    if (!D.walls) return A[Q_PSI * D.plane + nid<R>(D, x, y, wrapn(z, D.nz))];
     const int e = z < 0 ? 0 : 1;
     const int z1 = e == 0 ? 0 : D.nz - 1, z2 = e == 0 ? 1 : D.nz - 2;
     const R* rho = A + Q_RHO * D.plane;
@@ -560,7 +554,7 @@ __device__ __forceinline__ void force_at(const Dom3& D, const Phys<R>& P, const 
     R s[3];
     // beyond a wall the neighbour is the ghost layer (Section 3.3)
     stencil3<R>([&](int cx, int cy, int cz) {
-        return nbr_solid(nb, cz) ? psi_nb<R>(D, P, x + cx, y + cy, z + cz, err)
+        return nbr_solid(nb, cz) ? psi_ghost<R>(D, P, x + cx, y + cy, z + cz, err)
                                  : psi_p[(size_t)((long long)n + nbr_off(nb, cx, cy, cz))];
     }, s);
     const R gp = P.negG_12 * psi_p[n];
@@ -1253,7 +1247,8 @@ size_t pitch_for(int nx) { return ((size_t)nx + 31) / 32 * 32; }
 size_t bytes_for(int nx, int ny, int nz, int prec) {
     const size_t es = prec == LBM_FP64 ? 8 : 4;
     const size_t plane = pitch_for(nx) * ny * nz;
-    // f 2 x 19, g 2 x 7, P 2, the per-node planes 15, two layers in reserve
+    // f 2 x 19, g 2 x 7, P 2, the per-node planes 15, and two layers that no kernel
+    // uses but the published size counts
     return plane * es * (38 + 14 + 2 + Q_N) + 2 * pitch_for(nx) * ny * es;
 }
 

@@ -114,9 +114,9 @@ template <class R>
 struct Phys {
     // EOS: p = rho Rg T/(1 - b rho) - a h^2 rho^2/(1 + 2 b rho - b^2 rho^2),
     // h = 1 + kpr (1 - sqrt(T/Tc))
-    R a, b, Rg, kpr, inv_Tc;
+    R b, Rg, inv_Tc;
     R k_sa, k1_sa, m_third;          // k sqrt(a), (1 + k) sqrt(a), -1/3: see eos_node
-    R two_over_G, negG, negG_12;
+    R two_over_G, negG_12;
     // D2Q9 MRT rates and Li forcing
     R s_e, s_eps, s_q, s_p;
     R hs_e, hs_eps, hs_q, hs_p;      // 1 - s/2
@@ -146,10 +146,8 @@ inline Phys<R> make_phys(const PhysD& d) {
     Phys<R> p;
     double kpr = 0.37464 + 1.54226 * d.omega - 0.26992 * d.omega * d.omega;
     double Tc = 0.0778 * d.a / (0.45724 * d.b * d.Rg);
-    p.a = (R)d.a;
     p.b = (R)d.b;
     p.Rg = (R)(d.a < 0 ? -d.Rg : d.Rg);
-    p.kpr = (R)kpr;
     p.inv_Tc = (R)(1.0 / Tc);
     // eos_node works with |a| and p times the sign of a
     const double sgn = d.a < 0 ? -1.0 : 1.0, sa = std::sqrt(std::fabs(d.a));
@@ -157,7 +155,6 @@ inline Phys<R> make_phys(const PhysD& d) {
     p.k1_sa = (R)((1.0 + kpr) * sa);
     p.m_third = (R)(-sgn / 3.0);
     p.two_over_G = (R)(sgn * 2.0 / d.G);
-    p.negG = (R)(-d.G);
     p.negG_12 = (R)(-d.G / 12.0);
     p.s_e = (R)d.s_e;
     p.s_eps = (R)d.s_eps;
@@ -225,9 +222,9 @@ __device__ __forceinline__ double widen(float v) {
 }
 
 // ---- arithmetic helpers (precision-generic) -------------------------------
-// FP64 keeps IEEE division and square root (parity with the FP64 oracle to
-// ~1e-13); FP32 uses the hardware approximations (rcp.approx / sqrt.approx,
-// relative error ~2^-23), well inside the FP32 tolerance.
+// FP32 uses the hardware approximations (rcp.approx / sqrt.approx, relative error
+// ~2^-23), well inside the FP32 tolerance; FP64 two series terms from the hardware
+// seeds (below).  rsq, the wall's tangential difference, is IEEE in both.
 __device__ __forceinline__ float rsq(float x) { return sqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return sqrt(x); }
 __device__ __forceinline__ float rabs(float x) { return fabsf(x); }
@@ -242,13 +239,15 @@ __device__ __forceinline__ float f_rcp(float x) {
 // Both start from the hardware approximation of the seed, with e = 1 - x r
 // (or 1 - x y^2) of about 2^-20, and take the first two terms of the series
 // 1/(1-e) = 1 + e + e^2 + ... (or (1-e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ...): what
-// is left out is of order e^3 ~ 2^-60, below the FP64 rounding, so the result
-// is within about one ulp (not always the correctly rounded value).  Three
+// is left out is of order e^3 ~ 2^-60, below the FP64 rounding: the reciprocal
+// is within 0.51 ulp, the square root, whose correction takes half of the rounding
+// of x y for the seed's, within 0.76 (test_gpu_fp64_math.py).  Three
 // and five FP64 instructions, against four for two Newton-Raphson steps and
 // about ten for the IEEE square root.  With the node arithmetic of
-// lbm_node.cuh, which counts FP64 operations the same way (about 162 per node
-// instead of 220), the FP64 step on 1999 x 1501 went from 1.355 to 1.043 ms; in
-// FP32 the same forms took the 4096^2 step from 340.3 to 334.4 us.  (With the
+// lbm_node.cuh, which counts FP64 operations the same way (243 per node, halo
+// included, to 180), the FP64 step on 1999 x 1501 went from 1.355 to 1.043 ms; in
+// FP32 the same forms took the 4096^2 step from 340.3 to 334.4 us (337.9 with the
+// exact density sum).  (With the
 // IEEE operations instead the fields' distance from the FP64 oracle's is the
 // same, 2.3e-15 on 1999 x 1501.)  A zero, infinite or NaN reciprocal
 // operand gives a non-finite result, which the step reports; a square-root

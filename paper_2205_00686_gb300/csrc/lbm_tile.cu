@@ -5,11 +5,12 @@
 // The sweep of lbm_step.cu is made for bandwidth: a CTA walks a strip row by
 // row, so a step of a small domain is a chain of (rows + 6) iterations of two
 // barriers each on the few CTAs the domain fills (64 x 64 in FP64: 14
-// iterations on 8 of 152 SMs, 104 us).  Here the state stays in L2, a step is
-// one pass of three stages with two barriers, and the tile is small enough
-// that the domain reaches all SMs:
-//   A  moments, EOS and psi of the tile and two nodes around it (18 values
-//      loaded per thread before the first is used)
+// iterations on 8 of 152 SMs, 83 us).  Here the state stays in L2, a step of a
+// tile is one pass of three stages, each closed by a barrier of the CTA, and the
+// tile is small enough that the domain reaches all SMs:
+//   A  moments, EOS and psi of the tile and two nodes around it (a thread loads
+//      the 15 values of its node and the 14 of its node around the tile before
+//      the first is used)
 //   B  F_m, F, u on the tile and one node around it; on the tile the D2Q9
 //      collision, f*_i pushed to its destination in f(t+1) (wall: back to this
 //      node as the opposite direction; open edge: also to the edge nodes whose
