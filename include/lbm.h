@@ -357,7 +357,8 @@ void lbm_batch_destroy(lbm_batch* b);
  * device memory as the members, for the duration of the call).  The choice
  * is kept while members attach and detach (staging drops out while some
  * member cannot take it).  Without it a batch uses the lbm_create defaults
- * with a segment height chosen from the members' sizes.  lbm_batch_get_tile reports the tile in use. */
+ * with a segment height chosen from the members' sizes.  lbm_batch_get_tile
+ * reports the tile in use. */
 int lbm_batch_autotune(lbm_batch* b, int steps_per_trial);
 int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged);
 
@@ -369,11 +370,14 @@ int lbm_batch_get_tile(const lbm_batch* b, int* threads, int* rows, int* staged)
  * counts x heights (powers of two and the whole-wave heights) on a scratch
  * domain of the same size and precision, applies the fastest and caches the
  * choice per (precision, size).
- * Small domains (up to about 740 x 740 in FP32, 600 x 600 in FP64) take another
+ * Small domains (up to 736 x 736 in FP32, about 600 x 600 in FP64) take another
  * form of the same arithmetic unless a tile or load path is asked for: lbm_step
  * runs up to 1024 steps in one cooperative launch over tiles of nodes.  The
- * state is bit for bit the sweep's.  lbm_set_tile and lbm_set_staging select the sweep,
- * lbm_autotune times both forms; lbm_get_tile reports the sweep's tile.  Where
+ * state is bit for bit the sweep's.  lbm_set_tile and lbm_set_staging select the
+ * sweep, lbm_autotune times both forms; lbm_get_tile reports the sweep's tile.  A
+ * launch of that form takes the whole GPU for FP32 domains of some 256 x 256 nodes
+ * and more: several such contexts stepped at the same time are faster in a batch, or
+ * on the sweep (8 of 300 x 600: 66 us per step of all, 102 in this form).  Where
  * the cooperative launch is refused (a process or stream that may use only part
  * of the SMs), the context takes the sweep from that step on.
  * lbm_set_small_form: back from a sweep tile to that form, with the tile of its
@@ -421,7 +425,8 @@ int lbm_get_staging(const lbm_ctx* ctx);
  * give up at once at the grid barrier: they leave, the launches queued behind it
  * advance nothing, and the state is lost until lbm_init_fields, lbm_set_populations or
  * lbm_load.  on = 2: the cooperative launches of the small-domain form are
- * answered as if the device had refused them (nothing is launched).  Returns LBM_EINVAL for NULL, LBM_ESTATE in a batch. */
+ * answered as if the device had refused them (nothing is launched).  Returns
+ * LBM_EINVAL for NULL, LBM_ESTATE in a batch. */
 int lbm_set_wait_probe(lbm_ctx* ctx, int on);
 
 /* ---- diagnostics without any allocation -------------------------------- *

@@ -28,10 +28,11 @@
 // The arithmetic is that of lbm_node.cuh, so the state is bit for bit the one
 // the sweep would give.
 //
-// Measured per step (one GB300, lbm_step of 60-200 steps, sweep -> this): FP32
-// 64^2 18.8 -> 3.35 us, 256^2 19.2 -> 5.1, 300 x 600 pool 21.6 -> 15.3, 512^2
-// 23.5 -> 15.4; FP16-g 400 x 200 with a wall 21.8 -> 8.9; FP64 64^2 88 -> 8.7,
-// 200^2 92 -> 22.4, 384^2 154 -> 74.
+// Measured per step (one GB300, lbm_step of 60-300 steps, sweep -> this): FP32
+// 64^2 18.1 -> 3.45 us, 256^2 18.5 -> 5.0, 300 x 600 pool 20.5 -> 12.8, 512^2
+// 22.3 -> 14.9; FP16-g 400 x 200 with a wall 20.8 -> 7.7; FP64 64^2 82 -> 8.9,
+// 200^2 87 -> 21.4, 384^2 149 -> 71.  512^2 FP32: 837 thread instructions per node
+// (sweep 462), issue 40 % active, barriers the top stall.
 #include <algorithm>
 
 #include "lbm_node.cuh"
@@ -502,23 +503,28 @@ cudaError_t tile_run_any(const TileLaunch& L, const PhysD& phys, int grid, int t
 // barriers of the CTA per tile): about 1.6 us and, per round of resident tiles,
 // 3.45 us for 32 x 8 nodes (two CTAs per SM), 2.4 for 32 x 10 and 2.75 for 32 x
 // 12 (one).  Which one wastes least of its last round decides (us per step, 32
-// x 8 / 32 x 10 / 32 x 12): 256^2 5.1 / 6.8 / 7.2, 400 x 200 FP16-g 8.7 / 7.8 / 7.9,
-// 300 x 600 15.3 / 14.9 / 15.6, 512^2 15.2 / 16.0 / 15.1, 700^2 22.9 / 27.1 / 25.2.
+// x 8 / 32 x 10 / 32 x 12): 256^2 5.1 / 7.3 / 7.6, 400 x 200 FP16-g 8.8 / 7.7 / 7.9,
+// 300 x 600 pool 12.6 / 12.9 / 13.7, 512^2 15.2 / 16.8 / 15.0, 700^2 22.7 / 28.3 / 25.1.
+// Over 60 sizes from 64 to 768 (136 runs, open domains and pools) the choice is 2 %
+// off the best of the four on average, 16 % at most (358 x 713, open).
 // Full rows of 128 bytes beat 16 x 16, 16 x 8 and 8 x 8 everywhere except where 8
 // x 8 tiles with their surrounding nodes on threads of their own (one pass of
 // stage A instead of two) leave at most one per SM: 64^2 4.0 -> 3.35 us.  Against
 // the sweep with its best tile, 512^2 is 15.1 us against 23.5, 768^2 28.7 (8
 // rounds of 32 x 8) against 28.7 and 1024^2 48.5 against 40.6: up to 26 us here.
+// Walls, a heater and buoyancy add up to 2.5 us that this does not model, and cost
+// the sweep as much: pools at the limit, 700^2 24.6 against 27.5 us, 735^2 24.8
+// against 28.0, FP16-g 735^2 26.3 against 30.4, FP64 600^2 173 against 175.
 //
 // FP64: each of an SM's four partitions takes 64 cycles per FP64 warp
 // instruction, so the time is that of the busiest partition: about 170
 // instructions per warp of owned nodes, 65 per warp of surrounding nodes (90
 // in the first ring).  The candidates are compared by that count.  Measured /
-// modelled us per step: 64^2 8 x 4 with separate surrounding threads 8.7 / 8.7
-// (16 x 8 12.5 / 11.4), 200^2 20 x 14 22.4 / 23.3 (32 x 8 37.1 / 37.3), 384^2
-// 32 x 8 73.8 / 74.6; the sweep needs 92 at 200^2, 154 at 384^2, 156 at 512^2
-// (this form 124) and 198 at 640^2 (11 rounds of 32 x 8, 203 modelled), so
-// domains up to 190 modelled microseconds come here.
+// modelled us per step: 64^2 8 x 4 with separate surrounding threads 8.3 / 8.7
+// (16 x 8 12.1 / 11.4), 200^2 20 x 14 21.5 / 23.3 (32 x 8 35.7 / 37.3), 384^2
+// 32 x 8 71.1 / 74.6; the sweep needs 87 at 200^2, 149 at 384^2, 165 at 500^2
+// (this form 122) and 209 at 610^2, where 205 are modelled for 11 rounds of 32 x 8,
+// so domains up to 190 modelled microseconds come here.
 int tile_plan(int prec, const Inst& I, int sms, int want_tx, int want_ty, TilePlan* out) {
     out->tx = 0;
     const bool any = want_tx > 0;
